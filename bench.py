@@ -65,7 +65,7 @@ def kernel_peak(name, prec):
     # multiply-adds of 12 instructions, 48 per 8 flops; the pivoted QR's update, 102 per 16)
     df_per = {"k_zgemm_batched_df": 48.0 / 8.0, "k_pqr": 102.0 / 16.0, "k_cpqr": 102.0 / 16.0,
               "k_schur_solve": 48.0 / 8.0, "k_pgj": 48.0 / 8.0, "k_gj_inverse": 48.0 / 8.0,
-              "k_bgj_panel": 48.0 / 8.0}
+              "k_bgj_panel": 48.0 / 8.0, "k_gjx": 48.0 / 8.0}
     if name == "k_zgemm_batched_df" or (prec >= 1 and name in df_per):
         per = df_per[name]
         return ("alu", FP32_INSTR_PEAK / per / 1e12,
@@ -79,7 +79,7 @@ def kernel_peak(name, prec):
 FLOP_COUNT_NOTE = {
     "k_pqr": "8 m n k per m x n block of rank k (interpolative decomposition; Householder executes ~2x)",
     "k_cpqr": "8 m n k per m x n block of rank k (interpolative decomposition; Householder executes ~2x)",
-    "k_pgj": "8 n^3 per n x n block (Gauss-Jordan inverse)",
+    "k_gjx": "8 n^3 per n x n block (Gauss-Jordan inverse)",
     "k_zgemm_batched_df": "8 m n k per product",
     "k_zgemm_batched": "8 m n k per product",
     "k_oz_mma": "executed bf16 digit-plane flops on padded tiles",

@@ -316,12 +316,11 @@ hbs_status hbs_row_id(void* mt, int64_t m, int64_t n, double tol, int* rank, int
  * Batched in-place inverse of `count` complex128 blocks of size n x n (column-major,
  * back to back in device memory `a`), the per-node inversion step of Sec. 4 (D_tau^{-1}
  * in Eqs. def_muhD..def_muG): Gauss-Jordan elimination with partial pivoting, all
- * blocks in one launch (a persistent multi-CTA kernel for up to 128 blocks, one CTA per
- * block otherwise).  precision as for hbs_zgemm: _DOUBLE_FLOAT and _TENSOR run the
+ * blocks in the same launches (one launch per panel of columns, on clusters of CTAs, for up to
+ * 128 blocks; one CTA per block otherwise).  precision as for hbs_zgemm: _DOUBLE_FLOAT and _TENSOR run the
  * eliminations in double-float arithmetic.  1 <= n <= 4096, 1 <= count <= 2^20, else
  * HBS_ERR_INVALID_ARG.  Returns HBS_WARN_ILLCOND when a pivot is exactly zero (the
- * blocks' contents are then undefined) and HBS_ERR_TIMEOUT if a bounded barrier wait
- * of the persistent kernel gave up.  Synchronizes the stream.
+ * blocks' contents are then undefined).  Synchronizes the stream.
  */
 hbs_status hbs_batched_inverse(void* a, int64_t n, int64_t count, int precision, void* stream);
 
@@ -405,7 +404,7 @@ hbs_status hbs_row_id_static(void* mt, int64_t m, int64_t n, double tol, int* ra
  * Returns HBS_ERR_INVALID_ARG for an unknown kind or a negative value.
  *
  * hbs_barrier_selftest runs the library's bounded grid barrier (the one the
- * persistent QR, Gauss-Jordan and Schur kernels use) in a cooperative launch of
+ * persistent QR uses) in a cooperative launch of
  * `ctas` CTAs (1..64) passing three barriers; CTA `absent_cta` (if in [0, ctas))
  * leaves before the second, so the others give up after `limit_s` seconds (0 < limit_s
  * <= 10) and return.  *passed (host int) = CTAs that passed all three.  Returns

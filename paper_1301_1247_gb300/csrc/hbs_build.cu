@@ -28,10 +28,10 @@
 #include <numeric>
 
 #include "dense_kernels.cuh"
-#include "profile.hpp"
+#include "gjx.hpp"
 #include "handle.hpp"
+#include "profile.hpp"
 #include "qp_kernels.cuh"
-#include "tune.hpp"
 #include "zgemm.cuh"
 
 namespace hbs {
@@ -620,42 +620,10 @@ void batched_inverse(std::vector<InvJob>& jobs_in, cudaStream_t s, const char* w
   const bool all_big = jobs_in.size() <= 128;
   const bool use_big = all_big || (nbig > 0 && nbig <= 128);
   for (auto& j : jobs_in) {
-    if (use_big && (all_big || big_inverse(j.n))) big.push_back({j.a, j.n});
+    if (use_big && (all_big || big_inverse(j.n)) && gjx_fits(j.n)) big.push_back({j.a, j.n});
     else jobs.push_back(j);
   }
-  if (!big.empty()) {
-    // The multi-CTA inversion: the persistent Gauss-Jordan (pgj.cu, one grid barrier per
-    // column step; the default) or the blocked one (bgj.cu) on clusters of 1, 2, 4 or 8 CTAs
-    // per block; the autotuner measures them per shape class when it is on.
-    int nmax = 0;
-    for (const auto& m : big) nmax = std::max(nmax, m.second);
-    int n_pow = 1, c_pow = 1;
-    while (n_pow < nmax) n_pow *= 2;
-    while (c_pow < (int)big.size()) c_pow *= 2;
-    const std::string tkey = "inverse/n" + std::to_string(n_pow) + "/j" + std::to_string(c_pow) +
-                             (gemm_double_float() ? "/df" : "");
-    static const int kCs[5] = {0, 1, 2, 4, 8};
-    int var = tune::choose(tkey, 5, 0);
-    if (var > 0 && bgj_panel_width(nmax, kCs[var]) == 0) {  // does not fit: not a candidate
-      if (tune::exploring(tkey, 5)) tune::record(tkey, var, 5, 1e30f);
-      var = 0;
-    }
-    bool done = false;
-    if (var > 0) {
-      try {
-        tune::Timed timed(tkey, var, 5, s);
-        bgj_run(big, kCs[var], s, what);
-        done = true;
-      } catch (const Error& e) {
-        if (!bgj_unavailable(e)) throw;
-        tune::record(tkey, var, 5, 1e30f);  // this shape cannot run here: never choose it
-      }
-    }
-    if (!done) {
-      tune::Timed timed(tkey, 0, 5, s);
-      pgj_run(big, s, what);
-    }
-  }
+  if (!big.empty()) gjx_invert(big, s, what);
   if (jobs.empty()) return;
   for (size_t i = 0; i < jobs.size(); ++i) jobs[i].job = (int)i;
   int64_t piv = 0;

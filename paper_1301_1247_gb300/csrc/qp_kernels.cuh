@@ -55,21 +55,9 @@ void pqr_run(const std::vector<PqrSpec>& specs, double tol, cudaStream_t s, PqrO
 // W(:, c) <- R11^{-1} W(:, c) (first k rows) with R11 of matrix `job` of a pqr_run on A (m rows).
 void pqr_solve_r11(const cplx* A, int64_t m, const PqrOut& qr, int job, int k, cplx* W, int64_t ldw, int64_t ncols,
                    cudaStream_t s);
-// pgj.cu: in-place inverses of several large matrices (pointer, n) in one persistent
-// launch; throws HBS_WARN_ILLCOND on a singular block.
-void pgj_run(const std::vector<std::pair<cplx*, int>>& mats, cudaStream_t s, const char* what);
-// The same by blocked Gauss-Jordan (bgj.cu): panels of columns eliminated by a cluster of
-// cs CTAs per block (1, 2, 4 or 8), the rest of each block updated by the batched GEMM.
-void bgj_run(const std::vector<std::pair<cplx*, int>>& mats, int cs, cudaStream_t s, const char* what);
-// Panel width bgj_run uses for blocks up to nmax on clusters of cs CTAs (0: does not fit).
-int bgj_panel_width(int nmax, int cs);
-// True for bgj_run's error when the device cannot run the requested cluster shape; the
-// blocks are then untouched.
-struct Error;
-bool bgj_unavailable(const Error& e);
 struct InvJob;
-// In-place inverses of a batch of blocks (persistent Gauss-Jordan for few or large blocks,
-// one CTA per block otherwise); throws HBS_WARN_ILLCOND when a pivot is exactly zero.
+// In-place inverses of a batch of blocks (blocked Gauss-Jordan on clusters, gjx.cu, for few or
+// large blocks, one CTA per block otherwise); throws HBS_WARN_ILLCOND when a pivot is exactly zero.
 void batched_inverse(std::vector<InvJob>& jobs, cudaStream_t s, const char* what);
 // X(:, c) = R^{-1} B(:, c) for upper-triangular R (k x k, row-major); X may alias B.
 __global__ void k_tsolve_cols(const cplx* R, int k, const cplx* B, int64_t ldb, int64_t ncols, cplx* X, int64_t ldx);

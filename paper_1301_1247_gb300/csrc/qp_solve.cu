@@ -21,12 +21,11 @@
 #include <map>
 #include <mutex>
 #include <thread>
-#include <type_traits>
 
 #include "dense_kernels.cuh"
 #include "dfloat.cuh"
+#include "gjx.hpp"
 #include "profile.hpp"
-#include "gridsync.cuh"
 #include "qp_kernels.cuh"
 #include "tune.hpp"
 
@@ -1031,412 +1030,58 @@ __global__ void __launch_bounds__(NT) k_schur_solve(Dims D, const GroupJob* grou
   if (tid == 0) illcond[blockIdx.x] = (pmin <= 1e-28 * pmax) ? 1 : 0;
 }
 
-// The same blocked LU on CL CTAs per Bloch group (a cooperative launch over all groups):
-// CTA 0 of the group factors each panel while the others wait at a grid barrier, then all
-// CL CTAs share the U12 columns and the trailing-update tiles, and the back substitution's
-// right-hand sides.  Three bounded grid barriers per panel (all groups advance together;
-// `npan` is the largest panel count).  Used when the groups are fewer than the SMs, so
-// that every SM takes part.
-// Element arithmetic of the Schur LU for complex FP64 (cplx) and complex double-float (dfc).
-__device__ __forceinline__ long long lu_key(const cplx& v) { return nkey(cabs2(v)); }
-__device__ __forceinline__ long long lu_key(const dfc& v) {
-  return (long long)__float_as_uint(fmaf(v.rh, v.rh, v.ih * v.ih));  // |v|^2 to float precision
-}
-__device__ __forceinline__ bool lu_key_nonzero(long long k, const cplx*) { return __longlong_as_double(k) > 0.0; }
-__device__ __forceinline__ bool lu_key_nonzero(long long k, const dfc*) { return __uint_as_float((unsigned)k) > 0.f; }
-__device__ __forceinline__ double lu_key_value(long long k, const cplx*) { return __longlong_as_double(k); }
-__device__ __forceinline__ double lu_key_value(long long k, const dfc*) { return (double)__uint_as_float((unsigned)k); }
-__device__ __forceinline__ cplx lu_recip(const cplx& d) { return cabs2(d) > 0.0 ? cdiv(cmk(1, 0), d) : cmk(0, 0); }
-__device__ __forceinline__ dfc lu_recip(const dfc& d) { return dfc_recip(d); }
-__device__ __forceinline__ cplx lu_mul(const cplx& a, const cplx& b) { return cmul(a, b); }
-__device__ __forceinline__ dfc lu_mul(const dfc& a, const dfc& b) { return dfc_mul(a, b); }
-// c - a b
-__device__ __forceinline__ cplx lu_fms(const cplx& a, const cplx& b, const cplx& c) { return cfms(a, b, c); }
-__device__ __forceinline__ dfc lu_fms(const dfc& a, const dfc& b, const dfc& c) {
-  dfc r = c;
-  dfc_sub_mul(a, b, r);
-  return r;
-}
-// acc += a b (lazy for dfc; lu_norm finishes it)
-__device__ __forceinline__ void lu_acc(const cplx& a, const cplx& b, cplx& acc) { acc = cfma(a, b, acc); }
-__device__ __forceinline__ void lu_acc(const dfc& a, const dfc& b, dfc& acc) {
-  df_mac(a.rh, a.rl, b.rh, b.rl, acc.rh, acc.rl);
-  df_mac(-a.ih, -a.il, b.ih, b.il, acc.rh, acc.rl);
-  df_mac(a.rh, a.rl, b.ih, b.il, acc.ih, acc.il);
-  df_mac(a.ih, a.il, b.rh, b.rl, acc.ih, acc.il);
-}
-__device__ __forceinline__ void lu_norm(cplx&) {}
-__device__ __forceinline__ void lu_norm(dfc& a) { dfc_norm(a); }
-__device__ __forceinline__ cplx lu_sub(const cplx& c, const cplx& a) { return csub(c, a); }
-__device__ __forceinline__ dfc lu_sub(const dfc& c, const dfc& a) {
-  dfc r = c;
-  df_add_to(-a.rh, -a.rl, r.rh, r.rl);
-  df_add_to(-a.ih, -a.il, r.ih, r.il);
-  dfc_norm(r);
-  return r;
-}
-template <typename T> __device__ __forceinline__ T lu_zero();
-template <> __device__ __forceinline__ cplx lu_zero<cplx>() { return cmk(0, 0); }
-template <> __device__ __forceinline__ dfc lu_zero<dfc>() { return {0.f, 0.f, 0.f, 0.f}; }
-// warp sum (result in every lane)
-__device__ __forceinline__ cplx lu_warp_sum(cplx a) {
-  for (int o = 16; o > 0; o >>= 1) {
-    a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
-    a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
-  }
-  return a;
-}
-__device__ __forceinline__ dfc lu_warp_sum(dfc a) { return dfc_warp_sum(a); }
-
-// CL CTAs per Bloch group factor [S | R] with the panel-blocked LU of k_schur_solve: the
-// panel by CTA 0 of the group, U12 and the trailing update split over the group's CTAs,
-// three grid barriers per panel (every wait bounded).  The row interchanges are recorded
-// in pivpool (pstride per group) for a later refinement.  DF: the arithmetic is double-float on
-// the FP32 pipes, with [S | R] held in place as float pairs between a conversion pass at
-// the start and one at the end (pivots chosen on |a|^2 to float precision); the caller
-// then refines the solution once against the FP64 system.
-template <int NT, bool DF>
-__global__ void __launch_bounds__(NT) k_schur_coop(Dims D, const GroupJob* groups, int ng, int CL, int npan,
-                                                   cplx* Spool, cplx* Rpool, int* illcond, int* pivpool,
-                                                   int pstride, GridSync* gs) {
-  using T = typename std::conditional<DF, dfc, cplx>::type;
-  constexpr int NB = 16, TM = 64;
-  static_assert(NT == 256, "16 x 16 threads per trailing tile");
-  __shared__ long long redv[32];
-  __shared__ int redi[32];
-  __shared__ T sh_ip;
-  __shared__ T Ls[NB][TM + 1];
-  __shared__ T Us[NB][TM + 1];
-  __shared__ T L11[NB][NB + 1];
-  const int g = blockIdx.x / CL, rank = blockIdx.x % CL;
-  const bool act = g < ng;
-  int n = 0, q = 0;
-  cplx* A64 = nullptr;
-  cplx* B64 = nullptr;
-  int* piv = nullptr;
-  if (act) {
-    const GroupJob G = groups[g];
-    n = G.nsys;
-    q = G.q;
-    A64 = Spool + G.s_off;
-    B64 = Rpool + G.r_off;
-    piv = pivpool + (int64_t)g * pstride;
-  }
-  T* A = reinterpret_cast<T*>(A64);
-  T* B = reinterpret_cast<T*>(B64);
-  const int nc = n + q;
-  auto col = [&](int j) -> T* { return j < n ? A + (int64_t)j * n : B + (int64_t)(j - n) * n; };
-  auto col64 = [&](int j) -> cplx* { return j < n ? A64 + (int64_t)j * n : B64 + (int64_t)(j - n) * n; };
-  const int tid = threadIdx.x;
-  if constexpr (DF) {
-    if (act)
-      for (int j = rank; j < nc; j += CL) {
-        cplx* c64 = col64(j);
-        dfc* cd = reinterpret_cast<dfc*>(c64);
-        for (int i = tid; i < n; i += NT) cd[i] = to_dfc_bits(c64[i]);
-      }
-    if (grid_sync(gs) < 0) return;
-  }
-  double pmax = 0.0, pmin = 1e300;
-  for (int pn = 0; pn < npan; ++pn) {
-    const int k0 = pn * NB;
-    const bool live = act && k0 < n;
-    const int nb = live ? min(NB, n - k0) : 0;
-    if (live && rank == 0) {
-      for (int c = k0; c < k0 + nb; ++c) {
-        T* ac = A + (int64_t)c * n;
-        long long best = kNoKey;
-        int bi = 0x7fffffff;
-        for (int i = c + tid; i < n; i += NT) {
-          const long long v = lu_key(ac[i]);
-          if (better(v, i, best, bi)) { best = v; bi = i; }
-        }
-        long long kv;
-        int p;
-        block_argmax_key<NT>(best, bi, redv, redi, &kv, &p);
-        if (tid == 0) {  // pivot range for the conditioning flag (read by thread 0)
-          const double pv = lu_key_value(kv, A);
-          pmax = fmax(pmax, pv);
-          pmin = fmin(pmin, pv);
-          piv[c] = p;
-        }
-        if (p != c) {
-          for (int j = tid; j < nc; j += NT) {
-            T* cj = col(j);
-            const T t = cj[c];
-            cj[c] = cj[p];
-            cj[p] = t;
-          }
-        }
-        __syncthreads();
-        if (tid == 0) sh_ip = lu_recip(ac[c]);
-        __syncthreads();
-        const T ip = sh_ip;
-        for (int i = c + 1 + tid; i < n; i += NT) ac[i] = lu_mul(ac[i], ip);
-        __syncthreads();
-        for (int j = c + 1; j < k0 + nb; ++j) {
-          T* aj = A + (int64_t)j * n;
-          const T ucj = aj[c];
-          for (int i = c + 1 + tid; i < n; i += NT) aj[i] = lu_fms(ac[i], ucj, aj[i]);
-        }
-        __syncthreads();
-      }
-    }
-    if (grid_sync(gs) < 0) return;
-    const int j0 = k0 + nb;
-    const bool upd = live && j0 < nc;
-    if (upd) {
-      for (int e = tid; e < NB * NB; e += NT) {
-        const int r = e % NB, cc = e / NB;
-        L11[r][cc] = (r < nb && cc < nb) ? A[(int64_t)(k0 + cc) * n + k0 + r] : lu_zero<T>();
-      }
-      __syncthreads();
-      for (int j = j0 + rank * NT + tid; j < nc; j += CL * NT) {
-        T* aj = col(j) + k0;
-        T u[NB];
-#pragma unroll
-        for (int r = 0; r < NB; ++r) u[r] = r < nb ? aj[r] : lu_zero<T>();
-#pragma unroll
-        for (int cc = 0; cc < NB; ++cc)
-#pragma unroll
-          for (int r = cc + 1; r < NB; ++r) u[r] = lu_fms(L11[r][cc], u[cc], u[r]);
-#pragma unroll
-        for (int r = 0; r < NB; ++r)
-          if (r < nb) aj[r] = u[r];
-      }
-    }
-    if (grid_sync(gs) < 0) return;
-    if (upd) {
-      const int rows = n - j0, cols = nc - j0;
-      const int nrt = (rows + TM - 1) / TM, nct = (cols + TM - 1) / TM;
-      const int tr = tid & 15, tc = tid >> 4;
-      for (int tt = rank; tt < nrt * nct; tt += CL) {
-        const int rt = (tt % nrt) * TM, ct = (tt / nrt) * TM;
-        for (int e = tid; e < TM * NB; e += NT) {
-          const int r = e % TM, kk = e / TM;
-          const int i = j0 + rt + r;
-          Ls[kk][r] = (i < n && kk < nb) ? A[(int64_t)(k0 + kk) * n + i] : lu_zero<T>();
-        }
-        for (int e = tid; e < TM * NB; e += NT) {
-          const int kk = e % NB, c = e / NB;
-          const int j = j0 + ct + c;
-          Us[kk][c] = (j < nc && kk < nb) ? col(j)[k0 + kk] : lu_zero<T>();
-        }
-        __syncthreads();
-        T acc[4][4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) acc[a][b] = lu_zero<T>();
-        for (int kk = 0; kk < nb; ++kk) {
-          T la[4], ub[4];
-#pragma unroll
-          for (int a = 0; a < 4; ++a) la[a] = Ls[kk][tr + 16 * a];
-#pragma unroll
-          for (int b = 0; b < 4; ++b) ub[b] = Us[kk][tc + 16 * b];
-#pragma unroll
-          for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) lu_acc(la[a], ub[b], acc[a][b]);
-        }
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const int j = j0 + ct + tc + 16 * b;
-          if (j >= nc) continue;
-          T* cj = col(j);
-#pragma unroll
-          for (int a = 0; a < 4; ++a) {
-            const int i = j0 + rt + tr + 16 * a;
-            if (i < n) {
-              lu_norm(acc[a][b]);
-              cj[i] = lu_sub(cj[i], acc[a][b]);
-            }
-          }
-        }
-        __syncthreads();
-      }
-    }
-    if (grid_sync(gs) < 0) return;
-  }
-  if (act) {
-    // back substitution, one right-hand side per warp of the group's CTAs
-    const int lane = tid & 31, warp = tid >> 5;
-    for (int j = rank * (NT / 32) + warp; j < q; j += CL * (NT / 32)) {
-      T* b = B + (int64_t)j * n;
-      for (int i = n - 1; i >= 0; --i) {
-        T acc = lu_zero<T>();
-        for (int t = i + 1 + lane; t < n; t += 32) lu_acc(A[(int64_t)t * n + i], b[t], acc);
-        acc = lu_warp_sum(acc);
-        if (lane == 0) b[i] = lu_mul(lu_sub(b[i], acc), lu_recip(A[(int64_t)i * n + i]));
-        __syncwarp();
-      }
-    }
-    if (rank == 0 && tid == 0) illcond[g] = (pmin <= 1e-28 * pmax) ? 1 : 0;
-  }
-  if constexpr (DF) {
-    if (grid_sync(gs) < 0) return;  // every CTA of the group is done with [S | R]
-    if (act)
-      for (int j = rank; j < nc; j += CL) {
-        cplx* c64 = col64(j);
-        const dfc* cd = reinterpret_cast<const dfc*>(c64);
-        for (int i = tid; i < n; i += NT) c64[i] = from_dfc_bits(cd[i]);  // same 16-byte slot
-      }
-  }
-}
-
-// One step of iterative refinement per group against the FP64 system (after a factorization
-// in double-float): Rres holds R - S X (computed in FP64); solve (LU) d = P Rres with the
-// stored factors and pivots, and X += d.  One single-warp CTA per group and right-hand side
-// (CTA g qmax + j: right-hand side j of group g), in shared memory: the triangular solves are
-// sequential in the row index, so the parallelism is across the right-hand sides of all
-// groups.
-__global__ void __launch_bounds__(32) k_schur_refine(const GroupJob* groups, const cplx* Spool, cplx* Rpool,
-                                                     const cplx* Rres, const int* pivpool, int pstride, int qmax) {
-  extern __shared__ cplx sref[];  // n (1/U_ii) + n (the right-hand side)
-  const int g = (int)(blockIdx.x / (unsigned)qmax), j = (int)(blockIdx.x % (unsigned)qmax);
-  const GroupJob G = groups[g];
-  const int n = G.nsys;
-  if (j >= G.q) return;
-  const cplx* A = Spool + G.s_off;
-  const int* piv = pivpool + (int64_t)g * pstride;
-  const int lane = threadIdx.x;
-  cplx* inv = sref;
-  cplx* r = sref + n;
-  const cplx* rr = Rres + G.r_off + (int64_t)j * n;
-  for (int i = lane; i < n; i += 32) {
-    inv[i] = cdiv(cmk(1, 0), A[(int64_t)i * n + i]);
-    r[i] = rr[i];
-  }
-  __syncwarp();
-  if (lane == 0)
-    for (int c = 0; c < n; ++c) {
-      const int p = piv[c];
-      if (p != c) {
-        const cplx t = r[c];
-        r[c] = r[p];
-        r[p] = t;
-      }
-    }
-  __syncwarp();
-  for (int t = 0; t < n; ++t) {  // unit lower L
-    const cplx rt = r[t];
-    __syncwarp();
-    for (int i = t + 1 + lane; i < n; i += 32) r[i] = cfms(A[(int64_t)t * n + i], rt, r[i]);
-    __syncwarp();
-  }
-  for (int t = n - 1; t >= 0; --t) {  // upper U
-    if (lane == 0) r[t] = cmul(r[t], inv[t]);
-    __syncwarp();
-    const cplx rt = r[t];
-    for (int i = lane; i < t; i += 32) r[i] = cfms(A[(int64_t)t * n + i], rt, r[i]);
-    __syncwarp();
-  }
-  cplx* x = Rpool + G.r_off + (int64_t)j * n;
-  for (int i = lane; i < n; i += 32) x[i] = cadd(x[i], r[i]);
-}
-
-// Factor and solve every group's Schur system: CL CTAs per group in one cooperative launch
-// when the groups leave SMs idle, else one CTA per group.  In the thread's double-float
-// mode the cooperative factorization runs in double-float and the solution is refined once
-// against the FP64 system (residual by an FP64 product, correction with the same factors).
+// Factor and solve every group's Schur system by blocked Gauss-Jordan elimination (gjx.cu).  In
+// the thread's double-float mode it runs in double-float and the solution is refined once
+// against the FP64 system (residual by an FP64 product, correction with the same elimination).
+// Systems larger than the elimination's panels hold take the one-CTA LU above.
 static void schur_solve(const Dims& D, const std::vector<GroupJob>& gjobs, const GroupJob* dg, cplx* Sp, cplx* Rp,
                         int* ill, cudaStream_t s) {
   const int ng = (int)gjobs.size();
   const bool df = gemm_double_float();
-  // SM count and residency of the variant this call launches, per device (looked up once
-  // per device and variant under a lock: solves may run concurrently)
-  int sms = 0, per_sm = 0;
-  {
-    static std::mutex mu;
-    static std::map<std::pair<int, bool>, std::pair<int, int>> occ;
-    int dev = 0;
-    HBS_CUDA(cudaGetDevice(&dev));
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = occ.find({dev, df});
-    if (it == occ.end()) {
-      int sm = 0, per = 0;
-      HBS_CUDA(cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev));
-      if (df) HBS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_schur_coop<256, true>, 256, 0));
-      else HBS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_schur_coop<256, false>, 256, 0));
-      it = occ.emplace(std::make_pair(dev, df), std::make_pair(sm, per)).first;
-    }
-    sms = it->second.first;
-    per_sm = it->second.second;
+  int nmax = 0;
+  int64_t rend = 0;
+  for (const auto& G : gjobs) {
+    nmax = std::max(nmax, G.nsys);
+    rend = std::max<int64_t>(rend, G.r_off + (int64_t)G.nsys * G.q);
   }
-  // every CTA of the cooperative launch must be co-resident: ng * CL <= sms * per_sm
-  const int cl_max = std::min(4, (sms * std::min(per_sm, 2)) / std::max(ng, 1));
-  if (cl_max < 2) {
+  if (!gjx_fits(nmax)) {
     k_schur_solve<256><<<ng, 256, 0, s>>>(D, dg, Sp, Rp, ill);
     return;
   }
-  int nmax = 0;
-  int64_t send = 0, rend = 0;
-  for (const auto& G : gjobs) {
-    nmax = std::max(nmax, G.nsys);
-    send = std::max<int64_t>(send, G.s_off + (int64_t)G.nsys * G.nsys);
-    rend = std::max<int64_t>(rend, G.r_off + (int64_t)G.nsys * G.q);
-  }
-  // CTAs per group: 2, 3 or 4 (tuned per shape class when autotuning is on; the most that
-  // stay co-resident by default)
+  std::vector<GjxSys> sys;
+  for (const auto& G : gjobs) sys.push_back({Sp + G.s_off, Rp + G.r_off, G.nsys, G.q});
   int n_pow = 1, g_pow = 1;
   while (n_pow < nmax) n_pow *= 2;
   while (g_pow < ng) g_pow *= 2;
   const std::string tkey = "schur/n" + std::to_string(n_pow) + "/g" + std::to_string(g_pow) + (df ? "/df" : "");
-  int var = tune::choose(tkey, 3, cl_max - 2);
-  if (var + 2 > cl_max) {  // more CTAs than stay co-resident: not a candidate
-    if (tune::exploring(tkey, 3)) tune::record(tkey, var, 3, 1e30f);
-    var = cl_max - 2;
-  }
-  const int CL = var + 2;
-  tune::Timed timed(tkey, var, 3, s);
-  const int npan = (nmax + 15) / 16;
-  DevBuf<GridSync> gs(1);
-  DevBuf<int> piv((size_t)ng * std::max(nmax, 1));
-  DevBuf<cplx> S0, R0;
-  if (df) {  // the FP64 system, for the refinement
-    S0.alloc(std::max<int64_t>(send, 1));
-    R0.alloc(std::max<int64_t>(rend, 1));
-    HBS_CUDA(cudaMemcpyAsync(S0.get(), Sp, sizeof(cplx) * send, cudaMemcpyDeviceToDevice, s));
-    HBS_CUDA(cudaMemcpyAsync(R0.get(), Rp, sizeof(cplx) * rend, cudaMemcpyDeviceToDevice, s));
-  }
-  HBS_CUDA(cudaMemsetAsync(gs.get(), 0, sizeof(GridSync), s));
-  Dims a0 = D;
-  const GroupJob* a1 = dg;
-  int a2 = ng, a3 = CL, a4 = npan;
-  cplx* a5 = Sp;
-  cplx* a6 = Rp;
-  int* a7 = ill;
-  int* a8 = piv.get();
-  int a9 = nmax;
-  GridSync* a10 = gs.get();
-  void* args[] = {&a0, &a1, &a2, &a3, &a4, &a5, &a6, &a7, &a8, &a9, &a10};
+  const int cs = gjx_tuned_cluster(tkey, ng, nmax, df);
+  int var = 0;
+  while ((1 << var) < cs) ++var;
+  Gjx g;
   {
-    std::lock_guard<std::mutex> lock(coop_mutex());
-    const void* fn = df ? (const void*)k_schur_coop<256, true> : (const void*)k_schur_coop<256, false>;
-    HBS_CUDA(cudaLaunchCooperativeKernel(fn, dim3(ng * CL), dim3(256), args, 0, s));
-    GridSync hg{};
-    read_to_host(&hg, gs.get(), sizeof(GridSync), s);
-    if (hg.timed_out) throw Error(HBS_ERR_TIMEOUT, "Schur factorization: a grid barrier wait gave up");
+    tune::Timed timed(tkey, var, 4, s);
+    gjx_eliminate(g, sys, df, /*invert=*/false, cs, s);
   }
-  if (!df) return;
-  // R0 <- R0 - S0 X (FP64), then X += (LU)^{-1} P R0
-  {
+  DevBuf<cplx> X(std::max<int64_t>(rend, 1));
+  std::vector<cplx*> xp, rp;
+  for (const auto& G : gjobs) {
+    xp.push_back(X.get() + G.r_off);
+    rp.push_back(Rp + G.r_off);
+  }
+  DevBuf<cplx*> dx, dr;
+  dx.upload(xp, s);
+  dr.upload(rp, s);
+  gjx_solution(g, dx.get(), ill, s);
+  if (df) {  // R <- R - S X (FP64), then X += the elimination applied to it
     GemmModeScope fp64(HBS_PRECISION_FP64);
     std::vector<GemmJob> gj;
     for (const auto& G : gjobs)
-      gj.push_back({S0.get() + G.s_off, Rp + G.r_off, R0.get() + G.r_off, G.nsys, G.q, G.nsys, G.nsys, G.nsys,
-                    G.nsys, cmk(-1, 0), cmk(1, 0), 0, 0, 0});
+      gj.push_back({Sp + G.s_off, X.get() + G.r_off, Rp + G.r_off, G.nsys, G.q, G.nsys, G.nsys, G.nsys, G.nsys,
+                    cmk(-1, 0), cmk(1, 0), 0, 0, 0});
     run_gemms(gj, s);
+    gjx_apply(g, dr.get(), dx.get(), s);
   }
-  {
-    prof::KScope _ks("k_schur_refine", s);
-    const size_t shm = (size_t)2 * nmax * sizeof(cplx);
-    HBS_CUDA(raise_smem_limit((const void*)k_schur_refine, shm));
-    int qmax = 1;
-    for (const auto& G : gjobs) qmax = std::max(qmax, G.q);
-    k_schur_refine<<<(unsigned)(ng * qmax), 32, shm, s>>>(dg, Sp, Rp, R0.get(), piv.get(), nmax, qmax);
-  }
-  HBS_LAUNCH_CHECK("k_schur_refine");
+  HBS_CUDA(cudaMemcpyAsync(Rp, X.get(), sizeof(cplx) * rend, cudaMemcpyDeviceToDevice, s));
 }
 
 struct AngleJob {
