@@ -29,45 +29,24 @@ __device__ __forceinline__ void df_norm(float& ah, float& al) {
   ah = sum;
 }
 
-// Split of an FP64 value into a float pair (hi, lo) with integer operations only (the
-// FP64 conversion path shares the scarce FP64 pipe): hi carries the top 24 bits of the
-// significand, lo the remainder rounded to 24 bits, so hi + lo equals x to 2^-48
-// relative.  Values below the float range become 0.
+// Split of an FP64 value into a float pair (hi, lo) without the FP64 conversion path, which
+// shares the scarce FP64 pipe: hi carries the top 24 bits of the significand, lo the remainder (29
+// bits, an integer conversion) rounded to 24 bits, so hi + lo equals x to 2^-48 relative.
+// Values below the float range become 0, values above it infinite.  No branches and no bit
+// search: the operands of every double-float product pass through here (with both, the integer
+// pipe was 22 % busy beside the multiply-adds of the leaf products).
 __device__ __forceinline__ void df_split_bits(double x, float& hi, float& lo) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const unsigned int sgn = (unsigned int)(b >> 32) & 0x80000000u;
-  const int e = (int)((b >> 52) & 0x7ff);
-  const unsigned long long m = b & 0xFFFFFFFFFFFFFull;
-  const int fe = e - 1023 + 127;
-  if (e == 0 || fe < 1) {
-    hi = __uint_as_float(sgn);
-    lo = __uint_as_float(sgn);
-    return;
-  }
-  if (fe > 254) {
-    hi = __uint_as_float(sgn | 0x7f800000u);
-    lo = 0.0f;
-    return;
-  }
-  hi = __uint_as_float(sgn | ((unsigned int)fe << 23) | (unsigned int)(m >> 29));
-  const unsigned int r = (unsigned int)(m & 0x1FFFFFFFull);  // remainder, r 2^(e-1075)
-  if (r == 0u) {
-    lo = 0.0f;
-    return;
-  }
-  const int lz = __clz(r) - 3;  // leading zeros within the 29-bit field
-  int fel = fe - 24 - lz;
-  const unsigned int rn = r << lz;  // leading one at bit 28
-  unsigned int q = (rn + 16u) >> 5;  // 24-bit significand, rounded to nearest
-  if (q >> 24) {
-    q >>= 1;
-    ++fel;
-  }
-  if (fel < 1) {
-    lo = 0.0f;
-    return;
-  }
-  lo = __uint_as_float(sgn | ((unsigned int)fel << 23) | (q & 0x7FFFFFu));
+  const unsigned int h = (unsigned int)__double2hiint(x), l = (unsigned int)__double2loint(x);
+  const unsigned int sgn = h & 0x80000000u, a = h & 0x7FFFFFFFu;
+  const bool fits = a >= 0x38100000u && a < 0x47F00000u;  // 2^-126 <= |x| < 2^128
+  unsigned int f = __funnelshift_l(l, a - 0x38000000u, 3);  // exponent rebiased by 1023 - 127
+  f = fits ? f : (a < 0x38100000u ? 0u : 0x7F800000u);
+  // lo = r 2^(e - 1075), r < 2^29: r 2^-29 times 2^(fe - 150), fe the float's exponent field
+  const float r = __fmul_rn(__uint2float_rn(l & 0x1FFFFFFFu), 1.862645149230957e-09f);
+  const float scale = __uint_as_float((f & 0x7F800000u) - (23u << 23));
+  const float v = fits && f >= (24u << 23) ? __fmul_rn(r, scale) : 0.0f;
+  hi = __uint_as_float(sgn | f);
+  lo = __uint_as_float(sgn | __float_as_uint(v));
 }
 
 // float -> double with integer operations only (exact for normal floats; subnormal floats,

@@ -420,9 +420,9 @@ __global__ void k_splitk_reduce(const SplitRed* reds, int nred) {
   }
 }
 
-// Batched GEMMs.  Jobs with a long inner dimension and few output tiles (tall-skinny
-// products over all N boundary nodes) are split along K so that every SM gets work; the
-// partial products are summed in a fixed order by k_splitk_reduce.
+// Batched GEMMs.  Batches with few output tiles (small products, tall-skinny ones over all N
+// boundary nodes) are split along K so that every SM gets work; the partial products are summed
+// in a fixed order by k_splitk_reduce.
 static void launch_gemms(std::vector<GemmJob>& jobs_all, cudaStream_t s) {
   if (jobs_all.empty()) return;
   // large products on the tensor cores when the thread's mode asks for it
@@ -442,13 +442,17 @@ static void launch_gemms(std::vector<GemmJob>& jobs_all, cudaStream_t s) {
   std::vector<GemmJob> jobs;
   std::vector<SplitRed> reds;
   std::vector<size_t> red_ws_off;
-  int64_t ws = 0;
+  int64_t ws = 0, all_tiles = 0;
+  for (const auto& j : jobs_in) all_tiles += (int64_t)((j.m + GBM - 1) / GBM) * ((j.n + GBN - 1) / GBN);
+  // A batch with too few tiles for the SMs is split along k, into pieces of at least kmin: one
+  // SM's FP64 pipe runs a 32 x 32 tile at 8.3 GFLOP/s (8 us per slice of 8 k), so in FP64 even
+  // short pieces repay the second launch.  Four CTAs per SM are aimed at.
+  const int kmin = gemm_double_float() ? 64 : 24;
+  const int64_t want = all_tiles > 0 && all_tiles < 456 ? 608 / all_tiles : 1;
   for (const auto& j : jobs_in) {
     const int64_t tiles = (int64_t)((j.m + GBM - 1) / GBM) * ((j.n + GBN - 1) / GBN);
     int splits = 1;
-    if (j.k >= 8192 && tiles > 0 && tiles < 304) {
-      splits = (int)std::min<int64_t>((j.k + 4095) / 4096, std::max<int64_t>(1, 1216 / tiles));
-    }
+    if (tiles > 0 && want > 1) splits = (int)std::max<int64_t>(1, std::min<int64_t>(want, j.k / kmin));
     if (splits <= 1) {
       jobs.push_back(j);
       continue;
@@ -484,10 +488,10 @@ static void launch_gemms(std::vector<GemmJob>& jobs_all, cudaStream_t s) {
     HBS_CUDA(cudaMemcpyAsync(dj.get(), jobs.data(), jobs.size() * sizeof(GemmJob), cudaMemcpyHostToDevice, s));
     if (gemm_double_float()) {
       prof::KScope _ks("k_zgemm_batched_df", s, fl, by);
-      k_zgemm_batched_df<<<(unsigned)tiles, 256, 0, s>>>(dj.get(), (int)jobs.size());
+      k_zgemm_batched<dfc><<<(unsigned)tiles, 256, 0, s>>>(dj.get(), (int)jobs.size());
     } else {
       prof::KScope _ks("k_zgemm_batched", s, fl, by);
-      k_zgemm_batched<<<(unsigned)tiles, 256, 0, s>>>(dj.get(), (int)jobs.size());
+      k_zgemm_batched<cplx><<<(unsigned)tiles, 256, 0, s>>>(dj.get(), (int)jobs.size());
     }
   }
   HBS_LAUNCH_CHECK("k_zgemm_batched");
