@@ -3,30 +3,35 @@
 //
 // Each row r of op(A) is scaled by 2^-E_r (max |Re|, |Im| < 2^E_r) and each column c of B
 // by 2^-E_c, and every real part is written as a 49-bit integer M = sum_i q_i 2^{7(6-i)},
-// i = 0..6, with balanced digits: q_0 in [0, 128], q_1..q_6 in [-64, 64] (each one the
-// rounded quotient of the remainder left by the digits before it), small integers that
-// are exact in bf16.  A digit product (< 2^14) is exact in the tensor core, and
+// i = 0..6, with balanced digits: |q_0| <= 128, q_1..q_6 in [-64, 63], small integers that are exact
+// in bf16.  A digit product (at most 2^14) is exact in the tensor core, and
 //   C_rc = 2^{E_r + E_c - 14} sum_{l=0..6} 2^{-7 l} S_l,   S_l = sum_{i+j=l} sum_k q_i q_j
 // (the levels l >= 7 are dropped: together about 2^-48 of max|a| max|b| per product).  Over
-// 128 values of k every |S_l| stays below 2 x 128 x (2 x 2^13 + 5 x 2^12) < 2^24, so the FP32
-// accumulation in tensor memory is exact; every 128 k the seven level sums are combined in
-// double-float arithmetic (FP32 pipes) into a running double-float sum per output.
+// 224 values of k every |S_l| stays below 2 x 224 x (2 x 2^13 + 5 x 2^12) < 2^24, so the FP32
+// accumulation in tensor memory is exact; every 224 k the seven level sums are added, as
+// integers, to two 64-bit sums per real output (levels 0..3 and 4..6).  Nothing is rounded until the
+// sums become one FP64 value at the end.
 //
 // Per CTA: 128 x 32 outputs; tensor memory holds 7 levels x (re, im) x 32 columns of FP32
 // accumulators (level l in columns 32 l and 256 + 32 l).  Shared memory is a ring of three
 // stages of 16 k, each with 14 A sub-tiles (re/im x 7 digits, 128 x 16 bf16) and 14 B
-// sub-tiles (32 x 16) in the no-swizzle K-major core-matrix layout (8 rows x 16 bytes).  The
-// tensor memory accelerator fills a stage with four bulk tensor copies two stages ahead of
-// the MMAs: the digit planes are a 3-D tensor (k, row, plane), and a box of 8 k x all rows of
-// the tile x 14 planes lands as [plane][row][8 k], i.e. one k-group of every sub-tile, core
-// matrices of consecutive row groups 128 bytes apart; the two k-groups of a stage sit one
-// region apart (the descriptors' leading byte offset).  Since B's digit sub-tiles follow one
-// another, digit i of A meets digits 0..6-i of B in a single MMA of N = 32 (7 - i) columns
-// whose result falls into the levels i..6: one thread issues the copies and 28 MMAs per
-// stage (M = 128, K = 16) and commits them to the stage buffer's mbarrier; every wait is
-// bounded (one second) and a timeout is reported through a status word.
-#include <cuda.h>
-
+// sub-tiles (32 x 16) in the no-swizzle K-major core-matrix layout (8 rows x 16 bytes).  The digit
+// planes are stored in HBM in that layout, stage by stage ([tile][stage][k-group][plane][row][8
+// k]), so one bulk copy brings a stage's A and another its B, with no tensor map per product (a
+// tree level has thousands of products; encoding two maps for each took milliseconds of host
+// time).  Since B's digit sub-tiles follow one another, digit i of A meets digits 0..6-i of B in a
+// single MMA of N = 32 (7 - i) columns that adds to the levels i..6 at once.
+//
+// Roles: warp 8 issues the copies, warp 9 the MMAs, warps 0-7 read the accumulators (warp w the rows
+// 32 (w mod 4).. and columns 16 (w / 4)..) and write the outputs.  The copies and MMAs of the next
+// product run while the outputs of the last are written; only the read of the accumulators
+// itself, which fill 448 of tensor memory's 512 columns, stands between two periods.
+//
+// What bounds it: the MMAs (28 per 16 k, 3584 columns of N in all) and, within a factor of two, the
+// 70 KB that each stage brings from L2.  690 x 192 x 100 000: 2.36 ms, 1.40 PFLOP/s of executed
+// bf16 (0.73 of the measured 1.91), against 4.87 ms with a double-float combination of the levels
+// every 128 k (as long as the MMAs of the period, and alternating with them) and one thread for
+// copies and MMAs; the digit planes 0.84 ms against 3.35 (strided reads, two-byte stores).
 #include <algorithm>
 #include <cstdint>
 
@@ -44,105 +49,150 @@ constexpr int OZ_S = 7;        // digits per operand value
 constexpr int OZ_BM = 128;     // rows of C per CTA (tensor-memory lanes)
 constexpr int OZ_BN = 32;      // columns of C per CTA
 constexpr int OZ_BK = 16;      // k per shared-memory stage (one MMA)
-constexpr int OZ_FLUSH = 128;  // k per exact accumulation period
+constexpr int OZ_FLUSH = 224;  // k per exact accumulation period
 constexpr int OZ_RING = 3;     // stages in flight
 constexpr int OZ_NSUB = 2 * OZ_S;                         // sub-tiles per operand and stage
 constexpr int OZ_A_PL = OZ_BM * 16;                       // one plane's k-group of A: 128 rows x 16 B
 constexpr int OZ_B_PL = OZ_BN * 16;                       // one plane's k-group of B: 32 rows x 16 B
-constexpr int OZ_A_KG = OZ_NSUB * OZ_A_PL;                // a k-group of all 14 A planes (28 KB)
-constexpr int OZ_B_KG = OZ_NSUB * OZ_B_PL;                // a k-group of all 14 B planes (7 KB)
-constexpr int OZ_STAGE = 2 * (OZ_A_KG + OZ_B_KG);         // 70 KB: [A kg0 | A kg1 | B kg0 | B kg1]
-constexpr int OZ_SMEM = OZ_RING * OZ_STAGE;                // 210 KB
-
-// Exponent E with |x| < 2^E for the largest |x| given as IEEE bits (sign cleared); -2000
-// for zero rows (their digits are all zero).
-__device__ __forceinline__ int exp_above(unsigned long long absbits) {
-  const int e = (int)(absbits >> 52);
-  return e == 0 ? -2000 : e - 1022;
-}
+constexpr int OZ_A_ST = 2 * OZ_NSUB * OZ_A_PL;            // a stage of all 14 A planes (56 KB)
+constexpr int OZ_B_ST = 2 * OZ_NSUB * OZ_B_PL;            // a stage of all 14 B planes (14 KB)
+constexpr int OZ_STAGE = OZ_A_ST + OZ_B_ST;               // 70 KB
+constexpr int OZ_SMEM = OZ_RING * OZ_STAGE;               // 210 KB
+constexpr int OZ_EPI = 256;                               // threads that read accumulators
+constexpr int OZ_NT = OZ_EPI + 64;
+constexpr int kZeroRow = -2000;  // exponents up to this: a row of zeros (or of nothing yet)
 
 // One operand of one product: op(X) is rows x K with element (r, k) at X[r ld + k] (trans)
-// or X[k ld + r]; its exponents and digit planes (14 planes of rows_pad x Kpad bf16) go to
-// E and out.
+// or X[k ld + r]; its exponents and digit planes go to E and out, the planes stage by stage:
+// [row tile][stage of 16 k][k-group of 8][plane][row of the tile][8 k].
 struct OzOperand {
   const cplx* X;
   int ld, trans;
   int rows, K, rows_pad, Kpad;
+  int tile;     // rows per tile (128 for A, 32 for B)
+  int nplanes;  // leading digit planes kept (14; fewer when the rest are known to be zero)
   int* E;
   unsigned short* out;
-  int nplanes;  // leading digit planes written (14; fewer when the rest are known to be zero)
 };
 
-// max(|Re|, |Im|) over each row of operand blockIdx.y: one warp per row, integer compares on
-// the magnitude bits.  Rows past `rows` (padding) get the zero-row exponent.
-__global__ void k_oz_exponents(const OzOperand* ops) {
+// Exponent E with |x| < 2^E for the value whose FP64 high word is hi.
+__device__ __forceinline__ int exp_above(unsigned int hi) {
+  const int e = (int)((hi >> 20) & 0x7FFu);
+  return e == 0 ? kZeroRow : e - 1022;
+}
+__device__ __forceinline__ unsigned int abs_hi(const cplx& v) {
+  return max((unsigned int)__double2hiint(v.x) & 0x7FFFFFFFu, (unsigned int)__double2hiint(v.y) & 0x7FFFFFFFu);
+}
+
+// Row exponents of operand blockIdx.y (E preset to a large negative number): a block takes 32 rows x
+// 1024 k, reading along the operand's contiguous direction, and adds its maximum by atomics.
+__global__ void __launch_bounds__(256) k_oz_exponents(const OzOperand* ops) {
+  __shared__ unsigned int red[8][33];
   const OzOperand op = ops[blockIdx.y];
-  const int lane = threadIdx.x & 31;
-  for (int r = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5); r < op.rows_pad;
-       r += (int)((gridDim.x * (int64_t)blockDim.x) >> 5)) {
-    unsigned long long mx = 0;
-    if (r < op.rows) {
-      for (int k = lane; k < op.K; k += 32) {
-        const cplx v = op.trans ? op.X[(int64_t)r * op.ld + k] : op.X[(int64_t)k * op.ld + r];
-        const unsigned long long a = (unsigned long long)__double_as_longlong(v.x) & 0x7FFFFFFFFFFFFFFFull;
-        const unsigned long long b = (unsigned long long)__double_as_longlong(v.y) & 0x7FFFFFFFFFFFFFFFull;
-        mx = max(mx, max(a, b));
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int KC = 1024;
+  const int nrb = (op.rows + 31) / 32, nkc = (op.K + KC - 1) / KC;
+  for (int64_t u = blockIdx.x; u < (int64_t)nrb * nkc; u += gridDim.x) {
+    const int r0 = (int)(u % nrb) * 32, k0 = (int)(u / nrb) * KC, k1 = min(op.K, k0 + KC);
+    if (op.trans) {
+      for (int i = 0; i < 4; ++i) {
+        const int r = r0 + warp * 4 + i;
+        if (r >= op.rows) break;
+        const cplx* x = op.X + (int64_t)r * op.ld;
+        unsigned int mx = 0;
+        for (int k = k0 + lane; k < k1; k += 32) mx = max(mx, abs_hi(x[k]));
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (lane == 0) atomicMax(op.E + r, exp_above(mx));
+      }
+    } else {
+      unsigned int mx = 0;
+      const int r = r0 + lane;
+      if (r < op.rows) {
+        const cplx* x = op.X + r;
+#pragma unroll 4
+        for (int k = k0 + warp; k < k1; k += 8) mx = max(mx, abs_hi(x[(int64_t)k * op.ld]));
+      }
+      __syncthreads();  // red's last use
+      red[warp][lane] = mx;
+      __syncthreads();
+      if (warp == 0 && r < op.rows) {
+        for (int w = 1; w < 8; ++w) mx = max(mx, red[w][lane]);
+        atomicMax(op.E + r, exp_above(mx));
       }
     }
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, (unsigned long long)__shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) op.E[r] = exp_above(mx);
   }
 }
 
-// bf16 bits of the small integer (-1)^sign q (0 <= q <= 128), exact.
-__device__ __forceinline__ unsigned short bf16_of_digit(unsigned int q, unsigned int sign) {
-  if (q == 0u) return 0;
-  const int p = 31 - __clz(q);  // q in [2^p, 2^(p+1))
-  return (unsigned short)((sign << 15) | ((unsigned int)(127 + p) << 7) | ((q << (7 - p)) & 0x7Fu));
-}
-
-// The seven balanced digits of x (row exponent E) as bf16 bits, most significant first.
-__device__ __forceinline__ void digits_of(double x, int E, unsigned short* out) {
+// The seven balanced digits of x (row exponent E) as bf16 bits, most significant first, or'ed
+// into the 16-bit half `half` of w[0..6].  With 64 added at each of the six lower digit positions the
+// digits are the plain 7-bit fields less 64; a field is made a float by its place in the
+// significand of 2^23, and a small integer's bf16 is the upper half of its float.
+__device__ __forceinline__ void digits_of(double x, int E, int half, unsigned int* w) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const unsigned int sign = (unsigned int)(b >> 63);
   const int e = (int)((b >> 52) & 0x7FF);
   long long r = 0;
-  if (e != 0 && E > -2000) {
+  if (e != 0 && E > kZeroRow) {
     const unsigned long long mant = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
     const int sh = 1026 + E - e;  // |M| = round(mant 2^{e - 1075 + 49 - E}) = round(mant >> sh), sh >= 4
     if (sh < 64) r = (long long)((mant + (1ull << (sh - 1))) >> sh);
   }
+  if ((long long)b < 0) r = -r;
+  r += 0x20408102040ll;  // 64 (1 + 2^7 + ... + 2^35)
+  const unsigned int lo = (unsigned int)r, hi = (unsigned int)(r >> 28);  // digits 6..3 and 2..1 below 0
+  unsigned int f[OZ_S];
+  f[6] = lo & 127u;
+  f[5] = (lo >> 7) & 127u;
+  f[4] = (lo >> 14) & 127u;
+  f[3] = (lo >> 21) & 127u;
+  f[2] = hi & 127u;
+  f[1] = (hi >> 7) & 127u;
 #pragma unroll
-  for (int i = 0; i < OZ_S - 1; ++i) {
-    const int sh = 7 * (OZ_S - 1 - i);
-    const long long q = (r + (1ll << (sh - 1))) >> sh;  // rounded quotient (arithmetic shift)
-    r -= q * (1ll << sh);
-    out[i] = bf16_of_digit((unsigned int)(q < 0 ? -q : q), sign ^ (q < 0 ? 1u : 0u));
+  for (int i = 1; i < OZ_S; ++i) {
+    const float q = __fsub_rn(__uint_as_float(0x4B000000u | f[i]), 8388672.0f);  // 2^23 + 64
+    w[i] = half ? __byte_perm(w[i], __float_as_uint(q), 0x7610) : __float_as_uint(q) >> 16;
   }
-  out[OZ_S - 1] = bf16_of_digit((unsigned int)(r < 0 ? -r : r), sign ^ (r < 0 ? 1u : 0u));
+  const float q0 = (float)((int)hi >> 14);
+  w[0] = half ? __byte_perm(w[0], __float_as_uint(q0), 0x7610) : __float_as_uint(q0) >> 16;
 }
 
-// Digit planes of operand blockIdx.y: out[(part * 7 + d) * rows_pad * Kpad + r * Kpad + k]
-// (bf16; zero beyond rows and K).
-__global__ void k_oz_digits(const OzOperand* ops) {
+// Digit planes of operand blockIdx.y.  One thread per (row, k-group of 8): consecutive threads take
+// consecutive rows, so the 16-byte stores of a plane are contiguous, and the reads too unless
+// the operand is stored by rows (each thread then reads its own 128 bytes).
+__global__ void __launch_bounds__(256) k_oz_digits(const OzOperand* ops) {
   const OzOperand op = ops[blockIdx.y];
-  const int64_t plane = (int64_t)op.rows_pad * op.Kpad;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < plane; e += (int64_t)gridDim.x * blockDim.x) {
-    const int r = (int)(e / op.Kpad), k = (int)(e % op.Kpad);
-    unsigned short dre[OZ_S], dim[OZ_S];
-    if (r < op.rows && k < op.K) {
-      const cplx v = op.trans ? op.X[(int64_t)r * op.ld + k] : op.X[(int64_t)k * op.ld + r];
-      const int Er = op.E[r];
-      digits_of(v.x, Er, dre);
-      digits_of(v.y, Er, dim);
+  const int64_t tot = (int64_t)op.rows_pad * (op.Kpad / 8);
+  const int nkg = op.Kpad / 8;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
+    const int row = (int)(e % op.tile);
+    const int64_t t = e / op.tile;
+    const int kg = (int)(t % nkg), r = (int)(t / nkg) * op.tile + row, k = 8 * kg;
+    cplx v[8];
+    int E = kZeroRow;
+    if (r < op.rows) {
+      E = op.E[r];
+      const cplx* x = op.trans ? op.X + (int64_t)r * op.ld + k : op.X + (int64_t)k * op.ld + r;
+      const int64_t step = op.trans ? 1 : op.ld;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = k + i < op.K ? x[i * step] : cmk(0.0, 0.0);
     } else {
 #pragma unroll
-      for (int i = 0; i < OZ_S; ++i) dre[i] = dim[i] = 0;
+      for (int i = 0; i < 8; ++i) v[i] = cmk(0.0, 0.0);
     }
+    unsigned short* o = op.out + (t * op.nplanes * op.tile + row) * 8;
 #pragma unroll
-    for (int i = 0; i < OZ_S; ++i) {
-      if (i < op.nplanes) op.out[i * plane + e] = dre[i];
-      if (OZ_S + i < op.nplanes) op.out[(OZ_S + i) * plane + e] = dim[i];
+    for (int part = 0; part < 2; ++part) {
+      if (part * OZ_S >= op.nplanes) break;
+      unsigned int w[4][OZ_S];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        digits_of(part ? v[2 * i].y : v[2 * i].x, E, 0, w[i]);
+        digits_of(part ? v[2 * i + 1].y : v[2 * i + 1].x, E, 1, w[i]);
+      }
+#pragma unroll
+      for (int d = 0; d < OZ_S; ++d)
+        if (part * OZ_S + d < op.nplanes)
+          *reinterpret_cast<uint4*>(o + (int64_t)(part * OZ_S + d) * op.tile * 8) =
+              make_uint4(w[0][d], w[1][d], w[2][d], w[3][d]);
     }
   }
 }
@@ -171,8 +221,9 @@ __device__ __forceinline__ void oz_mma(uint32_t tmem, uint64_t da, uint64_t db, 
       "l"(da), "l"(db), "r"(idesc), "r"(acc));
 }
 
-// Waits for the mbarrier phase of the given parity; gives up after one second (globaltimer).
-__device__ __forceinline__ bool oz_wait(uint32_t bar, uint32_t parity) {
+// Waits for the mbarrier phase of the given parity; gives up after one second (globaltimer), or
+// once another wait of the CTA has given up (*gave_up, which this one then sets too).
+__device__ __forceinline__ bool oz_wait(uint32_t bar, uint32_t parity, volatile int* gave_up) {
   uint64_t t0;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
   for (;;) {
@@ -185,56 +236,72 @@ __device__ __forceinline__ bool oz_wait(uint32_t bar, uint32_t parity) {
     if (ok) return true;
     uint64_t t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    if (t - t0 > 1000000000ull) return false;
+    if (*gave_up || t - t0 > 1000000000ull) {
+      *gave_up = 1;
+      return false;
+    }
   }
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int c = 0; c < 16; ++c) v[c] = __uint_as_float(r[c]);
+__device__ __forceinline__ void oz_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// One bulk tensor copy of a box (8 k from x, rows from y, all 14 planes) of a digit-plane
-// tensor into shared memory at dst, completing on the mbarrier bar.  x is a multiple of 8
-// (16 bytes of bf16), as a tensor copy's innermost coordinate must be.
-__device__ __forceinline__ void oz_tma_load(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-      "[%5];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(0), "r"(bar)
-      : "memory");
+// Issues the read of 8 accumulator columns (32 lanes); the values are there after tmem_wait().
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+// The registers pass through the wait, so that no use of them can be moved before it.
+__device__ __forceinline__ void tmem_wait(uint32_t (&a)[8], uint32_t (&b)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
+                 "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7])
+               :
+               : "memory");
 }
 
-// One stage (16 k from kb) of the digit planes of A (rows row0..; the first planes_a of them,
-// as A's tensor map boxes hold) and of B (rows col0..) into the ring buffer at buf: announce
-// the stage's bytes on its full barrier, then four copies (two k-groups of each operand).
-__device__ __forceinline__ void oz_issue_stage(uint32_t buf, const CUtensorMap* tmA, const CUtensorMap* tmB, int row0,
-                                               int col0, int kb, uint32_t bar, int planes_a) {
-  const uint32_t bytes = 2u * (uint32_t)(planes_a * OZ_A_PL + OZ_B_KG);
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-  oz_tma_load(buf, tmA, kb, row0, bar);
-  oz_tma_load(buf + OZ_A_KG, tmA, kb + 8, row0, bar);
-  oz_tma_load(buf + 2 * OZ_A_KG, tmB, kb, col0, bar);
-  oz_tma_load(buf + 2 * OZ_A_KG + OZ_B_KG, tmB, kb + 8, col0, bar);
+// Bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) into shared memory,
+// completing on the mbarrier bar.
+__device__ __forceinline__ void oz_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
+// (hi 2^21 + lo) 2^e rounded to FP64, with integer operations (an FP64 instruction takes 64 cycles here
+// and an output needs several conversions).  |lo| < 2^58; the largest part beyond 64 bits is shifted out.
+__device__ __forceinline__ double oz_value(long long hi, long long lo, int e) {
+  const unsigned long long ah = (unsigned long long)(hi < 0 ? -hi : hi);
+  const int s = max(0, 64 - __clzll((long long)ah) - 41);  // bits of hi beyond 41
+  long long v;
+  if (s <= 21) v = (hi << (21 - s)) + (lo >> s);
+  else v = (hi >> (s - 21)) + (lo >> s);
+  if (v == 0) return 0.0;
+  const unsigned long long mag = (unsigned long long)(v < 0 ? -v : v);
+  const int lz = __clzll((long long)mag);
+  const unsigned long long norm = mag << lz;
+  unsigned long long m = norm >> 11;
+  const unsigned int rem = (unsigned int)norm & 0x7FFu;
+  m += (rem > 0x400u || (rem == 0x400u && (m & 1ull))) ? 1ull : 0ull;
+  const int be = 63 - lz + e + s + 1023;  // biased exponent before a carry out of the rounding
+  if (be < 1 || be > 2045) {
+    const double d = ldexp((double)m, 11 - lz + e + s);  // sub- or overnormal
+    return v < 0 ? -d : d;
+  }
+  const unsigned long long bits = ((unsigned long long)be << 52) + (m - (1ull << 52));
+  return __longlong_as_double((long long)(bits | (v < 0 ? 0x8000000000000000ull : 0ull)));
 }
 
 // One product of a batch on the tensor cores.  Work items are (tile_m, tile_n, split);
 // item_base is the prefix sum of tiles_m tiles_n splits over the earlier jobs.
 struct OzJob {
-  const unsigned short* Ad;  // digit planes of op(A): 14 x mpad x Kpad
-  const unsigned short* Bd;  // digit planes of B^T: 14 x npad x Kpad
-  const CUtensorMap* tmA;    // 3-D tensor maps of Ad and Bd (k, row, plane), boxes 8 x 128 x 14 and 8 x 32 x 14
-  const CUtensorMap* tmB;
+  const unsigned short* Ad;  // digit planes of op(A) and of B^T, stage by stage
+  const unsigned short* Bd;
   const int* Er;
   const int* Ec;
-  int m, n, mpad, npad, Kpad, klen, splits, tiles_m, tiles_n;
+  int m, n, nst, kst, splits, tiles_m, tiles_n;  // stages in all, stages per split
   int nre, nim;  // digit planes of op(A)'s real and imaginary parts that can be nonzero
   int64_t item_base;
   cplx alpha, beta;
@@ -244,216 +311,236 @@ struct OzJob {
   cplx* W;  // splits > 1: alpha (partial product) per split, splits x (m x n), reduced afterwards
 };
 
+struct OzItem {
+  int job, tm, tn, z, st0, nst;
+};
+
+__device__ __forceinline__ OzItem oz_item(const OzJob* jobs, int njobs, int64_t item) {
+  int lo = 0, hi = njobs - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (jobs[mid].item_base <= item) lo = mid; else hi = mid - 1;
+  }
+  const OzJob& jb = jobs[lo];
+  const int64_t local = item - jb.item_base;
+  const int per = jb.tiles_m * jb.tiles_n;
+  OzItem it;
+  it.job = lo;
+  it.z = (int)(local / per);
+  const int t2 = (int)(local % per);
+  it.tm = t2 % jb.tiles_m;
+  it.tn = t2 / jb.tiles_m;
+  it.st0 = it.z * jb.kst;
+  it.nst = min(jb.nst - it.st0, jb.kst);
+  return it;
+}
+
 // Persistent: CTA b takes items b, b + gridDim.x, ...; tensor memory, the mbarriers and the
-// shared-memory ring stay with the CTA across items (the stage counter G runs on, so every
-// buffer's barrier phases are known).  Thread 0 issues the copies and the MMAs of every stage
-// (warp 0 follows it stage by stage); at the end of each 128-k period all four warps meet it
-// at a barrier, wait for the period's MMAs and read the accumulators.  A wait that gives up clears the CTA-wide flag s_ok, which every thread
-// reads after the period's barrier, so all of them stop together.
-__global__ void __launch_bounds__(128, 1) k_oz_mma(const OzJob* jobs, int njobs, int64_t nitems, int* status) {
+// shared-memory ring stay with the CTA across items, and every role counts stages and periods on
+// through them, so each barrier's phases are known.  A wait that gives up sets s_gave_up, which
+// every other wait sees; all roles then leave their loops.
+__global__ void __launch_bounds__(OZ_NT, 1) k_oz_mma(const OzJob* jobs, int njobs, int64_t nitems, int* status) {
   extern __shared__ __align__(1024) unsigned char oz_smem[];
   __shared__ uint32_t s_tmem;
-  __shared__ __align__(8) uint64_t s_bar[OZ_RING];   // MMAs of the buffer's stage done
-  __shared__ __align__(8) uint64_t s_full[OZ_RING];  // the buffer's stage has landed
-  __shared__ int s_ok;
+  __shared__ __align__(8) uint64_t s_empty[OZ_RING];  // MMAs of the buffer's stage done
+  __shared__ __align__(8) uint64_t s_full[OZ_RING];   // the buffer's stage has landed
+  __shared__ __align__(8) uint64_t s_acc[2];          // period's MMAs done; accumulators read
+  __shared__ int s_gave_up;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&s_tmem)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
-  if (tid < OZ_RING) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_bar[tid])));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_full[tid])));
+  if (tid == 0) {
+    for (int b = 0; b < OZ_RING; ++b) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_empty[b])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_full[b])));
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_acc[0])));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;" ::"r"(smem_u32(&s_acc[1])));
+    s_gave_up = 0;
   }
-  if (tid == 0) s_ok = 1;
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s_tmem;
   const uint32_t ring = smem_u32(oz_smem);
-  const int per_flush = OZ_FLUSH / OZ_BK;
-  bool ok = true;  // CTA-uniform: refreshed from s_ok after every period's barrier
-  uint32_t G = 0;  // stages issued by this CTA so far
+  constexpr int per_flush = OZ_FLUSH / OZ_BK;
 
-  for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-    int lo = 0, hi = njobs - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (jobs[mid].item_base <= item) lo = mid; else hi = mid - 1;
+  if (warp == 8) {
+    // ---- copies
+    if (lane == 0) {
+      uint32_t G = 0;
+      bool ok = true;
+      for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+        const OzItem it = oz_item(jobs, njobs, item);
+        const OzJob& jb = jobs[it.job];
+        const int planes = jb.nim > 0 ? OZ_NSUB : jb.nre;
+        const uint32_t ab = 2u * (uint32_t)planes * OZ_A_PL;
+        const unsigned char* a = reinterpret_cast<const unsigned char*>(jb.Ad) + ((int64_t)it.tm * jb.nst + it.st0) * ab;
+        const unsigned char* b = reinterpret_cast<const unsigned char*>(jb.Bd) + ((int64_t)it.tn * jb.nst + it.st0) * OZ_B_ST;
+        for (int st = 0; st < it.nst; ++st, ++G) {
+          const int buf = (int)(G % OZ_RING);
+          if (G >= OZ_RING && !oz_wait(smem_u32(&s_empty[buf]), (G / OZ_RING - 1) & 1u, &s_gave_up)) {
+            ok = false;
+            break;
+          }
+          const uint32_t dst = ring + buf * OZ_STAGE, bar = smem_u32(&s_full[buf]);
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(ab + OZ_B_ST)
+                       : "memory");
+          oz_copy(dst, a + (int64_t)st * ab, ab, bar);
+          oz_copy(dst + OZ_A_ST, b + (int64_t)st * OZ_B_ST, OZ_B_ST, bar);
+        }
+      }
     }
-    const OzJob& jb = jobs[lo];
-    const int64_t local = item - jb.item_base;
-    const int per = jb.tiles_m * jb.tiles_n;
-    const int z = (int)(local / per), t2 = (int)(local % per);
-    const int row0 = (t2 % jb.tiles_m) * OZ_BM, col0 = (t2 / jb.tiles_m) * OZ_BN;
-    const int k0 = z * jb.klen, k1 = min(jb.Kpad, k0 + jb.klen);
-    const int nst = (k1 - k0) / OZ_BK;
-    const CUtensorMap* tmA = jb.tmA;
-    const CUtensorMap* tmB = jb.tmB;
-    const int planes_a = jb.nim > 0 ? OZ_NSUB : jb.nre;  // A's planes the copies bring
-
-    float Rh[2][OZ_BN], Rl[2][OZ_BN];  // running double-float sums (re, im) of this thread's row
+  } else if (warp == 9) {
+    // ---- MMAs
+    if (lane == 0) {
+      uint32_t G = 0, P = 0;
+      bool ok = true;
+      for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+        const OzItem it = oz_item(jobs, njobs, item);
+        const int nre = jobs[it.job].nre, nim = jobs[it.job].nim;
+        const uint32_t lbo_a = (uint32_t)(nim > 0 ? OZ_NSUB : nre) * OZ_A_PL;
+        for (int st = 0; st < it.nst; ++st, ++G) {
+          const bool fresh = st % per_flush == 0;
+          // the last period's accumulators have been read
+          if (fresh && P > 0 && !oz_wait(smem_u32(&s_acc[1]), (P - 1) & 1u, &s_gave_up)) {
+            ok = false;
+            break;
+          }
+          const int buf = (int)(G % OZ_RING);
+          if (!oz_wait(smem_u32(&s_full[buf]), (G / OZ_RING) & 1u, &s_gave_up)) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t sa = ring + buf * OZ_STAGE, sb = sa + OZ_A_ST;
+          const uint64_t dA = oz_desc(sa, lbo_a), dB = oz_desc(sb, OZ_NSUB * OZ_B_PL);
+          // digit i of A against digits 0..6-i of B in one MMA: B's digit planes lie one after
+          // another (32 rows each), and level l = i + j sits in columns 32 l (re) and
+          // 256 + 32 l (im), so the product lands in the levels i..6 at once.  Digits of A known to
+          // be zero (nre, nim) are skipped; digit 0 of the real part always runs, as it opens
+          // each period's accumulators.
 #pragma unroll
-    for (int p = 0; p < 2; ++p)
-#pragma unroll
-      for (int c = 0; c < OZ_BN; ++c) Rh[p][c] = Rl[p][c] = 0.f;
-
-    bool ok0 = true;  // thread 0's own waits in this item
-    if (tid == 0) {
-      // the tensor maps were written by the host before the launch; order their reads by the
-      // copy engine after that
-      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(tmA))
-                   : "memory");
-      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(tmB))
-                   : "memory");
-      // every earlier MMA has completed (the last period's wait covered it): all buffers are free
-      oz_issue_stage(ring + (G % OZ_RING) * OZ_STAGE, tmA, tmB, row0, col0, k0, smem_u32(&s_full[G % OZ_RING]),
-                     planes_a);
-      if (nst > 1)
-        oz_issue_stage(ring + ((G + 1) % OZ_RING) * OZ_STAGE, tmA, tmB, row0, col0, k0 + OZ_BK,
-                       smem_u32(&s_full[(G + 1) % OZ_RING]), planes_a);
-    }
-
-    for (int st = 0; st < nst; ++st) {
-      const uint32_t gs = G + (uint32_t)st;
-      const int buf = (int)(gs % OZ_RING);
-      if (warp == 0) {
-        if (lane == 0 && ok0) {
-          if (!oz_wait(smem_u32(&s_full[buf]), (gs / OZ_RING) & 1u)) {
-            ok0 = false;
-          } else {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t sa = ring + buf * OZ_STAGE, sb = sa + 2 * OZ_A_KG;
-            const uint64_t dA = oz_desc(sa, OZ_A_KG), dB = oz_desc(sb, OZ_B_KG);
-            const bool fresh = (st % per_flush) == 0;
-            // digit i of A against digits 0..6-i of B in one MMA: B's digit planes lie one after
-            // another (32 rows each), and level l = i + j sits in columns 32 l (re) and
-            // 256 + 32 l (im), so the product lands in the levels i..6 at once.
-#pragma unroll
-            // digits of A known to be zero (jb.nre, jb.nim) are skipped; digit 0 of the real
-            // part always runs, as it opens each period's accumulators
-            for (int i = 0; i < OZ_S; ++i) {
-              const int N = OZ_BN * (OZ_S - i);
-              const uint32_t ip = oz_idesc(false, N), in = oz_idesc(true, N);
-              const uint64_t ar = dA + (uint64_t)(i * (OZ_A_PL >> 4)), ai = dA + (uint64_t)((OZ_S + i) * (OZ_A_PL >> 4));
-              const uint64_t br = dB, bi = dB + (uint64_t)(OZ_S * (OZ_B_PL >> 4));
-              const uint32_t dre = tmem + OZ_BN * i, dim = tmem + 256 + OZ_BN * i;
-              const uint32_t first = (fresh && i == 0) ? 0u : 1u;
-              if (i < jb.nre) {
-                oz_mma(dre, ar, br, ip, first);  // re += Ar Br
-                oz_mma(dim, ar, bi, ip, first);  // im += Ar Bi
-              }
-              if (i < jb.nim) {
-                oz_mma(dre, ai, bi, in, 1u);  // re -= Ai Bi
-                oz_mma(dim, ai, br, ip, 1u);  // im += Ai Br
-              }
+          for (int i = 0; i < OZ_S; ++i) {
+            const int N = OZ_BN * (OZ_S - i);
+            const uint32_t ip = oz_idesc(false, N), in = oz_idesc(true, N);
+            const uint64_t ar = dA + (uint64_t)(i * (OZ_A_PL >> 4)), ai = dA + (uint64_t)((OZ_S + i) * (OZ_A_PL >> 4));
+            const uint64_t br = dB, bi = dB + (uint64_t)(OZ_S * (OZ_B_PL >> 4));
+            const uint32_t dre = tmem + OZ_BN * i, dim = tmem + 256 + OZ_BN * i;
+            const uint32_t first = (fresh && i == 0) ? 0u : 1u;
+            if (i < nre) {
+              oz_mma(dre, ar, br, ip, first);  // re += Ar Br
+              oz_mma(dim, ar, bi, ip, first);  // im += Ar Bi
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_u32(&s_bar[buf]))
-                         : "memory");
-            // refill the buffer of stage st - 1 with stage st + 2 once its MMAs are done
-            if (st + 2 < nst) {
-              const uint32_t pg = gs - 1;
-              if (st >= 1 && !oz_wait(smem_u32(&s_bar[pg % OZ_RING]), (pg / OZ_RING) & 1u)) {
-                ok0 = false;
-              } else {
-                const uint32_t nb = (gs + 2) % OZ_RING;
-                oz_issue_stage(ring + nb * OZ_STAGE, tmA, tmB, row0, col0, k0 + (st + 2) * OZ_BK,
-                               smem_u32(&s_full[nb]), planes_a);
-              }
+            if (i < nim) {
+              oz_mma(dre, ai, bi, in, 1u);  // re -= Ai Bi
+              oz_mma(dim, ai, br, ip, 1u);  // im += Ai Br
             }
           }
-          if (!ok0) atomicExch(&s_ok, 0);
+          oz_commit(smem_u32(&s_empty[buf]));
+          if (st % per_flush == per_flush - 1 || st == it.nst - 1) {
+            oz_commit(smem_u32(&s_acc[0]));
+            ++P;
+          }
         }
-        __syncwarp();
       }
-      if ((st % per_flush) == per_flush - 1 || st == nst - 1) {
-        // thread 0 arrives here only after committing this stage's MMAs, so the wait below
-        // is for the buffer's current phase (a parity wait tells only two phases apart: a
-        // warp running ahead of the issuing thread would see an older phase of the same
-        // parity complete)
-        __syncthreads();
-        const bool w = oz_wait(smem_u32(&s_bar[buf]), (gs / OZ_RING) & 1u);
-        if (!w) atomicExch(&s_ok, 0);
-        __syncwarp();
+    }
+  } else {
+    // ---- accumulators and outputs: row 32 (warp mod 4) + lane, columns 16 (warp / 4) ..
+    const int half = warp >> 2;
+    const uint32_t base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 16 * half;
+    uint32_t P = 0;
+    bool ok = true;
+    for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+      const OzItem it = oz_item(jobs, njobs, item);
+      const OzJob& jb = jobs[it.job];
+      long long Rh[2][16], Rl[2][16];  // sum of the levels 0..3 in units of level 3, and 4..6 of level 6
+#pragma unroll
+      for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int c = 0; c < 16; ++c) Rh[p][c] = Rl[p][c] = 0;
+      const int periods = (it.nst + per_flush - 1) / per_flush;
+      for (int q = 0; q < periods; ++q, ++P) {
+        if (!oz_wait(smem_u32(&s_acc[0]), P & 1u, &s_gave_up)) ok = false;
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (w) {
-          // T = sum_l 2^{-7 l} S_l (Horner from l = 6), R += T, in double-float
-          const uint32_t lanebase = tmem + ((uint32_t)(warp * 32) << 16);
 #pragma unroll
-          for (int p = 0; p < 2; ++p) {
+        for (int p = 0; p < 2; ++p) {
+          uint32_t a[8], b[8] = {};
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              float th[16], tl[16], sv[16];
+          for (int l = 0; l < OZ_S; l += 2) {
 #pragma unroll
-              for (int c = 0; c < 16; ++c) th[c] = tl[c] = 0.f;
-#pragma unroll 1
-              for (int l = OZ_S - 1; l >= 0; --l) {
-                tmem_ld16(lanebase + 256 * p + OZ_BN * l + 16 * h, sv);
+            for (int c0 = 0; c0 < 16; c0 += 8) {
+              tmem_ld8(base + 256 * p + OZ_BN * l + c0, a);
+              if (l + 1 < OZ_S) tmem_ld8(base + 256 * p + OZ_BN * (l + 1) + c0, b);
+              tmem_wait(a, b);
 #pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                  th[c] *= 0.0078125f;  // 2^-7, exact
-                  tl[c] *= 0.0078125f;
-                  df_add_to(sv[c], 0.f, th[c], tl[c]);
-                  df_norm(th[c], tl[c]);
+              for (int c = 0; c < 8; ++c) {
+                const long long x = __float2int_rn(__uint_as_float(a[c]));
+                if (l < 4) Rh[p][c0 + c] += x * (1 << (7 * (3 - l)));
+                else Rl[p][c0 + c] += x * (1 << (7 * (6 - l)));
+                if (l + 1 < OZ_S) {
+                  const long long y = __float2int_rn(__uint_as_float(b[c]));
+                  if (l + 1 < 4) Rh[p][c0 + c] += y * (1 << (7 * (2 - l)));
+                  else Rl[p][c0 + c] += y * (1 << (7 * (5 - l)));
                 }
-              }
-#pragma unroll
-              for (int c = 0; c < 16; ++c) {
-                df_add_to(th[c], tl[c], Rh[p][16 * h + c], Rl[p][16 * h + c]);
-                df_norm(Rh[p][16 * h + c], Rl[p][16 * h + c]);
               }
             }
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();  // tensor memory may be overwritten by the next period's MMAs
-        ok = s_ok != 0;
-        __syncthreads();  // every thread has read the flag before any can clear it again
-        if (!ok) break;
+        __syncwarp();
+        if (lane == 0)
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&s_acc[1])) : "memory");
       }
-    }
-    G += (uint32_t)nst;
-    // ---- epilogue: this item's 128 x 32 outputs (row of this thread)
-    const int row = row0 + warp * 32 + lane;
-    if (row < jb.m && ok) {
-      const int er = jb.Er[row];
+      if (!ok) break;
+      const int row = it.tm * OZ_BM + (warp & 3) * 32 + lane, c0 = it.tn * OZ_BN + 16 * half;
+      const int er = row < jb.m ? jb.Er[row] : 0;
       const cplx al = jb.alpha, be = jb.beta;
+      const bool unit = al.x == 1.0 && al.y == 0.0, minus = al.x == -1.0 && al.y == 0.0;
       const bool with_beta = jb.splits == 1 && (be.x != 0.0 || be.y != 0.0);
+      const bool unit_beta = be.x == 1.0 && be.y == 0.0;
 #pragma unroll
-      for (int c = 0; c < OZ_BN; ++c) {
-        const int col = col0 + c;
-        if (col >= jb.n) break;
-        const int sc = er + jb.Ec[col] - 14;
-        const double re = ldexp(f2d_bits(Rh[0][c]) + f2d_bits(Rl[0][c]), sc);
-        const double im = ldexp(f2d_bits(Rh[1][c]) + f2d_bits(Rl[1][c]), sc);
-        cplx v = cmk(al.x * re - al.y * im, al.x * im + al.y * re);
+      for (int c = 0; c < 16; ++c) {
+        const int col = c0 + c;
+        if (row >= jb.m || col >= jb.n) break;
+        const int sc = er + jb.Ec[col] - 56;  // 14 and the six digits below level 0
+        cplx v = cmk(oz_value(Rh[0][c], Rl[0][c], sc), oz_value(Rh[1][c], Rl[1][c], sc));
+        if (minus) v = cmk(-v.x, -v.y);
+        else if (!unit) v = cmk(al.x * v.x - al.y * v.y, al.x * v.y + al.y * v.x);
         if (jb.splits == 1) {
           cplx* cp = jb.transC ? jb.C + (int64_t)row * jb.ldc + col : jb.C + (int64_t)col * jb.ldc + row;
-          if (with_beta) v = cfma(be, *cp, v);
+          if (with_beta) v = unit_beta ? cadd(*cp, v) : cfma(be, *cp, v);
           *cp = v;
         } else {
-          jb.W[((int64_t)z * jb.n + col) * jb.m + row] = v;
+          jb.W[((int64_t)it.z * jb.n + col) * jb.m + row] = v;
         }
       }
+      __syncwarp();  // the accumulator reads are warp-wide
     }
   }
-  if (!ok && tid == 0) {
+  __syncwarp();
+  __syncthreads();
+  if (s_gave_up && tid == 0) {
     // a wait gave up: let the copies and MMAs in flight drain (bounded) before freeing
     // tensor memory and leaving the shared memory they write
-    for (int b = 0; b < OZ_RING; ++b) {
-      oz_wait(smem_u32(&s_full[b]), 0u);
-      oz_wait(smem_u32(&s_full[b]), 1u);
-      oz_wait(smem_u32(&s_bar[b]), 0u);
-      oz_wait(smem_u32(&s_bar[b]), 1u);
-    }
+    for (int b = 0; b < OZ_RING; ++b)
+      for (uint32_t par = 0; par < 2; ++par) {
+        int mine = 0;
+        oz_wait(smem_u32(&s_full[b]), par, &mine);
+        mine = 0;
+        oz_wait(smem_u32(&s_empty[b]), par, &mine);
+      }
+    atomicExch(status, 1);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
-  if (tid == 0 && !ok) atomicExch(status, 1);
 }
 
 // C = beta C + sum_s W_s (fixed order).
@@ -472,44 +559,11 @@ __global__ void k_oz_reduce(const cplx* W, int m, int n, int splits, cplx beta, 
 
 }  // namespace
 
-// cuTensorMapEncodeTiled from the driver (through the runtime's entry-point query, so the
-// library needs no link to the driver library).
-typedef CUresult (*TmapEncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-static TmapEncodeFn tmap_encoder() {
-  static TmapEncodeFn fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-    HBS_CUDA(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q));
-    if (q != cudaDriverEntryPointSuccess || p == nullptr)
-      throw Error(HBS_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
-    return reinterpret_cast<TmapEncodeFn>(p);
-  }();
-  return fn;
-}
-
-// Tensor map of one operand's digit planes (14 planes of rows_pad x Kpad bf16, k contiguous)
-// as a 3-D tensor (k, row, plane) with boxes of 8 k x box_rows x 14 planes.  The driver checks
-// the base (16-byte aligned), the strides (multiples of 16 bytes) and the box; a failure is an
-// error here, before any launch.
-static void encode_planes(CUtensorMap* m, const unsigned short* base, int Kpad, int rows_pad, int box_rows,
-                          int box_planes = OZ_NSUB) {
-  const cuuint64_t dims[3] = {(cuuint64_t)Kpad, (cuuint64_t)rows_pad, (cuuint64_t)OZ_NSUB};
-  const cuuint64_t strides[2] = {(cuuint64_t)Kpad * 2, (cuuint64_t)Kpad * 2 * (cuuint64_t)rows_pad};
-  const cuuint32_t box[3] = {8, (cuuint32_t)box_rows, (cuuint32_t)box_planes};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  const CUresult r = tmap_encoder()(m, CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, const_cast<unsigned short*>(base), dims,
-                                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                                    CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS)
-    throw Error(HBS_ERR_CUDA, "cuTensorMapEncodeTiled failed (CUresult " + std::to_string((int)r) + ")");
-}
-
 // Products worth the tensor cores: enough k for the digit planes to pay and enough rows for
 // the 128-row tiles.  (Routing the leaf products of the sweeps, k ~ 50, here as well was
 // measured slower: their digit planes cost as much as the double-float product.)
-bool ozaki_eligible(const GemmJob& j) { return j.k >= 96 && j.m >= 48 && j.n >= 8; }
+// (At most 2^26 values of k: the 64-bit sums hold 2^27.)
+bool ozaki_eligible(const GemmJob& j) { return j.k >= 96 && j.k <= (1 << 26) && j.m >= 48 && j.n >= 8; }
 
 // A batch of products on the tensor cores (see the head of this file): exponents and digit
 // planes of every operand (two launches), one persistent MMA launch over all tiles, and a
@@ -539,9 +593,7 @@ void ozaki_gemm_batched(const std::vector<GemmJob>& js, cudaStream_t s) {
     o.n = j.n;
     o.tiles_m = (j.m + OZ_BM - 1) / OZ_BM;
     o.tiles_n = (j.n + OZ_BN - 1) / OZ_BN;
-    o.mpad = o.tiles_m * OZ_BM;
-    o.npad = o.tiles_n * OZ_BN;
-    o.Kpad = (j.k + OZ_BK - 1) / OZ_BK * OZ_BK;  // stages of 16; the last period may be short
+    o.nst = (j.k + OZ_BK - 1) / OZ_BK;  // stages of 16; the last period may be short
     o.nre = j.a_real_digits > 0 ? std::min(j.a_real_digits, OZ_S) : OZ_S;
     o.nim = j.a_real_digits > 0 ? 0 : OZ_S;
     tiles_all += o.tiles_m * o.tiles_n;
@@ -549,12 +601,13 @@ void ozaki_gemm_batched(const std::vector<GemmJob>& js, cudaStream_t s) {
   for (int q = 0; q < nj; ++q) {
     const GemmJob& j = js[q];
     OzJob& o = oj[q];
-    // split along k only when the whole batch has too few tiles to fill the SMs
+    // split along k (in whole periods) only when the whole batch has too few tiles to fill the SMs
+    constexpr int kPer = OZ_FLUSH / OZ_BK;
+    const int periods = (o.nst + kPer - 1) / kPer;
     o.splits = 1;
-    if (tiles_all < sms && j.k >= 4096)
-      o.splits = std::max(1, std::min(o.Kpad / OZ_FLUSH, sms / std::max(1, tiles_all)));
-    o.klen = ((o.Kpad + OZ_FLUSH - 1) / OZ_FLUSH + o.splits - 1) / o.splits * OZ_FLUSH;
-    o.splits = (o.Kpad + o.klen - 1) / o.klen;
+    if (tiles_all < sms && j.k >= 4096) o.splits = std::max(1, std::min(periods, sms / std::max(1, tiles_all)));
+    o.kst = (periods + o.splits - 1) / o.splits * kPer;
+    o.splits = (o.nst + o.kst - 1) / o.kst;
     o.item_base = items;
     items += (int64_t)o.tiles_m * o.tiles_n * o.splits;
     o.alpha = j.alpha;
@@ -567,24 +620,24 @@ void ozaki_gemm_batched(const std::vector<GemmJob>& js, cudaStream_t s) {
     o.Er = reinterpret_cast<const int*>(eA);
     o.Ec = reinterpret_cast<const int*>(eB);
     o.W = reinterpret_cast<cplx*>(o.splits > 1 ? wtot : 0);
-    adig += (int64_t)OZ_NSUB * o.mpad * o.Kpad;
-    bdig += (int64_t)OZ_NSUB * o.npad * o.Kpad;
-    eA += o.mpad;
-    eB += o.npad;
+    const int64_t mpad = (int64_t)o.tiles_m * OZ_BM, npad = (int64_t)o.tiles_n * OZ_BN, Kpad = (int64_t)o.nst * OZ_BK;
+    adig += (o.nim > 0 ? OZ_NSUB : o.nre) * mpad * Kpad;
+    bdig += OZ_NSUB * npad * Kpad;
+    eA += j.m;
+    eB += j.n;
     if (o.splits > 1) wtot += (int64_t)o.splits * j.m * j.n;
     // executed: per digit i of A, 2 (7 - i) MMA units for its real part, 2 (7 - i) for its
     // imaginary part; 112 units in all for a general A (224 flops per m n k)
     double units = 0.0;
     for (int i = 0; i < OZ_S; ++i) units += 2.0 * (OZ_S - i) * ((i < o.nre) + (i < o.nim));
-    tflops += 2.0 * units * o.mpad * (double)o.npad * o.Kpad;
+    tflops += 2.0 * units * mpad * (double)npad * Kpad;
   }
   DevBuf<unsigned short> Ad(adig), Bd(bdig);
   DevBuf<int> E(eA + eB), st(1);
   DevBuf<cplx> W(std::max<int64_t>(wtot, 1));
   std::vector<OzOperand> ops;
   ops.reserve(2 * nj);
-  int maxrows = 0;
-  int64_t maxplane = 0;
+  int64_t maxexp = 1, maxdig = 1;
   for (int q = 0; q < nj; ++q) {
     const GemmJob& j = js[q];
     OzJob& o = oj[q];
@@ -593,23 +646,25 @@ void ozaki_gemm_batched(const std::vector<GemmJob>& js, cudaStream_t s) {
     int* er = E.get() + reinterpret_cast<int64_t>(o.Er);
     int* ec = E.get() + eA + reinterpret_cast<int64_t>(o.Ec);
     // op(A) row r, k: transA ? A[r lda + k] : A[k lda + r];  B^T row c, k: B[c ldb + k]
-    ops.push_back({j.A, j.lda, j.transA ? 1 : 0, j.m, j.k, o.mpad, o.Kpad, er, ad, o.nim > 0 ? OZ_NSUB : o.nre});
-    ops.push_back({j.B, j.ldb, 1, j.n, j.k, o.npad, o.Kpad, ec, bd, OZ_NSUB});
+    const int mpad = o.tiles_m * OZ_BM, npad = o.tiles_n * OZ_BN, Kpad = o.nst * OZ_BK;
+    ops.push_back({j.A, j.lda, j.transA ? 1 : 0, j.m, j.k, mpad, Kpad, OZ_BM, o.nim > 0 ? OZ_NSUB : o.nre, er, ad});
+    ops.push_back({j.B, j.ldb, 1, j.n, j.k, npad, Kpad, OZ_BN, OZ_NSUB, ec, bd});
     o.Ad = ad;
     o.Bd = bd;
     o.Er = er;
     o.Ec = ec;
     o.W = o.splits > 1 ? W.get() + reinterpret_cast<int64_t>(o.W) : nullptr;
-    maxrows = std::max(maxrows, std::max(o.mpad, o.npad));
-    maxplane = std::max(maxplane, (int64_t)std::max(o.mpad, o.npad) * o.Kpad);
+    maxexp = std::max(maxexp, (int64_t)((std::max(j.m, j.n) + 31) / 32) * ((j.k + 1023) / 1024));
+    maxdig = std::max(maxdig, (int64_t)std::max(mpad, npad) * (Kpad / 8));
   }
   HBS_CUDA(cudaMemsetAsync(st.get(), 0, sizeof(int), s));
+  HBS_CUDA(cudaMemsetAsync(E.get(), 0x80, sizeof(int) * (size_t)(eA + eB), s));  // below every exponent
   DevBuf<OzOperand> dops(ops.size());
   HBS_CUDA(cudaMemcpyAsync(dops.get(), ops.data(), ops.size() * sizeof(OzOperand), cudaMemcpyHostToDevice, s));
   {
     prof::KScope _ks("k_oz_digits", s);
-    const unsigned bx_e = (unsigned)std::min<int64_t>(1024, ((int64_t)maxrows * 32 + 255) / 256);
-    const unsigned bx_d = (unsigned)std::min<int64_t>(2048, (maxplane + 255) / 256);
+    const unsigned bx_e = (unsigned)std::min<int64_t>(4096, maxexp);
+    const unsigned bx_d = (unsigned)std::min<int64_t>(8192, (maxdig + 255) / 256);
     for (size_t o0 = 0; o0 < ops.size(); o0 += 65535) {
       const unsigned ny = (unsigned)std::min<size_t>(65535, ops.size() - o0);
       k_oz_exponents<<<dim3(bx_e, ny), 256, 0, s>>>(dops.get() + o0);
@@ -617,27 +672,13 @@ void ozaki_gemm_batched(const std::vector<GemmJob>& js, cudaStream_t s) {
     }
   }
   HBS_LAUNCH_CHECK("k_oz_digits");
-  // the digit planes' tensor maps, two per product, in device memory (128-byte aligned)
-  std::vector<CUtensorMap> maps(2 * (size_t)nj);
-  for (int q = 0; q < nj; ++q) {
-    const OzJob& o = oj[q];
-    encode_planes(&maps[2 * q], o.Ad, o.Kpad, o.mpad, OZ_BM, o.nim > 0 ? OZ_NSUB : o.nre);
-    encode_planes(&maps[2 * q + 1], o.Bd, o.Kpad, o.npad, OZ_BN);
-  }
-  DevBuf<CUtensorMap> dmaps;
-  dmaps.upload(maps, s);
-  if (reinterpret_cast<uintptr_t>(dmaps.get()) % 128 != 0) throw Error(HBS_ERR_INTERNAL, "tensor maps misaligned");
-  for (int q = 0; q < nj; ++q) {
-    oj[q].tmA = dmaps.get() + 2 * q;
-    oj[q].tmB = dmaps.get() + 2 * q + 1;
-  }
   DevBuf<OzJob> dj(nj);
   HBS_CUDA(cudaMemcpyAsync(dj.get(), oj.data(), nj * sizeof(OzJob), cudaMemcpyHostToDevice, s));
   {
     // executed tensor work: 28 digit pairs x 4 real products x 2 flops per (padded) m n k
     prof::KScope _ks("k_oz_mma", s, tflops, 0.0);
     const unsigned grid = (unsigned)std::min<int64_t>(sms, items);
-    k_oz_mma<<<grid, 128, OZ_SMEM, s>>>(dj.get(), nj, items, st.get());
+    k_oz_mma<<<grid, OZ_NT, OZ_SMEM, s>>>(dj.get(), nj, items, st.get());
   }
   HBS_LAUNCH_CHECK("k_oz_mma");
   for (int q = 0; q < nj; ++q) {
