@@ -22,10 +22,14 @@
 // time).  Since B's digit sub-tiles follow one another, digit i of A meets digits 0..6-i of B in a
 // single MMA of N = 32 (7 - i) columns that adds to the levels i..6 at once.
 //
-// Roles: warp 8 issues the copies, warp 9 the MMAs, warps 0-7 read the accumulators (warp w the rows
-// 32 (w mod 4).. and columns 16 (w / 4)..) and write the outputs.  The copies and MMAs of the next
+// Roles: warp 16 issues the copies, warp 17 the MMAs, warps 0-15 read the accumulators (warp w the rows
+// 32 (w mod 4).. and columns 8 (w / 4)..) and write the outputs.  The copies and MMAs of the next
 // product run while the outputs of the last are written; only the read of the accumulators
 // itself, which fill 448 of tensor memory's 512 columns, stands between two periods.
+//
+// Short products pay for their outputs: per 128 x 32 outputs 4 400 cycles to read the accumulators and 8
+// 200 of FP64 additions to round them, beside 7 200 of MMAs for k = 49 (with integer rounding the
+// outputs took 22 000).  690 x 8192 x 49: 0.124 ms, and 0.66 ms in double-float.
 //
 // What bounds it: the MMAs (28 per 16 k, 3584 columns of N in all) and, within a factor of two, the
 // 70 KB that each stage brings from L2.  690 x 192 x 100 000: 2.36 ms, 1.40 PFLOP/s of executed
@@ -58,7 +62,8 @@ constexpr int OZ_A_ST = 2 * OZ_NSUB * OZ_A_PL;            // a stage of all 14 A
 constexpr int OZ_B_ST = 2 * OZ_NSUB * OZ_B_PL;            // a stage of all 14 B planes (14 KB)
 constexpr int OZ_STAGE = OZ_A_ST + OZ_B_ST;               // 70 KB
 constexpr int OZ_SMEM = OZ_RING * OZ_STAGE;               // 210 KB
-constexpr int OZ_EPI = 256;                               // threads that read accumulators
+constexpr int OZ_EPI = 512;                               // threads that read accumulators
+constexpr int OZ_EC = 8;                                  // columns each of them holds
 constexpr int OZ_NT = OZ_EPI + 64;
 constexpr int kZeroRow = -2000;  // exponents up to this: a row of zeros (or of nothing yet)
 
@@ -224,8 +229,7 @@ __device__ __forceinline__ void oz_mma(uint32_t tmem, uint64_t da, uint64_t db, 
 // Waits for the mbarrier phase of the given parity; gives up after one second (globaltimer), or
 // once another wait of the CTA has given up (*gave_up, which this one then sets too).
 __device__ __forceinline__ bool oz_wait(uint32_t bar, uint32_t parity, volatile int* gave_up) {
-  uint64_t t0;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+  uint64_t t0 = 0;
   for (;;) {
     uint32_t ok;
     asm volatile(
@@ -236,6 +240,7 @@ __device__ __forceinline__ bool oz_wait(uint32_t bar, uint32_t parity, volatile 
     if (ok) return true;
     uint64_t t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    if (t0 == 0) t0 = t;
     if (*gave_up || t - t0 > 1000000000ull) {
       *gave_up = 1;
       return false;
@@ -270,28 +275,42 @@ __device__ __forceinline__ void oz_copy(uint32_t dst, const void* src, uint32_t 
                : "memory");
 }
 
-// (hi 2^21 + lo) 2^e rounded to FP64, with integer operations (an FP64 instruction takes 64 cycles here
-// and an output needs several conversions).  |lo| < 2^58; the largest part beyond 64 bits is shifted out.
-__device__ __forceinline__ double oz_value(long long hi, long long lo, int e) {
-  const unsigned long long ah = (unsigned long long)(hi < 0 ? -hi : hi);
-  const int s = max(0, 64 - __clzll((long long)ah) - 41);  // bits of hi beyond 41
-  long long v;
-  if (s <= 21) v = (hi << (21 - s)) + (lo >> s);
-  else v = (hi >> (s - 21)) + (lo >> s);
-  if (v == 0) return 0.0;
-  const unsigned long long mag = (unsigned long long)(v < 0 ? -v : v);
-  const int lz = __clzll((long long)mag);
-  const unsigned long long norm = mag << lz;
-  unsigned long long m = norm >> 11;
-  const unsigned int rem = (unsigned int)norm & 0x7FFu;
-  m += (rem > 0x400u || (rem == 0x400u && (m & 1ull))) ? 1ull : 0ull;
-  const int be = 63 - lz + e + s + 1023;  // biased exponent before a carry out of the rounding
-  if (be < 1 || be > 2045) {
-    const double d = ldexp((double)m, 11 - lz + e + s);  // sub- or overnormal
-    return v < 0 ? -d : d;
+// d 2^e: the exponent field moves, or two products (2^e might not be a number) where that leaves the
+// normal range.
+__device__ __forceinline__ double oz_scale(double d, int e) {
+  const int h = __double2hiint(d), x = (h >> 20) & 0x7FF;
+  if (x == 0) return d;  // a zero sum
+  if (x + e < 1 || x + e > 2046) {
+    const int e1 = max(-1000, min(1000, e)), e2 = max(-1000, min(1000, e - e1));
+    return d * __hiloint2double((1023 + e1) << 20, 0) * __hiloint2double((1023 + e2) << 20, 0);
   }
-  const unsigned long long bits = ((unsigned long long)be << 52) + (m - (1ull << 52));
-  return __longlong_as_double((long long)(bits | (v < 0 ? 0x8000000000000000ull : 0ull)));
+  return __hiloint2double(h + (e << 20), __double2loint(d));
+}
+
+// A 64-bit integer rounded to FP64, by its halves' places in the significands of 2^84 and 2^52: an FP64
+// instruction takes 64 cycles here and an output needs several, so the conversion instructions
+// (and the integer pipe: counting zeros and shifting took 22 000 cycles per 128 x 32 outputs) are
+// avoided; two additions.
+__device__ __forceinline__ double oz_narrow(long long v) {
+  const double a = __hiloint2double(0x45300000, (int)((unsigned int)(v >> 32) ^ 0x80000000u));
+  const double b = __hiloint2double(0x43300000, (int)(unsigned int)v);
+  return __dadd_rn(__dsub_rn(a, __longlong_as_double(0x4530000080100000ll)), b);  // 2^84 + 2^63 + 2^52
+}
+
+// hi 2^21 + lo rounded to FP64 once, times 2^e.  width 0: |hi| < 2^41, one 64-bit integer; 1: |hi| < 2^51, each
+// part by its place in the significand of 1.5 2^52, two exact subtractions and one multiply-add; 2: any
+// hi, the part beyond 64 bits shifted out (|lo| < 2^58).
+__device__ __forceinline__ double oz_value(long long hi, long long lo, int e, int width) {
+  if (width == 0) return oz_scale(oz_narrow((hi << 21) + lo), e);
+  if (width == 1) {
+    const double m = 6755399441055744.0;  // 1.5 2^52
+    const double a = __dsub_rn(__longlong_as_double(hi + 0x4338000000000000ll), m);
+    const double b = __dsub_rn(__longlong_as_double(lo + 0x4338000000000000ll), m);
+    return oz_scale(__fma_rn(a, 2097152.0, b), e);
+  }
+  const int s = max(0, 23 - __clzll(hi ^ (hi >> 63)));  // bits of |hi| beyond 41
+  const long long h = s <= 21 ? hi << (21 - s) : hi >> (s - 21);
+  return oz_scale(oz_narrow(h + (lo >> s)), e + s);
 }
 
 // One product of a batch on the tensor cores.  Work items are (tile_m, tile_n, split);
@@ -346,6 +365,7 @@ __global__ void __launch_bounds__(OZ_NT, 1) k_oz_mma(const OzJob* jobs, int njob
   __shared__ __align__(8) uint64_t s_full[OZ_RING];   // the buffer's stage has landed
   __shared__ __align__(8) uint64_t s_acc[2];          // period's MMAs done; accumulators read
   __shared__ int s_gave_up;
+  __shared__ OzItem s_next[OZ_EPI / 32];              // each output warp's next item
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (warp == 0) {
@@ -358,7 +378,7 @@ __global__ void __launch_bounds__(OZ_NT, 1) k_oz_mma(const OzJob* jobs, int njob
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_full[b])));
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_acc[0])));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;" ::"r"(smem_u32(&s_acc[1])));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 16;" ::"r"(smem_u32(&s_acc[1])));
     s_gave_up = 0;
   }
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -369,13 +389,15 @@ __global__ void __launch_bounds__(OZ_NT, 1) k_oz_mma(const OzJob* jobs, int njob
   const uint32_t ring = smem_u32(oz_smem);
   constexpr int per_flush = OZ_FLUSH / OZ_BK;
 
-  if (warp == 8) {
+  if (warp == OZ_EPI / 32) {
     // ---- copies
     if (lane == 0) {
       uint32_t G = 0;
       bool ok = true;
+      OzItem nx = oz_item(jobs, njobs, blockIdx.x);
       for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-        const OzItem it = oz_item(jobs, njobs, item);
+        const OzItem it = nx;
+        if (item + gridDim.x < nitems) nx = oz_item(jobs, njobs, item + gridDim.x);
         const OzJob& jb = jobs[it.job];
         const int planes = jb.nim > 0 ? OZ_NSUB : jb.nre;
         const uint32_t ab = 2u * (uint32_t)planes * OZ_A_PL;
@@ -395,13 +417,15 @@ __global__ void __launch_bounds__(OZ_NT, 1) k_oz_mma(const OzJob* jobs, int njob
         }
       }
     }
-  } else if (warp == 9) {
+  } else if (warp == OZ_EPI / 32 + 1) {
     // ---- MMAs
     if (lane == 0) {
       uint32_t G = 0, P = 0;
       bool ok = true;
+      OzItem nx = oz_item(jobs, njobs, blockIdx.x);
       for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-        const OzItem it = oz_item(jobs, njobs, item);
+        const OzItem it = nx;
+        if (item + gridDim.x < nitems) nx = oz_item(jobs, njobs, item + gridDim.x);
         const int nre = jobs[it.job].nre, nim = jobs[it.job].nim;
         const uint32_t lbo_a = (uint32_t)(nim > 0 ? OZ_NSUB : nre) * OZ_A_PL;
         for (int st = 0; st < it.nst; ++st, ++G) {
@@ -450,19 +474,32 @@ __global__ void __launch_bounds__(OZ_NT, 1) k_oz_mma(const OzJob* jobs, int njob
       }
     }
   } else {
-    // ---- accumulators and outputs: row 32 (warp mod 4) + lane, columns 16 (warp / 4) ..
-    const int half = warp >> 2;
-    const uint32_t base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 16 * half;
+    // ---- accumulators and outputs: row 32 (warp mod 4) + lane, columns 8 (warp / 4) ..
+    const uint32_t base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + OZ_EC * (warp >> 2);
     uint32_t P = 0;
     bool ok = true;
+    if (lane == 0) s_next[warp] = oz_item(jobs, njobs, blockIdx.x);
+    __syncwarp();
     for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-      const OzItem it = oz_item(jobs, njobs, item);
+      // what the outputs need is fetched before the wait for the accumulators, the next item too
+      const OzItem it = s_next[warp];
+      __syncwarp();
+      if (lane == 0 && item + gridDim.x < nitems) s_next[warp] = oz_item(jobs, njobs, item + gridDim.x);
       const OzJob& jb = jobs[it.job];
-      long long Rh[2][16], Rl[2][16];  // sum of the levels 0..3 in units of level 3, and 4..6 of level 6
+      const int row = it.tm * OZ_BM + (warp & 3) * 32 + lane, c0 = it.tn * OZ_BN + OZ_EC * (warp >> 2);
+      const int er = row < jb.m ? jb.Er[row] : 0;
+      const int ecl = c0 + (lane & 7) < jb.n ? jb.Ec[c0 + (lane & 7)] : 0;  // column c's in lane c
+      const bool with_beta = jb.splits == 1 && (jb.beta.x != 0.0 || jb.beta.y != 0.0);
+      const int64_t step = jb.splits > 1 ? jb.m : jb.transC ? 1 : jb.ldc;
+      cplx* out = jb.splits > 1 ? jb.W + ((int64_t)it.z * jb.n + c0) * jb.m + row
+                  : jb.transC   ? jb.C + (int64_t)row * jb.ldc + c0
+                                : jb.C + (int64_t)c0 * jb.ldc + row;
+      const int nc = row < jb.m ? min(OZ_EC, jb.n - c0) : 0;
+      long long Rh[2][OZ_EC], Rl[2][OZ_EC];  // sums of levels 0..3 in units of level 3, and 4..6 of level 6
 #pragma unroll
       for (int p = 0; p < 2; ++p)
 #pragma unroll
-        for (int c = 0; c < 16; ++c) Rh[p][c] = Rl[p][c] = 0;
+        for (int c = 0; c < OZ_EC; ++c) Rh[p][c] = Rl[p][c] = 0;
       const int periods = (it.nst + per_flush - 1) / per_flush;
       for (int q = 0; q < periods; ++q, ++P) {
         if (!oz_wait(smem_u32(&s_acc[0]), P & 1u, &s_gave_up)) ok = false;
@@ -471,24 +508,21 @@ __global__ void __launch_bounds__(OZ_NT, 1) k_oz_mma(const OzJob* jobs, int njob
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
-          uint32_t a[8], b[8] = {};
+          uint32_t a[OZ_EC], b[OZ_EC] = {};
 #pragma unroll
           for (int l = 0; l < OZ_S; l += 2) {
+            tmem_ld8(base + 256 * p + OZ_BN * l, a);
+            if (l + 1 < OZ_S) tmem_ld8(base + 256 * p + OZ_BN * (l + 1), b);
+            tmem_wait(a, b);
 #pragma unroll
-            for (int c0 = 0; c0 < 16; c0 += 8) {
-              tmem_ld8(base + 256 * p + OZ_BN * l + c0, a);
-              if (l + 1 < OZ_S) tmem_ld8(base + 256 * p + OZ_BN * (l + 1) + c0, b);
-              tmem_wait(a, b);
-#pragma unroll
-              for (int c = 0; c < 8; ++c) {
-                const long long x = __float2int_rn(__uint_as_float(a[c]));
-                if (l < 4) Rh[p][c0 + c] += x * (1 << (7 * (3 - l)));
-                else Rl[p][c0 + c] += x * (1 << (7 * (6 - l)));
-                if (l + 1 < OZ_S) {
-                  const long long y = __float2int_rn(__uint_as_float(b[c]));
-                  if (l + 1 < 4) Rh[p][c0 + c] += y * (1 << (7 * (2 - l)));
-                  else Rl[p][c0 + c] += y * (1 << (7 * (5 - l)));
-                }
+            for (int c = 0; c < OZ_EC; ++c) {
+              const long long x = __float2int_rn(__uint_as_float(a[c]));
+              if (l < 4) Rh[p][c] += x * (1 << (7 * (3 - l)));
+              else Rl[p][c] += x * (1 << (7 * (6 - l)));
+              if (l + 1 < OZ_S) {
+                const long long y = __float2int_rn(__uint_as_float(b[c]));
+                if (l + 1 < 4) Rh[p][c] += y * (1 << (7 * (2 - l)));
+                else Rl[p][c] += y * (1 << (7 * (5 - l)));
               }
             }
           }
@@ -499,26 +533,34 @@ __global__ void __launch_bounds__(OZ_NT, 1) k_oz_mma(const OzJob* jobs, int njob
           asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&s_acc[1])) : "memory");
       }
       if (!ok) break;
-      const int row = it.tm * OZ_BM + (warp & 3) * 32 + lane, c0 = it.tn * OZ_BN + 16 * half;
-      const int er = row < jb.m ? jb.Er[row] : 0;
       const cplx al = jb.alpha, be = jb.beta;
       const bool unit = al.x == 1.0 && al.y == 0.0, minus = al.x == -1.0 && al.y == 0.0;
-      const bool with_beta = jb.splits == 1 && (be.x != 0.0 || be.y != 0.0);
       const bool unit_beta = be.x == 1.0 && be.y == 0.0;
+      // how wide the sums are: |hi| < 2^41 for every value of the warp, or < 2^51, or more
+      long long ah = 0;
 #pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        const int col = c0 + c;
-        if (row >= jb.m || col >= jb.n) break;
-        const int sc = er + jb.Ec[col] - 56;  // 14 and the six digits below level 0
-        cplx v = cmk(oz_value(Rh[0][c], Rl[0][c], sc), oz_value(Rh[1][c], Rl[1][c], sc));
-        if (minus) v = cmk(-v.x, -v.y);
-        else if (!unit) v = cmk(al.x * v.x - al.y * v.y, al.x * v.y + al.y * v.x);
-        if (jb.splits == 1) {
-          cplx* cp = jb.transC ? jb.C + (int64_t)row * jb.ldc + col : jb.C + (int64_t)col * jb.ldc + row;
-          if (with_beta) v = unit_beta ? cadd(*cp, v) : cfma(be, *cp, v);
-          *cp = v;
-        } else {
-          jb.W[((int64_t)it.z * jb.n + col) * jb.m + row] = v;
+      for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int c = 0; c < OZ_EC; ++c) ah |= Rh[p][c] ^ (Rh[p][c] >> 63);
+      const int width = __all_sync(0xffffffffu, ah < (1ll << 41)) ? 0 : __all_sync(0xffffffffu, ah < (1ll << 51)) ? 1 : 2;
+#pragma unroll
+      for (int cb = 0; cb < OZ_EC; cb += 4) {
+        cplx old[4];  // four loads in flight: a store to C orders the loads after it
+        if (with_beta) {
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (cb + c < nc) old[c] = out[(cb + c) * step];
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int ec = __shfl_sync(0xffffffffu, ecl, cb + c);
+          if (cb + c >= nc) continue;
+          const int sc = er + ec - 56;  // 14 and the six digits below level 0
+          cplx v = cmk(oz_value(Rh[0][cb + c], Rl[0][cb + c], sc, width), oz_value(Rh[1][cb + c], Rl[1][cb + c], sc, width));
+          if (minus) v = cmk(-v.x, -v.y);
+          else if (!unit) v = cmk(al.x * v.x - al.y * v.y, al.x * v.y + al.y * v.x);
+          if (with_beta) v = unit_beta ? cadd(old[c], v) : cfma(be, old[c], v);
+          out[(cb + c) * step] = v;
         }
       }
       __syncwarp();  // the accumulator reads are warp-wide
@@ -559,11 +601,11 @@ __global__ void k_oz_reduce(const cplx* W, int m, int n, int splits, cplx beta, 
 
 }  // namespace
 
-// Products worth the tensor cores: enough k for the digit planes to pay and enough rows for
-// the 128-row tiles.  (Routing the leaf products of the sweeps, k ~ 50, here as well was
-// measured slower: their digit planes cost as much as the double-float product.)
-// (At most 2^26 values of k: the 64-bit sums hold 2^27.)
+// Products worth the tensor cores: k >= 96 and half a tile's rows; of those with 32 <= k < 96, which the
+// digit planes cost as much as the MMAs, the ones that nearly fill their 128-row tiles, and only when
+// the batch has enough of them (kOzakiShortWork): the path takes two more launches and a wait.  (At most 2^26 values of k: the 64-bit sums hold 2^27.)
 bool ozaki_eligible(const GemmJob& j) { return j.k >= 96 && j.k <= (1 << 26) && j.m >= 48 && j.n >= 8; }
+bool ozaki_eligible_short(const GemmJob& j) { return j.k >= 32 && j.k < 96 && j.m >= 96 && j.n >= 16; }
 
 // A batch of products on the tensor cores (see the head of this file): exponents and digit
 // planes of every operand (two launches), one persistent MMA launch over all tiles, and a
