@@ -541,7 +541,7 @@ DevGeom Handle_geom(const Handle& h) {
 
 // Work above which one matrix is decomposed by the multi-CTA kernels instead of one CTA.
 static bool big_cpqr(const CpqrJob& j) { return (double)j.m * j.n * std::min(j.m, j.n) > 4e6; }
-static bool big_inverse(int n) { return n > 128; }
+static bool big_inverse(int n) { return n > 72; }
 
 // Largest root (sum of the level-2 skeletons) for which level 1 is left uncompressed.  At the
 // top of the tree the level-1 ID and inversions are latency-bound work on two nodes; without
@@ -625,12 +625,19 @@ std::vector<int> batched_id(std::vector<CpqrJob>& jobs, double tol, cudaStream_t
 void batched_inverse(std::vector<InvJob>& jobs_in, cudaStream_t s, const char* what) {
   std::vector<InvJob> jobs;
   std::vector<std::pair<cplx*, int>> big;
-  // Same split as for the IDs: at most 128 blocks all go to one multi-CTA launch; with
-  // more, one CTA per block and the large ones (if at most 128) multi-CTA.
+  // The cluster elimination takes batches of at most 512 blocks, and blocks of more than 72 of larger
+  // ones; small blocks in large numbers stay with one CTA per block (49 x 2048: 1.25 ms there, 1.49 on
+  // clusters; 56 x 512: 0.58 and 0.46; 88 x 512: 1.93 and 1.37; 107 x 256: 2.8 and 1.0).  It works on a
+  // copy, which batches past 128 blocks may not always have the memory for: at most 4 GB there.
+  int64_t copy = 0;
   size_t nbig = 0;
-  for (const auto& j : jobs_in) nbig += big_inverse(j.n) ? 1 : 0;
-  const bool all_big = jobs_in.size() <= 128;
-  const bool use_big = all_big || (nbig > 0 && nbig <= 128);
+  for (const auto& j : jobs_in)
+    if (big_inverse(j.n) || jobs_in.size() <= 512) {
+      copy += 16 * (int64_t)j.n * j.n;
+      ++nbig;
+    }
+  const bool all_big = jobs_in.size() <= 512 && (jobs_in.size() <= 128 || copy <= (4ll << 30));
+  const bool use_big = all_big || (nbig <= 4096 && copy <= (4ll << 30));
   for (auto& j : jobs_in) {
     if (use_big && (all_big || big_inverse(j.n)) && gjx_fits(j.n)) big.push_back({j.a, j.n});
     else jobs.push_back(j);
