@@ -1,7 +1,6 @@
-// Batched small dense complex FP64 kernels used by the HBS build (Sec. 4):
-// column-pivoted QR for the interpolative decomposition (Def. 3.1) and
-// Gauss-Jordan inversion with partial pivoting for the per-node blocks.
-// One CTA works on one matrix; matrices live in global memory (L2-resident).
+// Batched small dense complex kernels used by the HBS build (Sec. 4): Gauss-Jordan inversion with
+// partial pivoting for the per-node blocks, one CTA per matrix, and helpers that the pivoted
+// factorizations share.
 #pragma once
 
 #include "common.cuh"
@@ -145,219 +144,6 @@ __device__ __forceinline__ void block_argmax(double v, int idx, double* redv, in
   *outv = redv[0];
   *outi = redi[0];
   __syncthreads();
-}
-
-// ---------------------------------------------------------------------------
-// Column-pivoted Householder QR of Mt (m x n) with rank revealed at
-// |R_ss| <= tol |R_00| (the interpolative decomposition of Def. 3.1 applied to
-// the rows of M = Mt^T).  Column norms are downdated after each reflection
-// and recomputed when cancellation has removed more than 7/8 of their digits
-// (relative to the norm at the last recomputation).
-// Dynamic shared memory: 2 n doubles + n ints.
-// ---------------------------------------------------------------------------
-// DF: the matrix is held in place as complex double-float (dfc) between the norm pass
-// and the triangular solve, and the rank-one updates run in double-float arithmetic on
-// the FP32 pipes; norms, pivots and the reflector scalars stay FP64.
-template <int NT, bool DF>
-__global__ void __launch_bounds__(NT) k_cpqr(const CpqrJob* jobs, int* rank_out, double tol, int kmax) {
-  extern __shared__ double smem[];
-  __shared__ long long redv[32];
-  __shared__ int redi[32];
-  __shared__ double redsig[NT];
-  __shared__ cplx sh_v0;
-  __shared__ double sh_tau;
-  __shared__ dfc sh_v0d;
-  __shared__ float sh_th, sh_tl;
-
-  const CpqrJob jb = jobs[blockIdx.x];
-  const int m = jb.m, n = jb.n;
-  cplx* A = jb.mt;
-  double* nrm = smem;          // current squared norms of the trailing parts
-  double* nrm_ref = smem + n;  // reference norms for the cancellation test
-  int* perm = reinterpret_cast<int*>(smem + 2 * n);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int NW = NT / 32;
-
-  dfc* D = reinterpret_cast<dfc*>(A);
-  // initial column norms (one warp per column)
-  for (int j = warp; j < n; j += NW) {
-    double s = 0.0;
-    cplx* col = A + (int64_t)j * m;
-    for (int i = lane; i < m; i += 32) {
-      const cplx x = col[i];
-      s += cabs2(x);
-      if constexpr (DF) reinterpret_cast<dfc*>(col)[i] = to_dfc_bits(x);
-    }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) { nrm[j] = s; nrm_ref[j] = s; }
-  }
-  for (int j = tid; j < n; j += NT) perm[j] = j;
-  __syncthreads();
-
-  const int kcap = min(min(m, n), kmax);
-  double r00 = 0.0, thr2 = 0.0;
-  int rank = 0;
-  for (int s = 0; s < kcap; ++s) {
-    long long best = kNoKey;
-    int bi = 0x7fffffff;
-    for (int j = s + tid; j < n; j += NT) {
-      const long long v = nkey(nrm[j]);
-      if (better(v, j, best, bi)) { best = v; bi = j; }
-    }
-    long long kv;
-    int p;
-    block_argmax_key<NT>(best, bi, redv, redi, &kv, &p);
-    const double pv = __longlong_as_double(kv);
-    if (s == 0) {
-      r00 = sqrt(pv);
-      thr2 = (tol * r00) * (tol * r00);
-    }
-    // |R_ss| <= tol |R_00|, compared squared
-    if (!(r00 > 0.0) || !(pv >= 0.0) || pv <= thr2) break;
-    // swap columns s and p
-    if (p != s) {
-      cplx* cs = A + (int64_t)s * m;
-      cplx* cp = A + (int64_t)p * m;
-      for (int i = tid; i < m; i += NT) { cplx t = cs[i]; cs[i] = cp[i]; cp[i] = t; }
-      if (tid == 0) {
-        double t = nrm[s]; nrm[s] = nrm[p]; nrm[p] = t;
-        t = nrm_ref[s]; nrm_ref[s] = nrm_ref[p]; nrm_ref[p] = t;
-        int ti = perm[s]; perm[s] = perm[p]; perm[p] = ti;
-      }
-    }
-    __syncthreads();
-    if constexpr (DF) {
-      // Householder reflector for x = A[s:m, s]
-      dfc* cs = D + (int64_t)s * m;
-      float qh = 0.f, ql = 0.f;
-      for (int i = s + 1 + tid; i < m; i += NT) df_abs2_acc(cs[i], qh, ql);
-      const double sig = block_sum_warp0<NT>(f2d_bits(qh) + f2d_bits(ql), redsig);
-      if (tid == 0) {
-        cplx v0, beta;
-        double tau;
-        householder_scalars(from_dfc_bits(cs[s]), sig, &v0, &beta, &tau);
-        sh_v0d = to_dfc_bits(v0);
-        float th, tl;
-        df_split_bits(tau, th, tl);
-        sh_th = th;
-        sh_tl = tl;
-        cs[s] = to_dfc_bits(beta);  // R_ss
-      }
-      __syncthreads();
-      const dfc v0 = sh_v0d;
-      const float th = sh_th, tl = sh_tl;
-      for (int j = s + 1 + warp; j < n; j += NW) {
-        dfc* cj = D + (int64_t)j * m;
-        dfc w = {0.f, 0.f, 0.f, 0.f};
-        for (int i = s + 1 + lane; i < m; i += 32) dfc_cdot_acc(cs[i], cj[i], w);
-        w = dfc_warp_sum(w);
-        const dfc ajs = cj[s];
-        dfc_cdot_acc(v0, ajs, w);
-        dfc_norm(w);
-        const dfc wv = dfc_scale(th, tl, w);
-        for (int i = s + 1 + lane; i < m; i += 32) {
-          dfc a = cj[i];
-          dfc_sub_mul(cs[i], wv, a);
-          cj[i] = a;
-        }
-        dfc top = ajs;
-        dfc_sub_mul(v0, wv, top);
-        __syncwarp();
-        // norm downdate, recomputation on cancellation (uniform over the warp)
-        float ph = 0.f, pl = 0.f;
-        df_abs2_acc(top, ph, pl);
-        double t = (nrm[j] - f2d_bits(ph)) - f2d_bits(pl);
-        if (t <= 0.0078125 * nrm_ref[j]) {
-          float rh = 0.f, rl = 0.f;
-          for (int i = s + 1 + lane; i < m; i += 32) df_abs2_acc(cj[i], rh, rl);
-          double q = f2d_bits(rh) + f2d_bits(rl);
-          for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-          t = q;
-          if (lane == 0) nrm_ref[j] = t;
-        }
-        __syncwarp();
-        if (lane == 0) {
-          cj[s] = top;
-          nrm[j] = t;
-        }
-      }
-      __syncthreads();
-      rank = s + 1;
-      continue;
-    }
-    // Householder reflector for x = A[s:m, s]
-    cplx* cs = A + (int64_t)s * m;
-    double sig = 0.0;
-    for (int i = s + 1 + tid; i < m; i += NT) sig += cabs2(cs[i]);
-    sig = block_sum_warp0<NT>(sig, redsig);
-    if (tid == 0) {
-      cplx v0, beta;
-      double tau;
-      householder_scalars(cs[s], sig, &v0, &beta, &tau);
-      sh_v0 = v0;
-      sh_tau = tau;
-      cs[s] = beta;  // R_ss
-    }
-    __syncthreads();
-    const cplx v0 = sh_v0;
-    const double tau = sh_tau;
-    // apply H = I - tau v v^H to columns s+1..n-1 (one warp per column)
-    for (int j = s + 1 + warp; j < n; j += NW) {
-      cplx* cj = A + (int64_t)j * m;
-      cplx w = cmk(0.0, 0.0);
-      for (int i = s + 1 + lane; i < m; i += 32) w = cfma(cconj(cs[i]), cj[i], w);
-      for (int o = 16; o > 0; o >>= 1) {
-        w.x += __shfl_xor_sync(0xffffffffu, w.x, o);
-        w.y += __shfl_xor_sync(0xffffffffu, w.y, o);
-      }
-      w = cfma(cconj(v0), cj[s], w);
-      w = cscale(w, tau);
-      if (lane == 0) cj[s] = cfms(v0, w, cj[s]);
-      for (int i = s + 1 + lane; i < m; i += 32) cj[i] = cfms(cs[i], w, cj[i]);
-      __syncwarp();
-      // norm downdate, recomputation on cancellation
-      if (lane == 0) {
-        double t = nrm[j] - cabs2(cj[s]);
-        nrm[j] = t;
-      }
-      __syncwarp();
-      if (nrm[j] <= 0.0078125 * nrm_ref[j]) {
-        double t = 0.0;
-        for (int i = s + 1 + lane; i < m; i += 32) t += cabs2(cj[i]);
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane == 0) { nrm[j] = t; nrm_ref[j] = t; }
-      }
-    }
-    __syncthreads();
-    rank = s + 1;
-  }
-  // T = R11^{-1} R12, one warp per column of R12
-  const int k = rank;
-  if constexpr (DF) {
-    // back to FP64: rows < k of every column (R11, R12; the rest is scratch)
-    __syncthreads();
-    for (int j = warp; j < n; j += NW)
-      for (int i = lane; i < min(k, m); i += 32) A[(int64_t)j * m + i] = from_dfc_bits(D[(int64_t)j * m + i]);
-    __syncthreads();
-  }
-  cplx* T = jb.t;
-  for (int c = warp; c < n - k; c += NW) {
-    const cplx* r12 = A + (int64_t)(k + c) * m;
-    cplx* tc = T + (int64_t)c * k;
-    for (int i = k - 1; i >= 0; --i) {
-      cplx acc = cmk(0.0, 0.0);
-      for (int l = i + 1 + lane; l < k; l += 32) acc = cfma(A[(int64_t)l * m + i], tc[l], acc);
-      for (int o = 16; o > 0; o >>= 1) {
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-      }
-      if (lane == 0) tc[i] = cdiv(csub(r12[i], acc), A[(int64_t)i * m + i]);
-      __syncwarp();
-    }
-  }
-  int* po = jb.perm;
-  for (int j = tid; j < n; j += NT) po[j] = perm[j];
-  if (tid == 0) rank_out[jb.job] = k;
 }
 
 // ---------------------------------------------------------------------------

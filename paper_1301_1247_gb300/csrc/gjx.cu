@@ -36,7 +36,7 @@
 #include <type_traits>
 
 #include "dense_kernels.cuh"
-#include "dfloat.cuh"
+#include "elem.cuh"
 #include "gjx.hpp"
 #include "profile.hpp"
 #include "qp_kernels.cuh"
@@ -53,10 +53,6 @@ constexpr int kW = kT / 32;
 constexpr int kTile = 64;  // rows of a strip's tile
 constexpr int kS = 16;     // columns of a strip
 
-// ---- element arithmetic: complex FP64 (cplx) and complex double-float (dfc) ----
-template <typename T> __device__ __forceinline__ T x_zero();
-template <> __device__ __forceinline__ cplx x_zero<cplx>() { return cmk(0.0, 0.0); }
-template <> __device__ __forceinline__ dfc x_zero<dfc>() { return {0.f, 0.f, 0.f, 0.f}; }
 // Pivot keys: |v|^2 to float precision (double-float), or the sign, exponent and upper
 // significand bits of |v|^2 (FP64), as unsigned integers that order alike; 1 is an exact zero and 0
 // no candidate.
@@ -64,41 +60,6 @@ __device__ __forceinline__ unsigned x_key(const cplx& v) { return (unsigned)__do
 __device__ __forceinline__ unsigned x_key(const dfc& v) { return __float_as_uint(fmaf(v.rh, v.rh, v.ih * v.ih)) + 1u; }
 __device__ __forceinline__ double x_key_value(unsigned k, const cplx*) { return __hiloint2double((int)(k - 1u), 0); }
 __device__ __forceinline__ double x_key_value(unsigned k, const dfc*) { return (double)__uint_as_float(k - 1u); }
-// 1 / d = conj(d) / |d|^2.  FP64: d is scaled by a power of two to a modulus near 1 and 1 / |d|^2
-// formed by two Newton steps r <- r (2 - s r) from the FP32 reciprocal (24, 48, then 53 bits), eight
-// dependent FP64 operations instead of a complex division's four quotients: the reciprocal is on
-// the serial chain of every pivot and an FP64 instruction takes 64 cycles.
-__device__ __forceinline__ cplx x_recip(const cplx& d) {
-  const int ex = max((__double2hiint(d.x) >> 20) & 0x7ff, (__double2hiint(d.y) >> 20) & 0x7ff);
-  if (ex < 64 || ex > 1980) return cabs2(d) > 0.0 ? cdiv(cmk(1.0, 0.0), d) : cmk(0.0, 0.0);
-  const double sc = __hiloint2double((2046 - ex) << 20, 0);  // 2^(1023 - ex)
-  const double x = d.x * sc, y = d.y * sc;
-  const double m = fma(x, x, y * y);  // in [1, 8)
-  double r = (double)(1.0f / (float)m);
-  r = fma(r, fma(-m, r, 1.0), r);
-  r = fma(r, fma(-m, r, 1.0), r);
-  r *= sc;
-  return cmk(x * r, -y * r);
-}
-__device__ __forceinline__ dfc x_recip(const dfc& d) { return dfc_recip(d); }
-__device__ __forceinline__ cplx x_neg(const cplx& a) { return cmk(-a.x, -a.y); }
-__device__ __forceinline__ dfc x_neg(const dfc& a) { return {-a.rh, -a.rl, -a.ih, -a.il}; }
-__device__ __forceinline__ cplx x_mul(const cplx& a, const cplx& b) { return cmul(a, b); }
-__device__ __forceinline__ dfc x_mul(const dfc& a, const dfc& b) { return dfc_mul(a, b); }
-// acc += a b (low parts lazy for dfc; x_norm finishes)
-__device__ __forceinline__ void x_mac(const cplx& a, const cplx& b, cplx& acc) { acc = cfma(a, b, acc); }
-__device__ __forceinline__ void x_mac(const dfc& a, const dfc& b, dfc& acc) {
-  df_mac(a.rh, a.rl, b.rh, b.rl, acc.rh, acc.rl);
-  df_mac(-a.ih, -a.il, b.ih, b.il, acc.rh, acc.rl);
-  df_mac(a.rh, a.rl, b.ih, b.il, acc.ih, acc.il);
-  df_mac(a.ih, a.il, b.rh, b.rl, acc.ih, acc.il);
-}
-__device__ __forceinline__ void x_norm(cplx&) {}
-__device__ __forceinline__ void x_norm(dfc& a) { dfc_norm(a); }
-__device__ __forceinline__ cplx x_in(const cplx& v, const cplx*) { return v; }
-__device__ __forceinline__ dfc x_in(const cplx& v, const dfc*) { return to_dfc_bits(v); }
-__device__ __forceinline__ cplx x_out(const cplx& v) { return v; }
-__device__ __forceinline__ cplx x_out(const dfc& v) { return from_dfc_bits(v); }
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool ok) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -142,11 +103,6 @@ __device__ __forceinline__ T* x_col(const GjxMat& mt, int j) {
   return j < mt.n ? reinterpret_cast<T*>(mt.A) + (int64_t)j * mt.n
                   : reinterpret_cast<T*>(mt.B) + (int64_t)(j - mt.n) * mt.n;
 }
-
-__device__ __forceinline__ cplx x_shfl(const cplx& v, int l) {
-  return cmk(__shfl_sync(0xffffffffu, v.x, l), __shfl_sync(0xffffffffu, v.y, l));
-}
-__device__ __forceinline__ dfc x_shfl(const dfc& v, int l) { return dfc_shfl(v, l); }
 
 // Rows of a cluster's CTA: `chunk` consecutive ones each.
 __device__ __forceinline__ int x_chunk(int n, int CS) { return (((n + CS - 1) / CS) + 31) & ~31; }

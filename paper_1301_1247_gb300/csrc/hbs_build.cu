@@ -539,8 +539,6 @@ DevGeom Handle_geom(const Handle& h) {
   return g;
 }
 
-// Work above which one matrix is decomposed by the multi-CTA kernels instead of one CTA.
-static bool big_cpqr(const CpqrJob& j) { return (double)j.m * j.n * std::min(j.m, j.n) > 4e6; }
 static bool big_inverse(int n) { return n > 72; }
 
 // Largest root (sum of the level-2 skeletons) for which level 1 is left uncompressed.  At the
@@ -555,69 +553,41 @@ static bool passthrough_level(const Handle& h, int l) {
   return lv.n.size() == 2 && lv.n[0] + lv.n[1] <= kPassThroughRootMax;
 }
 
-// Batched CPQR-ID of the matrices described by `jobs`.  Returns ranks.
-// Small matrices go to one launch with one CTA each; large ones (the top tree levels,
-// where a level has few nodes) share one persistent launch on all SMs (pqr.cu).
+// Pivoted-QR IDs of the matrices described by `jobs` on all SMs (pqr.cu), in launches of at most 128
+// matrices.  Returns the ranks.
 std::vector<int> batched_id(std::vector<CpqrJob>& jobs, double tol, cudaStream_t s) {
-  std::vector<int> ranks(jobs.size(), 0);
-  if (jobs.empty()) return ranks;
-  std::vector<CpqrJob> small;
-  std::vector<size_t> small_idx, big_idx;
-  // A level with at most 128 nodes runs all of them in one persistent multi-CTA launch
-  // (pqr.cu): one CTA per node would leave SMs idle and serialize on its largest node (at
-  // N = 10^5 the 128-node level took 80 ms that way against 28 ms in the persistent
-  // launch).  With more nodes, one CTA per node keeps every SM busy, and only the large
-  // nodes (if at most 128 of them) go to the persistent launch.
-  size_t nbig = 0;
-  for (const auto& j : jobs) nbig += big_cpqr(j) ? 1 : 0;
-  const bool all_big = jobs.size() <= 128;
-  const bool use_big = all_big || (nbig > 0 && nbig <= 128);
-  for (size_t i = 0; i < jobs.size(); ++i) {
-    if (use_big && (all_big || big_cpqr(jobs[i]))) {
-      big_idx.push_back(i);
-    } else {
-      small_idx.push_back(i);
-      small.push_back(jobs[i]);
-      small.back().job = (int)(small.size() - 1);
-    }
-  }
-  if (!small.empty()) {
-    int maxn = 0;
-    for (auto& j : small) maxn = std::max(maxn, j.n);
-    DevBuf<CpqrJob> dj = upload_jobs(small, s);
-    DevBuf<int> dr(small.size());
-    size_t sm = (size_t)maxn * (2 * sizeof(double) + sizeof(int));
-    // double-float updates on handles built with double-float precision
-    const bool df = gemm_double_float();
-    HBS_CUDA(raise_smem_limit(df ? (const void*)k_cpqr<256, true> : (const void*)k_cpqr<256, false>, sm));
-    {
-      prof::KScope _ks("k_cpqr", s);
-      if (df) k_cpqr<256, true><<<(unsigned)small.size(), 256, sm, s>>>(dj.get(), dr.get(), tol, 1 << 30);
-      else k_cpqr<256, false><<<(unsigned)small.size(), 256, sm, s>>>(dj.get(), dr.get(), tol, 1 << 30);
-    }
-    HBS_LAUNCH_CHECK("k_cpqr");
-    auto r = dr.download(s);
-    for (size_t t = 0; t < small.size(); ++t) ranks[small_idx[t]] = r[t];
-  }
-  if (!big_idx.empty()) {
+  std::vector<int> ranks;
+  for (size_t j0 = 0; j0 < jobs.size(); j0 += 128) {
     std::vector<BigQrJobSpec> specs;
-    for (size_t i : big_idx) {
-      const CpqrJob& j = jobs[i];
-      specs.push_back({j.mt, j.m, j.n, j.perm, j.t});
-    }
-    auto r = big_row_id_batched(specs, tol, s);
-    for (size_t t = 0; t < big_idx.size(); ++t) ranks[big_idx[t]] = r[t];
+    for (size_t i = j0; i < std::min(jobs.size(), j0 + 128); ++i)
+      specs.push_back({jobs[i].mt, jobs[i].m, jobs[i].n, jobs[i].perm, jobs[i].t});
+    const auto r = big_row_id_batched(specs, tol, s);
+    ranks.insert(ranks.end(), r.begin(), r.end());
   }
-  // algorithmic work of an interpolative decomposition of an m x n block of rank k: 8 m n k
-  // flops (the Householder factorization executes about twice that), and the block read
-  // once plus the interpolation matrix and the order written once
-  double fl = 0.0, by = 0.0;
-  for (size_t i = 0; i < jobs.size(); ++i) {
-    const double m = jobs[i].m, n = jobs[i].n, k = ranks[i];
-    fl += 8.0 * m * n * k;
-    by += 16.0 * m * n + 16.0 * k * (n - k) + 4.0 * n;
+  return ranks;
+}
+
+// IDs of a level's node matrices: in the shared memory of clusters (cqr.cu) where they fit, the others on all
+// SMs (pqr.cu).  Where some of at most 128 do not fit, all of them share one launch on all SMs.  In FP64,
+// where the multiply-adds weigh more than a step's chain, so do levels of fewer than 8 nodes that would
+// keep a cluster's FP64 pipes (eight SMs, 66 GFLOP/s) busy for more than a millisecond.
+static std::vector<int> node_ids(std::vector<CpqrJob>& jobs, double tol, cudaStream_t s) {
+  const bool df = gemm_double_float();
+  std::vector<size_t> in, out;
+  for (size_t i = 0; i < jobs.size(); ++i)
+    (cqr_cluster(jobs[i].m, jobs[i].n, jobs.size(), df) > 0 ? in : out).push_back(i);
+  double most = 0.0;  // multiply-adds of the largest decomposition, at a rank of about 0.6 n
+  for (const auto& j : jobs) most = std::max(most, 5.3 * j.m * (double)j.n * j.n);
+  if ((!out.empty() && jobs.size() <= 128) || (!df && jobs.size() < 8 && most > 66e6))
+    return batched_id(jobs, tol, s);
+  if (out.empty()) return cqr_run(jobs, tol, s);
+  std::vector<int> ranks(jobs.size(), 0);
+  for (const auto* part : {&in, &out}) {
+    std::vector<CpqrJob> pj;
+    for (size_t i : *part) pj.push_back(jobs[i]);
+    const std::vector<int> r = part == &in ? cqr_run(pj, tol, s) : batched_id(pj, tol, s);
+    for (size_t q = 0; q < part->size(); ++q) ranks[(*part)[q]] = r[q];
   }
-  prof::add_work("k_cpqr", fl, by);
   return ranks;
 }
 
@@ -1063,7 +1033,7 @@ void build_hbs_multi(const std::vector<Handle*>& hs, cudaStream_t s) {
                         (int)cj.size()});
         }
       }
-      std::vector<int> ranks = batched_id(cj, tasks[0].h->tol, s);
+      std::vector<int> ranks = node_ids(cj, tasks[0].h->tol, s);
       for (size_t i = 0; i < tasks.size(); ++i) {
         Handle& h = *tasks[i].h;
         Level& lv = h.levels[tasks[i].l];

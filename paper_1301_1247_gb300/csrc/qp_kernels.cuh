@@ -88,6 +88,10 @@ bool ozaki_eligible_short(const GemmJob& j);
 constexpr double kOzakiShortWork = 5e7;
 void ozaki_gemm_batched(const std::vector<GemmJob>& jobs, cudaStream_t s);
 std::vector<int> batched_id(std::vector<CpqrJob>& jobs, double tol, cudaStream_t s);
+// cqr.cu: the same with each matrix in the shared memory of one cluster; the cluster size for matrices up to
+// m x n in a batch of `count` (0: they do not fit).
+int cqr_cluster(int m, int n, size_t count, bool df);
+std::vector<int> cqr_run(const std::vector<CpqrJob>& jobs, double tol, cudaStream_t s);
 __global__ void k_geom(const double* dx, const double* dy, double* nx, double* ny, double* w, int64_t n);
 
 // qp_kernels.cu
