@@ -67,13 +67,6 @@ struct PqrJob {
   GridSync* gs;  // barrier of this matrix's CTAs
 };
 
-template <int NT>
-__device__ __forceinline__ cplx block_sum_c(cplx v, double* red) {
-  double a = block_sum<NT>(v.x, red);
-  double b = block_sum<NT>(v.y, red);
-  return cmk(a, b);
-}
-
 // Warp sum of a complex value with five FP64 additions instead of ten: after the first
 // exchange the lower half-warp carries real parts and the upper half imaginary parts.
 // The pairs added are those of the plain butterfly, so the sum is bitwise the same.
@@ -869,28 +862,39 @@ void pqr_solve_r11(const cplx* A, int64_t m, const PqrOut& qr, int job, int k, c
 }
 
 // Column j of conj(Q1) (Q1 = first k columns of H_0 ... H_{k-1}):  q = H_0 ... H_j e_j.
-// One CTA per column; q lives in the output column.
-__global__ void __launch_bounds__(kNT) k_form_qc(const cplx* A, int64_t m, const int* piv, const cplx* v0,
-                                                 const double* tau, int k, cplx* Qc) {
-  __shared__ double red[32];
+// One CTA per column; q lives in the output column, each thread keeping to its own rows (i mod 256), so that
+// a reflector costs one barrier: the warps' partial sums meet in a buffer that alternates, and every
+// thread adds them up.  The chain of the k reflectors bounds it (200 of 512 rows: 0.7 ms with the sums
+// formed by block reductions, 0.4 now), so the families' chains run side by side (blockIdx.y).
+__global__ void __launch_bounds__(kNT) k_form_qc(const QcJobs jobs, int64_t m) {
+  __shared__ cplx part[2][kNW];
+  const QcJob jb = jobs.j[blockIdx.y];
+  const cplx *A = jb.A, *v0 = jb.v0;
+  const int* piv = jb.piv;
+  const double* tau = jb.tau;
+  cplx* Qc = jb.Qc;
   const int j = blockIdx.x;
-  if (j >= k) return;
+  if (j >= jb.k) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   cplx* q = Qc + (int64_t)j * m;
-  for (int64_t i = threadIdx.x; i < m; i += kNT) q[i] = cmk(i == j ? 1.0 : 0.0, 0.0);
-  __syncthreads();
+  for (int64_t i = tid; i < m; i += kNT) q[i] = cmk(i == j ? 1.0 : 0.0, 0.0);
   for (int s = j; s >= 0; --s) {
     const cplx* ap = A + (int64_t)piv[s] * m;
     const cplx h0 = v0[s];
+    const double t = tau[s];
+    const int64_t i0 = s <= tid ? tid : tid + (int64_t)((s - tid + kNT - 1) / kNT) * kNT;  // first own row >= s
     cplx w = cmk(0.0, 0.0);
-    if (threadIdx.x == 0) w = cmul(cconj(h0), q[s]);
-    for (int64_t i = s + 1 + threadIdx.x; i < m; i += kNT) w = cfma(cconj(ap[i]), q[i], w);
-    w = block_sum_c<kNT>(w, red);
-    w = cscale(w, tau[s]);
-    if (threadIdx.x == 0) q[s] = cfms(h0, w, q[s]);
-    for (int64_t i = s + 1 + threadIdx.x; i < m; i += kNT) q[i] = cfms(ap[i], w, q[i]);
+    for (int64_t i = i0; i < m; i += kNT) w = cfma(cconj(i == s ? h0 : ap[i]), q[i], w);
+    w = warp_sum_c(w);
+    if (lane == 0) part[s & 1][warp] = w;
     __syncthreads();
+    w = part[s & 1][0];
+#pragma unroll
+    for (int u = 1; u < kNW; ++u) w = cadd(w, part[s & 1][u]);
+    w = cscale(w, t);
+    for (int64_t i = i0; i < m; i += kNT) q[i] = cfms(i == s ? h0 : ap[i], w, q[i]);
   }
-  for (int64_t i = threadIdx.x; i < m; i += kNT) q[i] = cconj(q[i]);
+  for (int64_t i = tid; i < m; i += kNT) q[i] = cconj(q[i]);
 }
 
 // R11 (k x k, row-major) from the factored matrix.

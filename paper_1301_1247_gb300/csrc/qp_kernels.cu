@@ -421,30 +421,6 @@ __global__ void k_expand_rows(const cplx* in, int64_t ldi, int ncol, const int2*
   }
 }
 
-// Column expansion by recipe: out[:, o] = in[:, idx] (kind 0), or sum_i T[i, idx] in[:, col(i)]
-// with col(i) = skel ? skel[i] : off + i (kind 1).
-__global__ void k_expand_cols(const cplx* in, int64_t ldi, int nrow, const int2* recipe, int nout, const cplx* T, int r,
-                              int off, const int* skel, cplx* out, int64_t ldo) {
-  const int64_t tot = (int64_t)nrow * nout;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
-    const int rw = (int)(e % nrow);
-    const int o = (int)(e / nrow);
-    const int2 rc = recipe[o];
-    cplx v;
-    if (rc.x == 0) {
-      v = in[rw + (int64_t)rc.y * ldi];
-    } else {
-      const cplx* tc = T + (int64_t)rc.y * r;
-      v = cmk(0, 0);
-      for (int i = 0; i < r; ++i) {
-        const int cc = skel ? skel[i] : off + i;
-        v = cfma(tc[i], in[rw + (int64_t)cc * ldi], v);
-      }
-    }
-    out[rw + (int64_t)o * ldo] = v;
-  }
-}
-
 // acc[0] += |a - b|^2, acc[1] += |b|^2 over an nrow x ncol block.
 __global__ void k_diff_norm2(const cplx* a, int64_t lda, const cplx* b, int64_t ldb, int nrow, int ncol, double* acc) {
   __shared__ double red[2][32];

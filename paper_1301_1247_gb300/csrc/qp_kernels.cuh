@@ -62,8 +62,19 @@ void batched_inverse(std::vector<InvJob>& jobs, cudaStream_t s, const char* what
 // X(:, c) = R^{-1} B(:, c) for upper-triangular R (k x k, row-major); X may alias B.
 __global__ void k_tsolve_cols(const cplx* R, int k, const cplx* B, int64_t ldb, int64_t ncols, cplx* X, int64_t ldx);
 // Columns of conj(Q1), Q1 = the first k columns of the factorization's Q (m x k, ld m).
-__global__ void k_form_qc(const cplx* A, int64_t m, const int* piv, const cplx* v0, const double* tau, int k,
-                          cplx* Qc);
+// Q1 of up to three factorizations of m-row matrices (reflectors as a pqr_run leaves them).
+struct QcJob {
+  const cplx* A;
+  const int* piv;
+  const cplx* v0;
+  const double* tau;
+  int k;
+  cplx* Qc;  // m x k
+};
+struct QcJobs {
+  QcJob j[3];
+};
+__global__ void k_form_qc(const QcJobs jobs, int64_t m);
 __global__ void k_r11_rows(const cplx* A, int64_t m, const int* piv, const cplx* beta, int k, cplx* R);
 __global__ void k_gather_cols(const cplx* src, int64_t lds, int64_t rows, const int64_t* idx, int64_t ncols, cplx* out,
                               int64_t ldo);
@@ -137,8 +148,6 @@ __global__ void k_gather_subcols_t(const cplx* src, int64_t lds, int nrows, cons
 __global__ void k_gather_rowrefs(const RowRef* refs, int nsel, int64_t ncol, cplx* out, int64_t ldo);
 __global__ void k_expand_rows(const cplx* in, int64_t ldi, int ncol, const int2* recipe, int nout, const cplx* T1,
                               int r1, int off1, const cplx* T2, int r2, int off2, cplx* out, int64_t ldo);
-__global__ void k_expand_cols(const cplx* in, int64_t ldi, int nrow, const int2* recipe, int nout, const cplx* T, int r,
-                              int off, const int* skel, cplx* out, int64_t ldo);
 __global__ void k_fill_dirs(DevGeom g, double cx, double cy, int K, cplx* out);
 __global__ void k_transpose(const cplx* in, int64_t rows, int64_t cols, cplx* out);
 __global__ void k_diff_norm2(const cplx* a, int64_t lda, const cplx* b, int64_t ldb, int nrow, int ncol, double* acc);
