@@ -744,6 +744,7 @@ struct GroupJob {
   int64_t s_off, r_off;      // offsets of S (nS x nS) and rhs (nS x q) in the pools
   int64_t piv_off;
   int nsys;                  // size of the Schur system solved for this group
+  int a0;                    // first angle of this group among the batch's
   // reduced path (compressed periodizer): per-group work arrays
   const cplx* ul;            // U_L, U_R (2M x rC): C_L, C_R rows from the skeleton rows
   const cplx* ur;
@@ -1330,11 +1331,6 @@ __global__ void k_red_tables(RedDims D, Dims DD, const GroupJob* groups) {
   }
 }
 
-// psi_t(s) for s in [S, 4S) from the group's table.
-__device__ __forceinline__ cplx wood_psi_tab(const GroupJob& G, int S, int t, int sidx) {
-  return G.wpsi[(int64_t)t * 3 * S + (sidx - S)];
-}
-
 // Per group: vt = (V_L + alpha V_R)^T and qu = Q^{-1} (alpha U_L - alpha^{-2} U_R).
 __global__ void k_red_prep(RedDims D, const GroupJob* groups) {
   const GroupJob G = groups[blockIdx.y];
@@ -1359,233 +1355,227 @@ __global__ void k_red_prep(RedDims D, const GroupJob* groups) {
   }
 }
 
-// Wood's rows of one group: wd[t] = [psi_t^T Wall(alpha) (2M) | that times qu (rC)].
-__global__ void k_red_wood(RedDims D, const GroupJob* groups, Dims DD) {
-  const GroupJob G = groups[blockIdx.x];
-  if (G.nw == 0) return;
-  const int M2 = 2 * D.M, S4 = 4 * D.S;
-  for (int t = 0; t < G.nw; ++t) {
-    cplx* w = G.wd + (int64_t)t * (M2 + D.rC);
-    for (int mm = threadIdx.x; mm < M2; mm += blockDim.x) {
-      cplx acc = cmk(0, 0);
-      for (int sidx = D.S; sidx < S4; ++sidx) {
-        cplx p = wood_psi_tab(G, D.S, t, sidx);
-        if (p.x == 0.0 && p.y == 0.0) continue;
-        acc = cfma(p, cfma(G.alpha, G.sr[(int64_t)mm * S4 + sidx], G.sl[(int64_t)mm * S4 + sidx]), acc);
-      }
-      w[mm] = acc;
-    }
-    __syncthreads();
-    for (int c = threadIdx.x; c < D.rC; c += blockDim.x) {
-      cplx acc = cmk(0, 0);
-      for (int mm = 0; mm < M2; ++mm) acc = cfma(w[mm], G.qu[mm + (int64_t)c * M2], acc);
-      w[M2 + c] = acc;
-    }
-    __syncthreads();
+// Wood's rows: wd[t] = [psi_t^T Wall(alpha) (2M) | that times qu (rC)], mode t = blockIdx.y of group
+// blockIdx.z, one warp an entry: its first part here, the second below.  The FP64 multiply-adds bound
+// both (about a million an SM would take 0.2 ms over), so a mode is spread over blockIdx.x.
+__device__ __forceinline__ cplx lane_sum(cplx v) {
+  for (int o = 16; o > 0; o >>= 1) {
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+    v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+  }
+  return v;
+}
+
+__global__ void __launch_bounds__(256) k_red_wood_wall(RedDims D, const GroupJob* groups) {
+  const GroupJob G = groups[blockIdx.z];
+  const int t = blockIdx.y, lane = threadIdx.x & 31;
+  if (t >= G.nw) return;
+  const int M2 = 2 * D.M, S4 = 4 * D.S, S3 = 3 * D.S;
+  const cplx* psi = G.wpsi + (int64_t)t * S3;
+  cplx* w = G.wd + (int64_t)t * (M2 + D.rC);
+  for (int mm = (blockIdx.x * 256 + threadIdx.x) >> 5; mm < M2; mm += gridDim.x * 8) {
+    const int64_t o = (int64_t)mm * S4 + D.S;
+    cplx acc = cmk(0, 0);
+    for (int i = lane; i < S3; i += 32) acc = cfma(psi[i], cfma(G.alpha, G.sr[o + i], G.sl[o + i]), acc);
+    acc = lane_sum(acc);
+    if (lane == 0) w[mm] = acc;
   }
 }
 
-// phi_t . X: Wood's sampling functional over the three images' E rows (ld 12S column X).
-__device__ __forceinline__ cplx wood_phi(const Dims& DD, const GroupJob& G, int t, const cplx* X) {
-  const int S = DD.S;
-  cplx acc = cmk(0, 0);
-  cplx aj = cdiv(cmk(1, 0), G.alpha);
-  for (int jj = 0; jj < 3; ++jj) {
-    cplx part = cmk(0, 0);
-    for (int sidx = S; sidx < 4 * S; ++sidx) {
-      cplx p = wood_psi_tab(G, S, t, sidx);
-      if (p.x == 0.0 && p.y == 0.0) continue;
-      part = cfma(p, X[4 * S * jj + sidx], part);
-    }
-    acc = cfma(aj, part, acc);
-    aj = cmul(aj, G.alpha);
+__global__ void __launch_bounds__(256) k_red_wood_qu(RedDims D, const GroupJob* groups) {
+  const GroupJob G = groups[blockIdx.z];
+  const int t = blockIdx.y, lane = threadIdx.x & 31;
+  if (t >= G.nw) return;
+  const int M2 = 2 * D.M;
+  cplx* w = G.wd + (int64_t)t * (M2 + D.rC);
+  for (int c = (blockIdx.x * 256 + threadIdx.x) >> 5; c < D.rC; c += gridDim.x * 8) {
+    cplx acc = cmk(0, 0);
+    for (int mm = lane; mm < M2; mm += 32) acc = cfma(w[mm], G.qu[mm + (int64_t)c * M2], acc);
+    acc = lane_sum(acc);
+    if (lane == 0) w[M2 + c] = acc;
   }
-  return acc;
 }
 
-__global__ void k_red_assemble(RedDims D, Dims DD, const GroupJob* groups, const cplx* Zc, const cplx* Psel,
-                               const cplx* EZ, const cplx* EP, double y0, cplx* Spool, cplx* Rpool) {
+// A reduced unknown's or right-hand side's column C: its kind (0 zeta, 1 beta, 2 Wood, 3 right-hand side),
+// its index among that kind, its factor, and its column of Zc / EZ or of the projections.
+struct RedCol {
+  int kind, idx, zcol, pcol;
+  cplx f;
+};
+__device__ __forceinline__ RedCol red_col(const RedDims& D, const GroupJob& G, int C, cplx ia) {
+  RedCol r;
+  const int l = D.l, rB = D.rB;
+  r.f = cmk(1, 0);
+  if (C >= G.nsys) { r.kind = 3; r.idx = C - G.nsys; }
+  else if (C < 2 * l) { r.kind = 0; r.idx = C < l ? C : C - l; r.f = C < l ? ia : G.alpha; }
+  else if (C < 2 * l + rB) { r.kind = 1; r.idx = C - 2 * l; }
+  else { r.kind = 2; r.idx = C - 2 * l - rB; }
+  r.zcol = r.kind == 0 ? r.idx : (r.kind == 1 ? l + r.idx : -1);
+  r.pcol = r.kind == 2 ? G.rhs_col + G.q + r.idx : (r.kind == 3 ? G.rhs_col + r.idx : -1);
+  return r;
+}
+
+// Rows of the neighbour unknowns and of beta; Wood's rows follow in k_red_wood_rows.
+__global__ void k_red_assemble(RedDims D, const GroupJob* groups, const cplx* Zc, const cplx* Psel, cplx* Spool,
+                               cplx* Rpool) {
   const GroupJob G = groups[blockIdx.y];
-  const int l = D.l, rB = D.rB, rC = D.rC, rsel = D.rsel, S12 = 12 * D.S;
-  const int n = G.nsys, M2 = 2 * D.M;
+  const int l = D.l, rB = D.rB, rsel = D.rsel, n = G.nsys, nr = 2 * l + rB;
   const cplx ia = cdiv(cmk(1, 0), G.alpha);
-  const int64_t tot = (int64_t)n * (n + G.q);
+  const int64_t tot = (int64_t)nr * (n + G.q);
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
-    const int r = (int)(e % n);
-    const int C = (int)(e / n);
-    // column description
-    int kind, idx;  // 0 zeta (base col idx, factor f), 1 beta (idx), 2 Wood (idx), 3 rhs (idx)
-    cplx f = cmk(1, 0);
-    if (C >= n) { kind = 3; idx = C - n; }
-    else if (C < 2 * l) { kind = 0; idx = C < l ? C : C - l; f = C < l ? ia : G.alpha; }
-    else if (C < 2 * l + rB) { kind = 1; idx = C - 2 * l; }
-    else { kind = 2; idx = C - 2 * l - rB; }
-    // Zc / Psel column for this unknown
-    const int zcol = kind == 0 ? idx : (kind == 1 ? l + idx : -1);
-    const int pcol = kind == 2 ? G.rhs_col + G.q + idx : (kind == 3 ? G.rhs_col + idx : -1);
+    const int r = (int)(e % nr);
+    const int C = (int)(e / nr);
+    const RedCol rc = red_col(D, G, C, ia);
     cplx v;
     if (r < 2 * l) {
-      if (zcol >= 0) v = cmul(f, Zc[r + (int64_t)zcol * rsel]);
-      else v = Psel[r + (int64_t)pcol * rsel];
+      if (rc.zcol >= 0) v = cmul(rc.f, Zc[r + (int64_t)rc.zcol * rsel]);
+      else v = Psel[r + (int64_t)rc.pcol * rsel];
       v = cmk(-v.x, -v.y);
-      if (kind == 0 && C == r) v.x -= 1.0;
-    } else if (r < 2 * l + rB) {
-      const int ii = r - 2 * l;
-      const int hcol = kind == 0 ? idx : (kind == 1 ? l + idx : (kind == 2 ? l + rB + G.q + idx : l + rB + idx));
-      v = cmul(f, G.hc[ii + (int64_t)hcol * rB]);
-      v = cmk(-v.x, -v.y);
-      if (kind == 1 && idx == ii) v.x += 1.0;
+      if (rc.kind == 0 && C == r) v.x -= 1.0;
     } else {
-      const int tw = r - 2 * l - rB;
-      const cplx* w = G.wd + (int64_t)tw * (M2 + rC) + M2;
-      const cplx* X = zcol >= 0 ? EZ + (int64_t)zcol * S12 : EP + (int64_t)pcol * S12;
-      cplx ph = wood_phi(DD, G, tw, X);
-      cplx wz = cmk(0, 0);
-      if (zcol >= 0)
-        for (int c = 0; c < rC; ++c) wz = cfma(w[c], Zc[2 * l + c + (int64_t)zcol * rsel], wz);
-      else
-        for (int c = 0; c < rC; ++c) wz = cfma(w[c], Psel[2 * l + c + (int64_t)pcol * rsel], wz);
-      v = cmul(f, csub(wz, ph));
-      if (kind == 2) {
-        cplx acc = cmk(0, 0);
-        for (int sidx = D.S; sidx < 4 * D.S; ++sidx) {
-          cplx p = wood_psi_tab(G, D.S, tw, sidx);
-          if (p.x == 0.0 && p.y == 0.0) continue;
-          acc = cfma(p, sample_point_pw(DD, G, idx, sidx, y0), acc);
-        }
-        v = cadd(v, acc);
-      }
+      const int ii = r - 2 * l;
+      const int hcol = rc.zcol >= 0 ? rc.zcol : (rc.kind == 2 ? l + rB + G.q + rc.idx : l + rB + rc.idx);
+      v = cmul(rc.f, G.hc[ii + (int64_t)hcol * rB]);
+      v = cmk(-v.x, -v.y);
+      if (rc.kind == 1 && rc.idx == ii) v.x += 1.0;
     }
-    if (kind == 3) Rpool[G.r_off + (int64_t)idx * n + r] = v;
+    if (rc.kind == 3) Rpool[G.r_off + (int64_t)rc.idx * n + r] = v;
     else Spool[G.s_off + (int64_t)C * n + r] = v;
   }
 }
 
-// Sum_j A[j ld] x[j] for an FP64 column-strided A and a vector x in shared memory: in FP64,
-// or (DF) in double-float on the FP32 pipes, A split on load and x already held as pairs,
-// renormalised every 8 terms.  Eight loads of A are issued together ahead of their
-// multiply-adds (each thread runs a long dot product alone; one load at a time would wait
-// out the L2 latency at every term).
-template <bool DF>
-__device__ __forceinline__ cplx red_dot(const cplx* A, int64_t ld, const cplx* x, int n) {
-  if constexpr (DF) {
-    const dfc* xd = reinterpret_cast<const dfc*>(x);
-    dfc acc{0.f, 0.f, 0.f, 0.f};
-    int j = 0;
-    for (; j + 8 <= n; j += 8) {
-      cplx a[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) a[q] = A[(int64_t)(j + q) * ld];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) dfc_mac_tile(to_dfc_bits(a[q]), xd[j + q], acc);
-      dfc_norm(acc);
-    }
-    for (; j < n; ++j) dfc_mac_tile(to_dfc_bits(A[(int64_t)j * ld]), xd[j], acc);
-    dfc_norm(acc);
-    return from_dfc_bits(acc);
-  } else {
-    cplx acc = cmk(0, 0);
-    int j = 0;
-    for (; j + 8 <= n; j += 8) {
-      cplx a[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) a[q] = A[(int64_t)(j + q) * ld];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) acc = cfma(a[q], x[j + q], acc);
-    }
-    for (; j < n; ++j) acc = cfma(A[(int64_t)j * ld], x[j], acc);
-    return acc;
-  }
-}
-
-// Entry i of a shared vector read by red_dot: FP64, or (DF) its double-float pair in place.
-template <bool DF>
-__device__ __forceinline__ void red_store(cplx* x, int i, cplx v) {
-  if constexpr (DF) reinterpret_cast<dfc*>(x)[i] = to_dfc_bits(v);
-  else x[i] = v;
-}
-
-// Bragg amplitudes from the reduced solution: gamma, xi = Q^{-1} U gamma, samples, DFT.
-// The image columns of the neighbour unknowns enter as w = [alpha^{-1} u_1 + alpha u_2; u_B]
-// (both images' columns of Z and of the E rows are the same skeleton columns).
-template <bool DF>
-__global__ void k_red_bragg(RedDims D, Dims DD, const GroupJob* groups, const AngleJob* angles, const cplx* Zc,
-                            const cplx* Psel, const cplx* EZ, const cplx* EP, const cplx* Rpool, double y0,
-                            cplx* cout, cplx* dout, double* flux) {
-  extern __shared__ cplx sh[];
-  const AngleJob A = angles[blockIdx.x];
-  const GroupJob G = groups[A.group];
-  const int l = D.l, rB = D.rB, rC = D.rC, rsel = D.rsel, S = D.S, S4 = 4 * D.S, S12 = 12 * D.S, M2 = 2 * D.M;
-  const int n = G.nsys, nz = l + rB;
-  cplx* w = sh;
-  cplx* gam = sh + nz;
-  cplx* xi = gam + rC;
-  cplx* samp = xi + M2;
-  const cplx* u = Rpool + G.r_off + (int64_t)A.col * n;
+// Wood's row t (blockIdx.y) of group blockIdx.z: w . gamma(C) - phi_t . X(C) for every column C, with X the
+// column's E rows over the three images (9S + rC terms).  One warp a column: one thread a column, beside
+// the other rows' one-term entries, held the assembly up for 0.2 ms.
+__global__ void __launch_bounds__(256) k_red_wood_rows(RedDims D, Dims DD, const GroupJob* groups, const cplx* Zc,
+                                                       const cplx* Psel, const cplx* EZ, const cplx* EP, double y0,
+                                                       cplx* Spool, cplx* Rpool) {
+  const GroupJob G = groups[blockIdx.z];
+  const int t = blockIdx.y, lane = threadIdx.x & 31;
+  if (t >= G.nw) return;
+  const int l = D.l, rB = D.rB, rC = D.rC, rsel = D.rsel, S = D.S, S3 = 3 * D.S, S12 = 12 * D.S, n = G.nsys;
   const cplx ia = cdiv(cmk(1, 0), G.alpha);
-  for (int j = threadIdx.x; j < nz; j += blockDim.x)
-    red_store<DF>(w, j, j < l ? cadd(cmul(ia, u[j]), cmul(G.alpha, u[l + j])) : u[2 * l + (j - l)]);
-  __syncthreads();
-  for (int c = threadIdx.x; c < rC; c += blockDim.x) {
-    const int row = 2 * l + c;
-    cplx acc = red_dot<DF>(Zc + row, rsel, w, nz);
-    for (int t = 0; t < G.nw; ++t) acc = cfma(Psel[row + (int64_t)(G.rhs_col + G.q + t) * rsel], u[2 * l + rB + t], acc);
-    red_store<DF>(gam, c, csub(acc, Psel[row + (int64_t)(G.rhs_col + A.col) * rsel]));
-  }
-  __syncthreads();
-  for (int mm = threadIdx.x; mm < M2; mm += blockDim.x) red_store<DF>(xi, mm, red_dot<DF>(G.qu + mm, M2, gam, rC));
-  __syncthreads();
-  for (int r = threadIdx.x; r < 2 * S; r += blockDim.x) {
+  const cplx* psi = G.wpsi + (int64_t)t * S3;
+  const cplx* w = G.wd + (int64_t)t * (2 * D.M + rC) + 2 * D.M;
+  for (int C = (blockIdx.x * 256 + threadIdx.x) >> 5; C < n + G.q; C += gridDim.x * 8) {
+    const RedCol rc = red_col(D, G, C, ia);
+    const cplx* X = rc.zcol >= 0 ? EZ + (int64_t)rc.zcol * S12 : EP + (int64_t)rc.pcol * S12;
+    const cplx* gam = 2 * l + (rc.zcol >= 0 ? Zc + (int64_t)rc.zcol * rsel : Psel + (int64_t)rc.pcol * rsel);
     cplx acc = cmk(0, 0);
-    cplx aj = ia;
+    for (int c = lane; c < rC; c += 32) acc = cfma(w[c], gam[c], acc);
+    cplx aj = cmk(-ia.x, -ia.y);
     for (int jj = 0; jj < 3; ++jj) {
-      const int row = S4 * jj + r;
-      cplx part = csub(EP[row + (int64_t)(G.rhs_col + A.col) * S12], red_dot<DF>(EZ + row, S12, w, nz));
-      for (int t = 0; t < G.nw; ++t)
-        part = csub(part, cmul(EP[row + (int64_t)(G.rhs_col + G.q + t) * S12], u[2 * l + rB + t]));
+      cplx part = cmk(0, 0);
+      for (int i = lane; i < S3; i += 32) part = cfma(psi[i], X[4 * S * jj + S + i], part);
       acc = cfma(aj, part, acc);
       aj = cmul(aj, G.alpha);
     }
-    // the wall samples (SL + alpha SR) xi
-    acc = cadd(acc, red_dot<DF>(G.sl + r, S4, xi, M2));
-    acc = cfma(G.alpha, red_dot<DF>(G.sr + r, S4, xi, M2), acc);
-    for (int t = 0; t < G.nw; ++t) acc = cfma(sample_point_pw(DD, G, t, r, y0), u[2 * l + rB + t], acc);
+    cplx pw = cmk(0, 0);
+    if (rc.kind == 2)
+      for (int i = lane; i < S3; i += 32) pw = cfma(psi[i], sample_point_pw(DD, G, rc.idx, S + i, y0), pw);
+    const cplx v = lane_sum(cadd(cmul(rc.f, acc), pw));
+    if (lane) continue;
+    if (rc.kind == 3) Rpool[G.r_off + (int64_t)rc.idx * n + 2 * l + rB + t] = v;
+    else Spool[G.s_off + (int64_t)C * n + 2 * l + rB + t] = v;
+  }
+}
+
+// ---- Bragg amplitudes from the reduced solutions of a batch's angles: gamma, xi = Q^{-1} U gamma, the
+// samples on y = +-y0, their DFT.  The neighbour unknowns' image columns enter as
+// w = [alpha^{-1} u_1 + alpha u_2; u_B] (both images' columns of Z and of the E rows are the same skeleton
+// columns).  The products run as batched GEMMs over all angles: gamma and the E rows' samples share one
+// matrix, xi has one per group and the wall samples one per contour.  One CTA an angle, each thread with
+// dot products of up to 3 nz + 4M terms of its own, took 1.0 ms for 8 angles and 3.0 for 1000 (n = 400);
+// these launches and products take 0.35 and 1.4.
+
+// Column b = blockIdx.x of w.
+__global__ void k_red_w(RedDims D, const GroupJob* groups, const AngleJob* angles, const cplx* Rpool, cplx* W) {
+  const AngleJob A = angles[blockIdx.x];
+  const GroupJob& G = groups[A.group];
+  const int l = D.l, nz = D.l + D.rB;
+  const cplx alpha = G.alpha, ia = cdiv(cmk(1, 0), alpha);
+  const cplx* u = Rpool + G.r_off + (int64_t)A.col * G.nsys;
+  cplx* w = W + (int64_t)blockIdx.x * nz;
+  for (int j = threadIdx.x; j < nz; j += blockDim.x)
+    w[j] = j < l ? cadd(cmul(ia, u[j]), cmul(alpha, u[l + j])) : u[2 * l + (j - l)];
+}
+
+// gamma (column b, formed as C_sel w) += Wood's columns, -= the incident field's.
+__global__ void k_red_gamma(RedDims D, const GroupJob* groups, const AngleJob* angles, const cplx* Psel,
+                            const cplx* Rpool, cplx* Gam) {
+  const AngleJob A = angles[blockIdx.x];
+  const GroupJob& G = groups[A.group];
+  const cplx* a = Rpool + G.r_off + (int64_t)A.col * G.nsys + 2 * D.l + D.rB;
+  cplx* gam = Gam + (int64_t)blockIdx.x * D.rC;
+  const cplx* P = Psel + (int64_t)G.rhs_col * D.rsel + 2 * D.l;
+  for (int c = threadIdx.x; c < D.rC; c += blockDim.x) {
+    cplx acc = gam[c];
+    for (int t = 0; t < G.nw; ++t) acc = cfma(P[c + (int64_t)(G.q + t) * D.rsel], a[t], acc);
+    gam[c] = csub(acc, P[c + (int64_t)A.col * D.rsel]);
+  }
+}
+
+// Samples and their DFT.  E: rows 2S jj + r of image jj (6S x angles); XL, XR: the wall samples SL xi, SR xi
+// (2S x angles).  One warp an order, lanes over the samples: a sine and cosine each, so one thread an
+// order would run through S of them (0.3 ms).
+__global__ void __launch_bounds__(256) k_red_bragg(RedDims D, Dims DD, const GroupJob* groups, const AngleJob* angles,
+                                                   const cplx* E, const cplx* XL, const cplx* XR, const cplx* EP,
+                                                   const cplx* Rpool, double y0, cplx* cout, cplx* dout,
+                                                   double* flux) {
+  extern __shared__ cplx samp[];
+  __shared__ double fl[8];
+  const AngleJob A = angles[blockIdx.x];
+  const GroupJob G = groups[A.group];
+  const int S = D.S, S4 = 4 * D.S, S12 = 12 * D.S, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t b = blockIdx.x;
+  const cplx* a = Rpool + G.r_off + (int64_t)A.col * G.nsys + 2 * D.l + D.rB;
+  const cplx* ep = EP + (int64_t)G.rhs_col * S12;
+  for (int r = threadIdx.x; r < 2 * S; r += 256) {
+    cplx acc = cfma(G.alpha, XR[r + b * 2 * S], XL[r + b * 2 * S]);
+    cplx aj = cdiv(cmk(1, 0), G.alpha);
+    for (int jj = 0; jj < 3; ++jj) {
+      const int row = S4 * jj + r;
+      cplx part = csub(ep[row + (int64_t)A.col * S12], E[2 * S * jj + r + b * 6 * S]);
+      for (int t = 0; t < G.nw; ++t) part = csub(part, cmul(ep[row + (int64_t)(G.q + t) * S12], a[t]));
+      acc = cfma(aj, part, acc);
+      aj = cmul(aj, G.alpha);
+    }
+    for (int t = 0; t < G.nw; ++t) acc = cfma(sample_point_pw(DD, G, t, r, y0), a[t], acc);
     samp[r] = acc;
   }
   __syncthreads();
-  __shared__ double fl[32];
-  const int no = A.n_max - A.n_min + 1;
   double fsum = 0.0;
-  for (int o = threadIdx.x; o < no; o += blockDim.x) {
+  for (int o = warp; o < A.n_max - A.n_min + 1; o += 8) {
     const int nn = A.n_min + o;
     const double kap = A.kappa + 2.0 * HBS_PI * nn / D.d;
     cplx cn = cmk(0, 0), dn = cmk(0, 0);
-    for (int si = 0; si < S; ++si) {
+    for (int si = lane; si < S; si += 32) {
       const double xs = -0.5 * D.d + (si + 0.5) * D.d / S;
       double sn, cs;
       sincos(-kap * xs, &sn, &cs);
-      cplx ev = cmk(cs / S, sn / S);
+      const cplx ev = cmk(cs / S, sn / S);
       cn = cfma(ev, samp[si], cn);
       dn = cfma(ev, samp[S + si], dn);
     }
+    cn = lane_sum(cn);
+    dn = lane_sum(dn);
+    if (lane) continue;
     cout[A.out_off + o] = cn;
     dout[A.out_off + o] = dn;
     const double kn2 = D.omega * D.omega - kap * kap;
     const double kn = kn2 > 0 ? sqrt(kn2) : 0.0;
-    cplx dd = dn;
     if (nn == 0) {
       double sn, cs;
       sincos(A.k0 * y0, &sn, &cs);
-      dd = cadd(dd, cmk(cs, sn));
+      dn = cadd(dn, cmk(cs, sn));
     }
-    fsum += (kn / A.k0) * (cabs2(cn) + cabs2(dd));
+    fsum += (kn / A.k0) * (cabs2(cn) + cabs2(dn));
   }
-  for (int o = 16; o > 0; o >>= 1) fsum += __shfl_xor_sync(0xffffffffu, fsum, o);
-  if ((threadIdx.x & 31) == 0) fl[threadIdx.x >> 5] = fsum;
+  if (lane == 0) fl[warp] = fsum;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += fl[w];
+    for (int w = 0; w < 8; ++w) t += fl[w];
     flux[blockIdx.x] = fabs(t - 1.0);
   }
 }
@@ -1621,8 +1611,11 @@ static void reduced_batch(Handle& h, std::vector<GroupJob>& gjobs, std::vector<s
   }
   // per-group work arrays
   int64_t nvt = 0, nqu = 0, nhm = 0, nhc = 0, nwd = 0, nps = 0, so = 0, ro = 0;
+  int na0 = 0;
   for (auto& G : gjobs) {
     G.nsys = 2 * l + rB + G.nw;
+    G.a0 = na0;
+    na0 += G.q;
     nps += (int64_t)G.nw * 3 * S;
     nvt += (int64_t)rB * M2;
     nqu += (int64_t)M2 * rC;
@@ -1677,14 +1670,29 @@ static void reduced_batch(Handle& h, std::vector<GroupJob>& gjobs, std::vector<s
     }
     run_gemms(gj, s);
   }
-  {
-    prof::KScope _ks("k_red_wood", s);
-    k_red_wood<<<ng, 256, 0, s>>>(R, dg.get(), DD);
+  int nw = 0, nrow = 0;
+  for (auto& G : gjobs) {
+    nw = std::max(nw, G.nw);
+    nrow = std::max(nrow, G.nsys + G.q);
   }
   {
     prof::KScope _ks("k_red_assemble", s);
-    k_red_assemble<<<dim3(64, ng), 256, 0, s>>>(R, DD, dg.get(), h.Zc.get(), Psel, h.EZ.get(), EP.get(), h.y0,
-                                                 Sp.get(), Rp.get());
+    k_red_assemble<<<dim3(64, ng), 256, 0, s>>>(R, dg.get(), h.Zc.get(), Psel, Sp.get(), Rp.get());
+  }
+  if (nw > 0) {
+    {
+      prof::KScope _ks("k_red_wood_wall", s);
+      k_red_wood_wall<<<dim3(32, nw, ng), 256, 0, s>>>(R, dg.get());
+    }
+    {
+      prof::KScope _ks("k_red_wood_qu", s);
+      k_red_wood_qu<<<dim3(16, nw, ng), 256, 0, s>>>(R, dg.get());
+    }
+    {
+      prof::KScope _ks("k_red_wood_rows", s);
+      k_red_wood_rows<<<dim3((nrow + 7) / 8, nw, ng), 256, 0, s>>>(R, DD, dg.get(), h.Zc.get(), Psel, h.EZ.get(),
+                                                                   EP.get(), h.y0, Sp.get(), Rp.get());
+    }
   }
   HBS_LAUNCH_CHECK("k_red_assemble");
   DevBuf<int> ill(ng);
@@ -1709,21 +1717,51 @@ static void reduced_batch(Handle& h, std::vector<GroupJob>& gjobs, std::vector<s
   da.upload(ajobs, s);
   DevBuf<cplx> cbuf(std::max<int64_t>(oo, 1)), dbuf(std::max<int64_t>(oo, 1));
   DevBuf<double> fbuf(ajobs.size());
+  const int64_t na = (int64_t)ajobs.size();
+  const int nz = l + rB, S2 = 2 * S;
+  DevBuf<cplx> W(std::max<int64_t>(nz * na, 1)), Gam(std::max<int64_t>(rC * na, 1)), Eb(3 * S2 * na), Xi(M2 * na),
+      XL(S2 * na), XR(S2 * na);
+  {
+    prof::KScope _ks("k_red_w", s);
+    k_red_w<<<(unsigned)na, 256, 0, s>>>(R, dg.get(), da.get(), Rp.get(), W.get());
+  }
+  HBS_LAUNCH_CHECK("k_red_w");
+  {
+    const cplx one = cmk(1, 0), zero = cmk(0, 0);
+    const int q = (int)na;
+    std::vector<GemmJob> gj;
+    gj.push_back({h.Zc.get() + 2 * l, W.get(), Gam.get(), rC, q, nz, rsel, nz, rC, one, zero, 0, 0, 0, 0});
+    for (int jj = 0; jj < 3; ++jj)
+      gj.push_back({h.EZ.get() + 4 * S * jj, W.get(), Eb.get() + S2 * jj, S2, q, nz, S12, nz, 3 * S2, one, zero, 0, 0, 0,
+                    0});
+    run_gemms(gj, s);
+    {
+      prof::KScope _ks("k_red_gamma", s);
+      k_red_gamma<<<(unsigned)na, 256, 0, s>>>(R, dg.get(), da.get(), Psel, Rp.get(), Gam.get());
+    }
+    HBS_LAUNCH_CHECK("k_red_gamma");
+    gj.clear();
+    for (auto& G : gjobs)
+      gj.push_back({G.qu, Gam.get() + (int64_t)G.a0 * rC, Xi.get() + (int64_t)G.a0 * M2, M2, G.q, rC, M2, rC, M2, one,
+                    zero, 0, 0, 0, 0});
+    run_gemms(gj, s);
+    gj.clear();
+    for (int g0 = 0, g1; g0 < ng; g0 = g1) {  // consecutive groups on one contour
+      const GroupJob& G = gjobs[g0];
+      int cq = 0;
+      for (g1 = g0; g1 < ng && gjobs[g1].contour == G.contour; ++g1) cq += gjobs[g1].q;
+      const int64_t o = (int64_t)G.a0;
+      gj.push_back({G.sl, Xi.get() + o * M2, XL.get() + o * S2, S2, cq, M2, 4 * S, M2, S2, one, zero, 0, 0, 0, 0});
+      gj.push_back({G.sr, Xi.get() + o * M2, XR.get() + o * S2, S2, cq, M2, 4 * S, M2, S2, one, zero, 0, 0, 0, 0});
+    }
+    run_gemms(gj, s);
+  }
   {
     prof::KScope _ks("k_red_bragg", s);
-    const size_t shm = (size_t)(l + rB + rC + M2 + 2 * S) * sizeof(cplx);
-    // double-float products on double-float handles (the FP64 pipe's rate bounds this kernel)
-    const bool df = gemm_double_float();
-    const void* fn = df ? (const void*)k_red_bragg<true> : (const void*)k_red_bragg<false>;
-    HBS_CUDA(raise_smem_limit(fn, shm));
-    if (df)
-      k_red_bragg<true><<<(unsigned)ajobs.size(), 128, shm, s>>>(R, DD, dg.get(), da.get(), h.Zc.get(), Psel,
-                                                                 h.EZ.get(), EP.get(), Rp.get(), h.y0, cbuf.get(),
-                                                                 dbuf.get(), fbuf.get());
-    else
-      k_red_bragg<false><<<(unsigned)ajobs.size(), 128, shm, s>>>(R, DD, dg.get(), da.get(), h.Zc.get(), Psel,
-                                                                  h.EZ.get(), EP.get(), Rp.get(), h.y0, cbuf.get(),
-                                                                  dbuf.get(), fbuf.get());
+    const size_t shm = (size_t)S2 * sizeof(cplx);
+    HBS_CUDA(raise_smem_limit((const void*)k_red_bragg, shm));
+    k_red_bragg<<<(unsigned)na, 256, shm, s>>>(R, DD, dg.get(), da.get(), Eb.get(), XL.get(), XR.get(), EP.get(),
+                                               Rp.get(), h.y0, cbuf.get(), dbuf.get(), fbuf.get());
   }
   HBS_LAUNCH_CHECK("k_red_bragg");
   auto hcv = cbuf.download(s), hdv = dbuf.download(s);
