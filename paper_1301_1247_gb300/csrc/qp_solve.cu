@@ -41,7 +41,7 @@ static inline cplx to_c(zc v) { return cmk(v.real(), v.imag()); }
 // Periodizer precompute
 // ---------------------------------------------------------------------------
 
-static void contour_nodes(ContourData& c, int M, double h, double cc, double cw, double t0) {
+static void contour_nodes(ContourData& c, int M, double h, double cc, double cw, double t0, cudaStream_t s) {
   c.t0 = t0;
   c.k.resize(M);
   c.wk.resize(M);
@@ -54,8 +54,8 @@ static void contour_nodes(ContourData& c, int M, double h, double cc, double cw,
   }
   std::vector<cplx> kk(M), ww(M);
   for (int m = 0; m < M; ++m) { kk[m] = to_c(c.k[m]); ww[m] = to_c(c.wk[m]); }
-  c.dk.upload(kk, 0);
-  c.dwk.upload(ww, 0);
+  c.dk.upload(kk, s);
+  c.dwk.upload(ww, s);
 }
 
 // Pole-free crossing point for angles at or near a Wood's anomaly: half the smallest
@@ -208,7 +208,7 @@ void build_periodizer(Handle& h, cudaStream_t s, bool with_hbs) {
   const int nc = shift > 0 ? 2 : 1;
   h.contours.clear();
   h.contours.resize(nc);
-  for (int c = 0; c < nc; ++c) contour_nodes(h.contours[c], M, h.ch, h.cc, h.cw, c == 0 ? 0.0 : shift);
+  for (int c = 0; c < nc; ++c) contour_nodes(h.contours[c], M, h.ch, h.cc, h.cw, c == 0 ? 0.0 : shift, s);
 
   // ---- Bragg sampling rows (Remarks 2.2, 2.3)
   h.S = h.opts.n_bragg_samples > 0 ? h.opts.n_bragg_samples

@@ -49,3 +49,18 @@ def test_candidate_members_at_other_contour_steps(contour_h, precision):
     info = hbs.Handle(*_geometry(), 1.0, OMEGA, 1e-12,
                       hbs.default_options(precision=precision, contour_h=contour_h)).info()
     assert 0 < info["pid_residual"] < 1e-11
+
+
+def test_build_and_solve_on_a_stream_of_their_own():
+    """On a stream that does not order itself after the default stream, the same operations give the
+    default stream's amplitudes."""
+    import torch
+    hbs = require_lib()
+    geo, th = _geometry(600), np.linspace(-2.8, -0.4, 5)
+    want = hbs.Handle(*geo, 1.0, OMEGA, 1e-12).solve(th)
+    for _ in range(5):
+        stream = torch.cuda.Stream()
+        got = hbs.Handle(*geo, 1.0, OMEGA, 1e-12, stream=stream.cuda_stream).solve(th, stream=stream.cuda_stream)
+        for i in range(len(th)):
+            assert np.allclose(got.bragg(i)[1], want.bragg(i)[1], rtol=0, atol=1e-11)
+            assert np.allclose(got.bragg(i)[2], want.bragg(i)[2], rtol=0, atol=1e-11)
