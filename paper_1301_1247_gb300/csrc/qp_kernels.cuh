@@ -1,6 +1,8 @@
 // Declarations shared between the library's translation units.
 #pragma once
 
+#include <future>
+
 #include <vector>
 
 #include "common.cuh"
@@ -157,7 +159,10 @@ __global__ void k_diff_norm2(const cplx* a, int64_t lda, const cplx* b, int64_t 
 // and inversion (build_hbs) runs meanwhile on a second stream from a worker thread: the
 // neighbour and periodizer IDs and the selected rows depend on the geometry only, and the
 // two share the device until the transposed sweep, which needs both.
-void build_periodizer(Handle& h, cudaStream_t s, bool with_hbs = false);
+// with_hbs: runs the compression beside it on a thread of its own.  compressed: the compression runs
+// elsewhere and is waited for before V is formed.
+void build_periodizer(Handle& h, cudaStream_t s, bool with_hbs = false,
+                      const std::shared_future<void>* compressed = nullptr);
 void solve_angles(Handle& h, const double* theta, int64_t n_theta, bool plain, Result& out, cudaStream_t s);
 // The same angles with the proxy-point / wall-discrepancy periodizer (proxy.cu).
 void solve_angles_proxy(Handle& h, const double* theta, int64_t n_theta, Result& out, cudaStream_t s);

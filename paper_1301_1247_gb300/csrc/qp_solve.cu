@@ -153,7 +153,7 @@ struct BackgroundScope {
 };
 }  // namespace
 
-void build_periodizer(Handle& h, cudaStream_t s, bool with_hbs) {
+void build_periodizer(Handle& h, cudaStream_t s, bool with_hbs, const std::shared_future<void>* compressed) {
   HbsWorker hbs_worker;
   if (with_hbs) hbs_worker.start(h);
   BackgroundScope background(with_hbs);
@@ -611,6 +611,9 @@ void build_periodizer(Handle& h, cudaStream_t s, bool with_hbs) {
     ph.next("build:wait_hbs");
     hbs_worker.join();  // the compressed inverse is complete
     background.end();
+  } else if (compressed) {
+    ph.next("build:wait_hbs");
+    compressed->get();
   }
   ph.next("build:V_apply");
   h.VT.alloc((size_t)N * h.rsel);
