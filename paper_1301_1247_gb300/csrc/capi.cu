@@ -32,9 +32,9 @@ bool& gemm_tensor() {
   return tc;
 }
 
-bool& background_chain() {
-  static thread_local bool bg = false;
-  return bg;
+QrShare& qr_share() {
+  static thread_local QrShare share = kQrAlone;
+  return share;
 }
 
 std::mutex& coop_mutex() {
@@ -343,7 +343,7 @@ class BatchPeriodizers {
         HBS_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
         gemm_double_float() = df;
         gemm_tensor() = tc;
-        background_chain() = true;  // one CTA of a persistent QR an SM
+        qr_share() = kQrShared;
         StreamScope scope(s);
         for (size_t j; !failed_.load() && (j = next_.fetch_add(1)) < hs_.size();) {
           build_periodizer(*hs_[j], s, false, &compressed_);

@@ -133,10 +133,14 @@ bool& gemm_double_float();
 std::mutex& coop_mutex();
 // Large products on the tensor cores (digit-plane splitting) on this thread.
 bool& gemm_tensor();
-// True on the thread that builds the periodizer while another thread runs the compression
-// chain (the build's critical path) on a higher-priority stream: this thread's persistent
-// QRs take one CTA per SM instead of two and leave half of every SM to the compression.
-bool& background_chain();
+// How much of the device this thread's persistent QRs leave to other chains.  kQrAlone: two CTAs an SM.
+// kQrShared (beside a short compression, and a batch's periodizers, whose QRs exclude one another): one
+// CTA an SM, which leaves half of every SM.  kQrBeside (beside a compression that is the longer chain): one
+// CTA on every other SM, so that the compression's kernels that need a whole SM's registers or shared
+// memory (the tensor-core products, the clusters' eliminations and QRs) find free ones instead of
+// waiting for the QR to end.
+enum QrShare { kQrAlone, kQrShared, kQrBeside };
+QrShare& qr_share();
 
 // Sets the thread's arithmetic modes from an HBS_PRECISION_* value for a call's duration.
 struct GemmModeScope {

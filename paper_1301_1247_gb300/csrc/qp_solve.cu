@@ -144,19 +144,26 @@ struct HbsWorker {
 }  // namespace
 
 namespace {
-// Marks this thread as the background chain while the compression runs beside it.
-struct BackgroundScope {
-  bool prev;
-  explicit BackgroundScope(bool on) : prev(background_chain()) { background_chain() = on || prev; }
-  void end() { background_chain() = prev; }
-  ~BackgroundScope() { end(); }
+// Keeps this thread's QRs to their share of the device while the compression runs beside it: every other SM
+// from 6000 unknowns on, where the compression is the longer chain.  Build and solve, one CTA an SM
+// against every other SM (double-float with tensor cores): star of 800 nodes 10.6 / 11.3 ms, 2000 13.1 / 14.8,
+// 4000 16.6 / 17.4, 6000 17.1 / 17.1, 8000 19.5 / 18.7, 12 000 24.2 / 22.4; wiggly of 6000 21.0 / 19.5, 20 000
+// 33.2 / 31.0, FP64 56.2 / 54.3 and 121.6 / 119.9.  Two fifths of the SMs were slower again.
+constexpr int64_t kQrBesideUnknowns = 6000;
+struct QrShareScope {
+  QrShare prev;
+  QrShareScope(bool beside, int64_t unknowns) : prev(qr_share()) {
+    if (beside) qr_share() = unknowns >= kQrBesideUnknowns ? kQrBeside : kQrShared;
+  }
+  void end() { qr_share() = prev; }
+  ~QrShareScope() { end(); }
 };
 }  // namespace
 
 void build_periodizer(Handle& h, cudaStream_t s, bool with_hbs, const std::shared_future<void>* compressed) {
   HbsWorker hbs_worker;
   if (with_hbs) hbs_worker.start(h);
-  BackgroundScope background(with_hbs);
+  QrShareScope share(with_hbs, h.N);
   const int64_t N = h.N;
   const DevGeom g = Handle_geom(h);
   const double d = h.d, omega = h.omega;
@@ -610,7 +617,7 @@ void build_periodizer(Handle& h, cudaStream_t s, bool with_hbs, const std::share
   if (with_hbs) {
     ph.next("build:wait_hbs");
     hbs_worker.join();  // the compressed inverse is complete
-    background.end();
+    share.end();
   } else if (compressed) {
     ph.next("build:wait_hbs");
     compressed->get();
