@@ -57,14 +57,15 @@ typedef struct hbs_geometry {
 /* Dense products (the telescoping applies, the level products E, F*, G and the
  * periodizer projections) in double-float arithmetic: each FP64 operand is split into
  * two floats and multiplied and accumulated error-free on the FP32 pipes (about 48
- * significant bits, relative error near 1e-14 per product).  Kernel evaluations, the
- * interpolative decompositions, the inversions and the Schur solves stay in FP64. */
+ * significant bits, relative error near 1e-14 per product).  The updates of the interpolative
+ * decompositions, the inversions, the Hankel polynomials and the Schur solves (with one step of
+ * refinement against the FP64 system) run in the same arithmetic. */
 #define HBS_PRECISION_DOUBLE_FLOAT 1
-/* As HBS_PRECISION_DOUBLE_FLOAT, and the large dense products (inner dimension >= 4096,
- * at least 64 rows) run on the tcgen05 tensor cores: every FP64 row of op(A) and column
+/* As HBS_PRECISION_DOUBLE_FLOAT, and the larger dense products (inner dimension >= 96 and at least 48
+ * rows; in large batches >= 32 and at least 96 rows) run on the tcgen05 tensor cores: every FP64 row of op(A) and column
  * of B is scaled by a power of two and cut into seven 7-bit integer digits held exactly
- * in bf16; the digit products are accumulated exactly in FP32 tensor memory over 64
- * values of k and recombined in double-float arithmetic (relative error about 2^-46 of
+ * in bf16; the digit products are accumulated exactly, in FP32 tensor memory over 224
+ * values of k and as 64-bit integers beyond, and rounded once (relative error about 2^-46 of
  * max|a_ik| max|b_kj| per product term). */
 #define HBS_PRECISION_TENSOR 2
 
@@ -316,8 +317,8 @@ hbs_status hbs_row_id(void* mt, int64_t m, int64_t n, double tol, int* rank, int
  * Batched in-place inverse of `count` complex128 blocks of size n x n (column-major,
  * back to back in device memory `a`), the per-node inversion step of Sec. 4 (D_tau^{-1}
  * in Eqs. def_muhD..def_muG): Gauss-Jordan elimination with partial pivoting, all
- * blocks in the same launches (one launch per panel of columns, on clusters of CTAs, for up to
- * 128 blocks; one CTA per block otherwise).  precision as for hbs_zgemm: _DOUBLE_FLOAT and _TENSOR run the
+ * blocks in the same launches (small blocks in the shared memory of one CTA each; others one launch
+ * per panel of columns, on clusters of CTAs).  precision as for hbs_zgemm: _DOUBLE_FLOAT and _TENSOR run the
  * eliminations in double-float arithmetic.  1 <= n <= 4096, 1 <= count <= 2^20, else
  * HBS_ERR_INVALID_ARG.  Returns HBS_WARN_ILLCOND when a pivot is exactly zero (the
  * blocks' contents are then undefined).  Synchronizes the stream.

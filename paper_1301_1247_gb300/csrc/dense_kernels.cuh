@@ -5,6 +5,7 @@
 
 #include "common.cuh"
 #include "dfloat.cuh"
+#include "elem.cuh"
 
 namespace hbs {
 
@@ -273,6 +274,87 @@ __global__ void __launch_bounds__(NT) k_gj_inverse(const InvJob* jobs, int* flag
       }
     }
     __syncthreads();
+  }
+  if (tid == 0) flag_out[jb.job] = bad;
+}
+
+// The same for n <= kSmallInverse, the block in shared memory throughout and nothing interchanged: step c
+// exchanges column c with its pivot row p among the rows not taken yet,
+//   M(i, j) <- [i != p, j != c] M(i, j) - W(i) P(j),
+//   W(i) = M(i, c) / d, W(p) = -1 / d,   P(j) = M(p, j), P(c) = 1,
+// and Inv(c, p_t) = M(p_c, t) at the end (as gjx.cu).  W and P are copies, so a step costs two barriers; every
+// warp finds the pivot for itself.  The multiply-adds bound it (FP32 pipes in double-float, FP64
+// pipe in FP64), with several blocks an SM to cover the barriers.  2048 blocks of 49 in
+// double-float: 0.77 ms, and 1.25 with the kernel above, which streams the block from L1 and L2 at every step.
+constexpr int kSmallInverse = 96;
+inline size_t small_inverse_smem(int n) { return (size_t)n * (n + 2) * sizeof(cplx) + (size_t)n * sizeof(int); }
+
+template <typename T>
+__global__ void __launch_bounds__(128) k_gj_small(const InvJob* jobs, int* flag_out) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  const InvJob jb = jobs[blockIdx.x];
+  const int n = jb.n, tid = threadIdx.x, lane = tid & 31;
+  cplx* A = jb.a;
+  T* M = reinterpret_cast<T*>(sm_raw);
+  T* W = M + n * n;
+  T* P = W + n;
+  int* perm = reinterpret_cast<int*>(P + n);
+  for (int e = tid; e < n * n; e += 128) M[e] = x_in(A[e], (const T*)nullptr);
+  const int i0 = tid % n, j0 = tid / n, di = 128 % n, dj = 128 / n;
+  unsigned used = 0;  // rows lane, lane + 32, lane + 64
+  bool bad = false;
+  __syncthreads();
+  for (int c = 0; c < n; ++c) {
+    unsigned best = 0;
+    int bi = 0x7fffffff;
+#pragma unroll
+    for (int q = 0; q < (kSmallInverse + 31) / 32; ++q) {
+      const int i = lane + 32 * q;
+      if (i < n && !(used >> q & 1u)) {
+        const unsigned k = x_key(M[c * n + i]);
+        if (k > best) { best = k; bi = i; }
+      }
+    }
+    const unsigned top = __reduce_max_sync(0xffffffffu, best);
+    const int p = __reduce_min_sync(0xffffffffu, best == top ? bi : 0x7fffffff);
+    const T d = M[c * n + p];
+    if (!x_nonzero(d)) {  // the same in every thread
+      bad = true;
+      break;
+    }
+    if ((p & 31) == lane) used |= 1u << (p >> 5);
+    const T ip = x_recip(d);
+    if (tid < n) {
+      W[tid] = tid == p ? x_neg(ip) : x_mul(M[c * n + tid], ip);
+      P[tid] = tid == c ? x_in(cmk(1.0, 0.0), (const T*)nullptr) : M[tid * n + p];
+    }
+    if (tid == 0) perm[c] = p;
+    __syncthreads();
+    int i = i0, j = j0;
+    for (int e = tid; e < n * n; e += 128) {
+      T x = (i == p || j == c) ? x_zero<T>() : M[e];
+      x_submul(W[i], P[j], x);
+      M[e] = x;
+      i += di;
+      j += dj;
+      if (i >= n) {
+        i -= n;
+        ++j;
+      }
+    }
+    __syncthreads();
+  }
+  if (!bad) {
+    int i = i0, j = j0;
+    for (int e = tid; e < n * n; e += 128) {
+      A[perm[j] * n + i] = x_out(M[j * n + perm[i]]);
+      i += di;
+      j += dj;
+      if (i >= n) {
+        i -= n;
+        ++j;
+      }
+    }
   }
   if (tid == 0) flag_out[jb.job] = bad;
 }

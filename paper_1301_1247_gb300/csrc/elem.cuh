@@ -50,6 +50,15 @@ __device__ __forceinline__ cplx x_shfl(const cplx& v, int l) {
 }
 __device__ __forceinline__ dfc x_shfl(const dfc& v, int l) { return dfc_shfl(v, l); }
 
+// Pivot keys: |v|^2 to float precision (double-float), or the sign, exponent and upper
+// significand bits of |v|^2 (FP64), as unsigned integers that order alike; 1 is an exact zero and 0
+// no candidate.
+__device__ __forceinline__ unsigned x_key(const cplx& v) { return (unsigned)__double2hiint(cabs2(v)) + 1u; }
+__device__ __forceinline__ unsigned x_key(const dfc& v) { return __float_as_uint(fmaf(v.rh, v.rh, v.ih * v.ih)) + 1u; }
+__device__ __forceinline__ double x_key_value(unsigned k, const cplx*) { return __hiloint2double((int)(k - 1u), 0); }
+__device__ __forceinline__ double x_key_value(unsigned k, const dfc*) { return (double)__uint_as_float(k - 1u); }
+__device__ __forceinline__ bool x_nonzero(const cplx& v) { return cabs2(v) > 0.0; }
+__device__ __forceinline__ bool x_nonzero(const dfc& v) { return fmaf(v.rh, v.rh, v.ih * v.ih) > 0.f; }
 
 // r = 1 / sqrt(x) for a normal x > 0: two Newton steps r <- r + r (1 - x r^2) / 2 from the FP32 value, on x
 // scaled by a power of four (as x_recip, instead of FP64's long square-root and division chains).

@@ -53,14 +53,6 @@ constexpr int kW = kT / 32;
 constexpr int kTile = 64;  // rows of a strip's tile
 constexpr int kS = 16;     // columns of a strip
 
-// Pivot keys: |v|^2 to float precision (double-float), or the sign, exponent and upper
-// significand bits of |v|^2 (FP64), as unsigned integers that order alike; 1 is an exact zero and 0
-// no candidate.
-__device__ __forceinline__ unsigned x_key(const cplx& v) { return (unsigned)__double2hiint(cabs2(v)) + 1u; }
-__device__ __forceinline__ unsigned x_key(const dfc& v) { return __float_as_uint(fmaf(v.rh, v.rh, v.ih * v.ih)) + 1u; }
-__device__ __forceinline__ double x_key_value(unsigned k, const cplx*) { return __hiloint2double((int)(k - 1u), 0); }
-__device__ __forceinline__ double x_key_value(unsigned k, const dfc*) { return (double)__uint_as_float(k - 1u); }
-
 __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool ok) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
   const int bytes = ok ? 16 : 0;  // 0: the destination is zero-filled and nothing is read

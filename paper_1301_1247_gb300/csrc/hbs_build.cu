@@ -595,18 +595,23 @@ static std::vector<int> node_ids(std::vector<CpqrJob>& jobs, double tol, cudaStr
 void batched_inverse(std::vector<InvJob>& jobs_in, cudaStream_t s, const char* what) {
   std::vector<InvJob> jobs;
   std::vector<std::pair<cplx*, int>> big;
-  // The cluster elimination takes batches of at most 512 blocks, and blocks of more than 72 of larger
-  // ones; small blocks in large numbers stay with one CTA per block (49 x 2048: 1.25 ms there, 1.49 on
-  // clusters; 56 x 512: 0.58 and 0.46; 88 x 512: 1.93 and 1.37; 107 x 256: 2.8 and 1.0).  It works on a
-  // copy, which batches past 128 blocks may not always have the memory for: at most 4 GB there.
+  // Blocks of at most 56 go to the kernel that holds one in shared memory; so do blocks of at most 72 in
+  // batches of more than 512; the cluster elimination takes the others.  Double-float, shared memory against
+  // clusters: 33 x 64 0.086 / 0.120 ms, 49 x 128 0.148 / 0.178, 49 x 512 0.265 / 0.425, 64 x 300 0.311 / 0.311,
+  // 64 x 64 0.260 / 0.178 (one kernel that streamed the block from L2: 49 x 2048 1.25 ms, now 0.77).  The
+  // clusters work on a copy, which batches past 128 blocks may not always have the memory for: at most
+  // 4 GB there.
   int64_t copy = 0;
   size_t nbig = 0;
+  int nmax = 0;
+  for (const auto& j : jobs_in) nmax = std::max(nmax, j.n);
+  const bool few = jobs_in.size() <= 512 && nmax > 56;
   for (const auto& j : jobs_in)
-    if (big_inverse(j.n) || jobs_in.size() <= 512) {
+    if (big_inverse(j.n) || few) {
       copy += 16 * (int64_t)j.n * j.n;
       ++nbig;
     }
-  const bool all_big = jobs_in.size() <= 512 && (jobs_in.size() <= 128 || copy <= (4ll << 30));
+  const bool all_big = few && (jobs_in.size() <= 128 || copy <= (4ll << 30));
   const bool use_big = all_big || (nbig <= 4096 && copy <= (4ll << 30));
   for (auto& j : jobs_in) {
     if (use_big && (all_big || big_inverse(j.n)) && gjx_fits(j.n)) big.push_back({j.a, j.n});
@@ -614,21 +619,44 @@ void batched_inverse(std::vector<InvJob>& jobs_in, cudaStream_t s, const char* w
   }
   if (!big.empty()) gjx_invert(big, s, what);
   if (jobs.empty()) return;
-  for (size_t i = 0; i < jobs.size(); ++i) jobs[i].job = (int)i;
+  std::stable_partition(jobs.begin(), jobs.end(), [](const InvJob& j) { return j.n <= kSmallInverse; });
+  size_t nsmall = 0;
+  int smax = 0;
+  double fl[2] = {0.0, 0.0};
   int64_t piv = 0;
-  for (auto& j : jobs) piv += j.n;
+  for (size_t i = 0; i < jobs.size(); ++i) {
+    InvJob& j = jobs[i];
+    const bool small = j.n <= kSmallInverse;
+    j.job = (int)i;
+    fl[small ? 0 : 1] += 8.0 * (double)j.n * j.n * j.n;
+    if (small) {
+      ++nsmall;
+      smax = std::max(smax, j.n);
+    } else {
+      piv += j.n;
+    }
+  }
   DevBuf<int> dpiv(std::max<int64_t>(piv, 1));
   piv = 0;
-  for (auto& j : jobs) { j.piv = dpiv.get() + piv; piv += j.n; }
+  for (size_t i = nsmall; i < jobs.size(); ++i) {
+    jobs[i].piv = dpiv.get() + piv;
+    piv += jobs[i].n;
+  }
   DevBuf<InvJob> dj = upload_jobs(jobs, s);
   DevBuf<int> flags(jobs.size());
-  double fl = 0.0;
-  for (auto& j : jobs) fl += 8.0 * (double)j.n * j.n * j.n;
-  {
-    prof::KScope _ks("k_gj_inverse", s, fl, 0.0);
-    // double-float eliminations on handles built with double-float precision
-    if (gemm_double_float()) k_gj_inverse<256, true><<<(unsigned)jobs.size(), 256, 0, s>>>(dj.get(), flags.get());
-    else k_gj_inverse<256, false><<<(unsigned)jobs.size(), 256, 0, s>>>(dj.get(), flags.get());
+  const bool df = gemm_double_float();  // double-float eliminations on handles built with double-float precision
+  if (nsmall > 0) {
+    prof::KScope _ks("k_gj_small", s, fl[0], 0.0);
+    const size_t sm = small_inverse_smem(smax);
+    HBS_CUDA(raise_smem_limit(df ? (const void*)k_gj_small<dfc> : (const void*)k_gj_small<cplx>, sm));
+    if (df) k_gj_small<dfc><<<(unsigned)nsmall, 128, sm, s>>>(dj.get(), flags.get());
+    else k_gj_small<cplx><<<(unsigned)nsmall, 128, sm, s>>>(dj.get(), flags.get());
+  }
+  HBS_LAUNCH_CHECK("k_gj_small");
+  if (const unsigned nb = (unsigned)(jobs.size() - nsmall)) {
+    prof::KScope _ks("k_gj_inverse", s, fl[1], 0.0);
+    if (df) k_gj_inverse<256, true><<<nb, 256, 0, s>>>(dj.get() + nsmall, flags.get());
+    else k_gj_inverse<256, false><<<nb, 256, 0, s>>>(dj.get() + nsmall, flags.get());
   }
   HBS_LAUNCH_CHECK("k_gj_inverse");
   auto f = flags.download(s);

@@ -1,7 +1,7 @@
 // Launch-shape autotuner for the batched kernels.
 //
 // A tuned call site names its kernel family and shape class (a key such as
-// "bgj/n512/b4") and the number of launch variants it can run.  With tuning on
+// "inverse/n512/j4/df") and the number of launch variants it can run.  With tuning on
 // (HBS_AUTOTUNE=1 in the environment), the first calls for a key run each variant once,
 // timed with CUDA events on the launching stream, and later calls run the fastest.  The
 // measured choices are read from and written to the file named by HBS_TUNE_FILE (one

@@ -47,3 +47,23 @@ def test_compressed_inverse_with_unusual_leaves(leaf, precision):
     h.apply_inverse(b, x, 3)
     torch.cuda.synchronize()
     assert float(torch.linalg.norm(x @ at - b) / torch.linalg.norm(b)) < 1e-10
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 63, 64, 65, 72])
+def test_many_small_inverses(n, precision):
+    """Enough blocks for the kernel that holds a block in shared memory, at the edges of its warps and of its
+    largest size in use; bounds as above.  A block of exact zeros is reported."""
+    hbs = require_lib()
+    rng = np.random.default_rng(100 + n)
+    count = 520
+    a = rng.standard_normal((count, n, n)) + 1j * rng.standard_normal((count, n, n))
+    a += 4 * np.sqrt(n) * np.eye(n)[None]
+    a = a[:, rng.permutation(n), :]  # no pivot on the diagonal
+    buf = dev(np.ascontiguousarray(np.transpose(a, (0, 2, 1))).ravel())
+    assert hbs.batched_inverse(buf, n, count, precision) == hbs.HBS_OK
+    got = np.transpose(buf.cpu().numpy().reshape(count, n, n), (0, 2, 1))
+    assert relerr(got, np.linalg.inv(a)) < (1e-13 if precision == 0 else 1e-12)
+    a[count // 2] = 0.0
+    buf = dev(np.ascontiguousarray(np.transpose(a, (0, 2, 1))).ravel())
+    assert hbs.batched_inverse(buf, n, count, precision) == hbs.HBS_WARN_ILLCOND
