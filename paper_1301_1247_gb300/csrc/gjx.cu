@@ -366,7 +366,7 @@ __device__ __forceinline__ void gjx_strip(const GjxMat& mt, int u, int j0, int j
           if (cb) xb[r] = v[q][1];
         }
     }
-    __syncthreads();  // the buffer just read is staged again in the next round
+    __syncthreads();  // the buffer just read is staged again for the next tile
     buf ^= 1;
   }
 }
