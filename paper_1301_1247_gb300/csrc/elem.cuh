@@ -50,12 +50,21 @@ __device__ __forceinline__ cplx x_shfl(const cplx& v, int l) {
 }
 __device__ __forceinline__ dfc x_shfl(const dfc& v, int l) { return dfc_shfl(v, l); }
 
-// Pivot keys: |v|^2 to float precision (double-float), or the sign, exponent and upper
-// significand bits of |v|^2 (FP64), as unsigned integers that order alike; 1 is an exact zero and 0
-// no candidate.
-__device__ __forceinline__ unsigned x_key(const cplx& v) { return (unsigned)__double2hiint(cabs2(v)) + 1u; }
-__device__ __forceinline__ unsigned x_key(const dfc& v) { return __float_as_uint(fmaf(v.rh, v.rh, v.ih * v.ih)) + 1u; }
-__device__ __forceinline__ double x_key_value(unsigned k, const cplx*) { return __hiloint2double((int)(k - 1u), 0); }
+// Pivot keys: |v|^2 to float precision (double-float), or the exponent and upper significand bits of |v|^2
+// (FP64), as unsigned integers that order alike; 1 is an exact zero and 0 no candidate.  A square
+// carries no sign, so a sign bit belongs to a NaN and is dropped: a key made from it could wrap to 0, and a column
+// whose candidates all have key 0 has no pivot row.  A NaN's key is above every number's.
+__device__ __forceinline__ unsigned x_key(const cplx& v) {
+  const double m = cabs2(v);
+  const unsigned hi = (unsigned)__double2hiint(m) & 0x7FFFFFFFu;
+  return hi + ((hi | (unsigned)__double2loint(m)) ? 2u : 1u);
+}
+__device__ __forceinline__ unsigned x_key(const dfc& v) {
+  return (__float_as_uint(fmaf(v.rh, v.rh, v.ih * v.ih)) & 0x7FFFFFFFu) + 1u;
+}
+__device__ __forceinline__ double x_key_value(unsigned k, const cplx*) {
+  return k < 2u ? 0.0 : __hiloint2double((int)(k - 2u), k == 2u ? 1 : 0);  // below 2^-1042: some positive value
+}
 __device__ __forceinline__ double x_key_value(unsigned k, const dfc*) { return (double)__uint_as_float(k - 1u); }
 __device__ __forceinline__ bool x_nonzero(const cplx& v) { return cabs2(v) > 0.0; }
 __device__ __forceinline__ bool x_nonzero(const dfc& v) { return fmaf(v.rh, v.rh, v.ih * v.ih) > 0.f; }
