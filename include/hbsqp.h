@@ -320,8 +320,9 @@ hbs_status hbs_row_id(void* mt, int64_t m, int64_t n, double tol, int* rank, int
  * blocks in the same launches (small blocks in the shared memory of one CTA each; others one launch
  * per panel of columns, on clusters of CTAs).  precision as for hbs_zgemm: _DOUBLE_FLOAT and _TENSOR run the
  * eliminations in double-float arithmetic.  1 <= n <= 4096, 1 <= count <= 2^20, else
- * HBS_ERR_INVALID_ARG.  Returns HBS_WARN_ILLCOND when a pivot is exactly zero (the
- * blocks' contents are then undefined).  Synchronizes the stream.
+ * HBS_ERR_INVALID_ARG.  Returns HBS_WARN_ILLCOND when a pivot is exactly zero, a NaN or an infinity, or
+ * past the arithmetic's range (double-float: a modulus below about 1e-19 or above 1e19), and the
+ * blocks' contents are then undefined.  Synchronizes the stream.
  */
 hbs_status hbs_batched_inverse(void* a, int64_t n, int64_t count, int precision, void* stream);
 

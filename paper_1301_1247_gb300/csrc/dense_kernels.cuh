@@ -318,12 +318,12 @@ __global__ void __launch_bounds__(128) k_gj_small(const InvJob* jobs, int* flag_
     const unsigned top = __reduce_max_sync(0xffffffffu, best);
     const int p = __reduce_min_sync(0xffffffffu, best == top ? bi : 0x7fffffff);
     const T d = M[c * n + p];
-    if (!x_nonzero(d)) {  // the same in every thread
+    const T ip = x_recip(d);
+    if (top <= 1u || !x_usable(ip)) {  // the same in every thread
       bad = true;
       break;
     }
     if ((p & 31) == lane) used |= 1u << (p >> 5);
-    const T ip = x_recip(d);
     if (tid < n) {
       W[tid] = tid == p ? x_neg(ip) : x_mul(M[c * n + tid], ip);
       P[tid] = tid == c ? x_in(cmk(1.0, 0.0), (const T*)nullptr) : M[tid * n + p];

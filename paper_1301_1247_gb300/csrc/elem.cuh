@@ -66,8 +66,17 @@ __device__ __forceinline__ double x_key_value(unsigned k, const cplx*) {
   return k < 2u ? 0.0 : __hiloint2double((int)(k - 2u), k == 2u ? 1 : 0);  // below 2^-1042: some positive value
 }
 __device__ __forceinline__ double x_key_value(unsigned k, const dfc*) { return (double)__uint_as_float(k - 1u); }
-__device__ __forceinline__ bool x_nonzero(const cplx& v) { return cabs2(v) > 0.0; }
-__device__ __forceinline__ bool x_nonzero(const dfc& v) { return fmaf(v.rh, v.rh, v.ih * v.ih) > 0.f; }
+// Whether x_recip found a reciprocal: of a zero, a NaN, an infinity or a value out of the arithmetic's range it
+// gives a zero or something not finite, and a block with such a pivot has no inverse.  Integer compares: this
+// is beside the serial chain of every pivot.
+__device__ __forceinline__ bool x_usable(const cplx& r) {
+  const unsigned x = (unsigned)__double2hiint(r.x) & 0x7FFFFFFFu, y = (unsigned)__double2hiint(r.y) & 0x7FFFFFFFu;
+  return max(x, y) < 0x7FF00000u && (x | y | (unsigned)__double2loint(r.x) | (unsigned)__double2loint(r.y)) != 0u;
+}
+__device__ __forceinline__ bool x_usable(const dfc& r) {
+  const unsigned x = __float_as_uint(r.rh) & 0x7FFFFFFFu, y = __float_as_uint(r.ih) & 0x7FFFFFFFu;
+  return max(x, y) < 0x7F800000u && (x | y) != 0u;
+}
 
 // r = 1 / sqrt(x) for a normal x > 0: two Newton steps r <- r + r (1 - x r^2) / 2 from the FP32 value, on x
 // scaled by a power of four (as x_recip, instead of FP64's long square-root and division chains).

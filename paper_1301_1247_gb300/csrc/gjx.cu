@@ -237,7 +237,7 @@ __device__ __forceinline__ void gjx_panel(const GjxMat& mt, int t, int CS, int r
     if (rank == 0 && tid == 0) {
       mt.piv[c0 + s] = p;
       mt.pmag[c0 + s] = x_key_value(win->key, (const T*)nullptr);
-      if (win->key <= 1u) *mt.singular = 1;
+      if (win->key <= 1u || !x_usable(ip)) *mt.singular = 1;
     }
     const bool own = h == ho;
 #pragma unroll
@@ -437,7 +437,7 @@ __global__ void k_gjx_inverse_out(const GjxMat* mats) {
   }
 }
 
-// The solution x(c) = B(p_c) and the conditioning flag (smallest against largest pivot).
+// The solution x(c) = B(p_c) and the conditioning flag (smallest against largest pivot, or one without a reciprocal).
 template <typename T>
 __global__ void __launch_bounds__(kT) k_gjx_solution_out(const GjxMat* mats, cplx* const* out, int* illcond) {
   __shared__ double smn[kW], smx[kW];
@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(kT) k_gjx_solution_out(const GjxMat* mats, cpl
       mn = fmin(mn, smn[w]);
       mx = fmax(mx, smx[w]);
     }
-    illcond[blockIdx.x] = mn <= 1e-28 * mx ? 1 : 0;
+    illcond[blockIdx.x] = (mn <= 1e-28 * mx || *mt.singular) ? 1 : 0;
   }
 }
 
