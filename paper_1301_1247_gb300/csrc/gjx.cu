@@ -471,42 +471,94 @@ __global__ void __launch_bounds__(kT) k_gjx_solution_out(const GjxMat* mats, cpl
   }
 }
 
-// x += the elimination applied to a residual: one CTA per matrix and right-hand side
-// (CTA m qmax + j), the vector in shared memory, one panel after another (two barriers and
-// one 16-term product per row and panel).
-template <typename T, int B>
-__global__ void __launch_bounds__(kT) k_gjx_apply(const GjxMat* mats, int qmax, const cplx* const* res, cplx* const* out) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* r = reinterpret_cast<T*>(smem_raw);  // n
-  __shared__ T xs[B];
-  const int m = (int)blockIdx.x / qmax, j = (int)blockIdx.x % qmax;
-  const GjxMat mt = mats[m];
-  if (j >= mt.q) return;
-  const int n = mt.n;
-  const cplx* rr = res[m] + (int64_t)j * n;
-  for (int i = threadIdx.x; i < n; i += kT) r[i] = x_in(rr[i], (const T*)nullptr);
-  for (int c0 = 0; c0 < n; c0 += B) {
-    const int nk = min(B, n - c0);
-    __syncthreads();
-    if (threadIdx.x < nk) xs[threadIdx.x] = r[mt.piv[c0 + threadIdx.x]];
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += kT) {
-      const int ci = mt.colof[i];
-      const T* w = reinterpret_cast<const T*>(mt.A) + (int64_t)c0 * n + i;
-      T wv[B];
-#pragma unroll
-      for (int kk = 0; kk < B; ++kk) wv[kk] = kk < nk ? w[(int64_t)kk * n] : x_zero<T>();
-      T v = (ci >= c0 && ci < c0 + nk) ? x_zero<T>() : r[i];
-#pragma unroll
-      for (int kk = 0; kk < B; ++kk) {
-        if (kk < nk) x_mac(wv[kk], xs[kk], v);
-        if ((kk & 3) == 3) x_norm(v);
-      }
-      r[i] = v;
-    }
+// The eliminated matrices' double-float pairs as FP64, in place (the same 16 bytes), for k_gjx_apply.
+__global__ void __launch_bounds__(kT) k_gjx_widen(const GjxMat* mats) {
+  const GjxMat mt = mats[blockIdx.y];
+  const int64_t na = (int64_t)mt.n * mt.n;
+  const dfc* d = reinterpret_cast<const dfc*>(mt.A);
+  cplx* a = reinterpret_cast<cplx*>(mt.A);
+  for (int64_t e = blockIdx.x * (int64_t)kT + threadIdx.x; e < na; e += (int64_t)gridDim.x * kT) {
+    const dfc v = d[e];
+    a[e] = from_dfc_bits(v);
   }
-  cplx* x = out[m] + (int64_t)j * n;
-  for (int i = threadIdx.x; i < n; i += kT) x[mt.colof[i]] = cadd(x[mt.colof[i]], x_out(r[i]));
+}
+
+// x += the elimination applied to a residual, in FP64: one cluster of CS CTAs per matrix and QB right-hand sides,
+// the rows dealt to its CTAs in chunks, the vectors in their shared memory (two copies, so that a panel costs
+// one cluster barrier: a panel reads its pivot rows' values from one copy and writes the other).  Two
+// threads a row, real and imaginary part: the FP64 multiply-adds bound it (n^2 of 4 for a right-hand side), and a
+// warp instruction keeps its quarter of an SM for 64 cycles.  The first rows' W are on their way
+// before the barrier.  One right-hand side of one system of 394: 0.077 ms; ten for each of 100 systems
+// 1.45 ms (0.98 at the FP64 pipes' rate), and 0.76 in double-float, which would round the correction to 48 bits.
+template <int B, int QB>
+__global__ void __launch_bounds__(kT) k_gjx_apply(const GjxMat* mats, int CS, int qblocks, const cplx* const* res,
+                                                  cplx* const* out) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double xs[B][QB][2];
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)blockIdx.x % CS, item = (int)blockIdx.x / CS;
+  const int m = item / qblocks, j0 = item % qblocks * QB;
+  const GjxMat mt = mats[m];
+  if (j0 >= mt.q) return;  // the whole cluster
+  const int n = mt.n, tid = threadIdx.x, chunk = (n + CS - 1) / CS;
+  const int r0 = rank * chunk, rows = max(0, min(chunk, n - r0));
+  double* r = reinterpret_cast<double*>(smem_raw);  // [2][chunk][QB][2]
+  const int half = chunk * QB * 2;
+  const cplx* A = reinterpret_cast<const cplx*>(mt.A);
+  for (int e = tid; e < rows * QB; e += kT) {
+    const int i = e / QB, j = j0 + e % QB;
+    const cplx v = j < mt.q ? res[m][(int64_t)j * n + r0 + i] : cmk(0.0, 0.0);
+    r[2 * e] = v.x;
+    r[2 * e + 1] = v.y;
+  }
+  int p = tid < B * QB && tid / QB < n ? mt.piv[tid / QB] : 0;
+  int buf = 0;
+  for (int c0 = 0; c0 < n; c0 += B, buf ^= 1) {
+    const int nk = min(B, n - c0);
+    cplx w[B];
+    int ci = -1;
+    auto load = [&](int e) {
+      const cplx* wg = A + (int64_t)c0 * n + r0 + (e >> 1);
+#pragma unroll
+      for (int k = 0; k < B; ++k) w[k] = k < nk ? wg[(int64_t)k * n] : cmk(0.0, 0.0);
+      ci = mt.colof[r0 + (e >> 1)];
+    };
+    if (tid < 2 * rows) load(tid);
+    cl.sync();  // the previous panel's values are there, and its readers of the other copy are done
+    if (tid < nk * QB) {
+      const double* src = cl.map_shared_rank(r + buf * half, p / chunk) + (p % chunk) * QB * 2 + tid % QB * 2;
+      xs[tid / QB][tid % QB][0] = src[0];
+      xs[tid / QB][tid % QB][1] = src[1];
+    }
+    if (tid < B * QB && c0 + B + tid / QB < n) p = mt.piv[c0 + B + tid / QB];
+    __syncthreads();
+    for (int e = tid; e < 2 * rows; e += kT) {
+      if (e != tid) load(e);
+      const int part = e & 1, flip = part ? 0 : (int)0x80000000;
+      const bool isp = ci >= c0 && ci < c0 + nk;
+      const int o = buf * half + (e >> 1) * QB * 2 + part;
+      double v[QB];
+#pragma unroll
+      for (int q = 0; q < QB; ++q) v[q] = isp ? 0.0 : r[o + 2 * q];
+#pragma unroll
+      for (int k = 0; k < B; ++k) {
+        if (k >= nk) break;
+        const double wy = __hiloint2double(__double2hiint(w[k].y) ^ flip, __double2loint(w[k].y));  // off the FP64 pipe
+#pragma unroll
+        for (int q = 0; q < QB; ++q) v[q] = fma(w[k].x, xs[k][q][part], fma(wy, xs[k][q][1 - part], v[q]));
+      }
+#pragma unroll
+      for (int q = 0; q < QB; ++q) r[o + (buf ? -half : half) + 2 * q] = v[q];
+    }
+    __syncthreads();  // xs
+  }
+  cl.sync();  // nobody reads another CTA's memory any more
+  for (int e = tid; e < rows * QB; e += kT) {
+    const int i = e / QB, j = j0 + e % QB;
+    if (j >= mt.q) continue;
+    cplx* x = out[m] + (int64_t)j * n + mt.colof[r0 + i];
+    *x = cadd(*x, cmk(r[buf * half + 2 * e], r[buf * half + 2 * e + 1]));
+  }
 }
 
 template <typename T, int B, int TPR, int RPT>
@@ -665,13 +717,47 @@ void gjx_solution(Gjx& g, cplx* const* out, int* illcond, cudaStream_t s) {
   HBS_LAUNCH_CHECK("k_gjx_solution_out");
 }
 
+template <int QB>
+static void launch_apply(const Gjx& g, int qblocks, const cplx* const* res, cplx* const* out, cudaStream_t s) {
+  // eight CTAs a system until there are eight for every SM, then fewer, whose warps have fewer idle lanes
+  int CS = 8;
+  const auto smem = [&](int c) { return (size_t)2 * QB * sizeof(cplx) * ((g.nmax + c - 1) / c); };
+  while (CS > 1 && (int64_t)g.nm * qblocks * CS > 1216 && smem(CS / 2) <= 48 * 1024) CS /= 2;
+  const auto fn = k_gjx_apply<PanelWidth<dfc>::value, QB>;
+  HBS_CUDA(raise_smem_limit((const void*)fn, smem(CS)));
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(g.nm * qblocks * CS));
+  cfg.blockDim = dim3(kT);
+  cfg.dynamicSmemBytes = smem(CS);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)CS;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  HBS_CUDA(cudaLaunchKernelEx(&cfg, fn, (const GjxMat*)g.mats.get(), CS, qblocks, res, out));
+}
+
 void gjx_apply(Gjx& g, const cplx* const* res, cplx* const* out, cudaStream_t s) {
-  const size_t sm = (size_t)g.nmax * sizeof(cplx);
-  const void* fn = g.df ? (const void*)k_gjx_apply<dfc, PanelWidth<dfc>::value> : (const void*)k_gjx_apply<cplx, PanelWidth<cplx>::value>;
-  HBS_CUDA(raise_smem_limit(fn, sm + 4096));
+  if (!g.df || g.qmax < 1) throw Error(HBS_ERR_INTERNAL, "elimination: nothing to refine");
+  {
+    prof::KScope _ks("k_gjx_widen", s);
+    const int bx = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)g.nmax * g.nmax + 1023) / 1024, 1216 / g.nm + 1));
+    k_gjx_widen<<<dim3(bx, g.nm), kT, 0, s>>>(g.mats.get());
+  }
+  HBS_LAUNCH_CHECK("k_gjx_widen");
   prof::KScope _ks("k_gjx_apply", s);
-  if (g.df) k_gjx_apply<dfc, PanelWidth<dfc>::value><<<g.nm * g.qmax, kT, sm, s>>>(g.mats.get(), g.qmax, res, out);
-  else k_gjx_apply<cplx, PanelWidth<cplx>::value><<<g.nm * g.qmax, kT, sm, s>>>(g.mats.get(), g.qmax, res, out);
+  // right-hand sides in even blocks of at most five, one at a time where the vectors of five are too long
+  const int qblocks = g.nmax > 8 * 1200 ? g.qmax : (g.qmax + 4) / 5;
+  switch ((g.qmax + qblocks - 1) / qblocks) {
+    case 1: launch_apply<1>(g, qblocks, res, out, s); break;
+    case 2: launch_apply<2>(g, qblocks, res, out, s); break;
+    case 3: launch_apply<3>(g, qblocks, res, out, s); break;
+    case 4: launch_apply<4>(g, qblocks, res, out, s); break;
+    default: launch_apply<5>(g, qblocks, res, out, s); break;
+  }
   HBS_LAUNCH_CHECK("k_gjx_apply");
 }
 

@@ -52,7 +52,8 @@ int gjx_tuned_cluster(const std::string& tkey, int nm, int nmax, bool df);
 void gjx_eliminate(Gjx& g, const std::vector<GjxSys>& sys, bool df, bool invert, int cs, cudaStream_t s);
 // After a solve: out[m] (n x q) = the solutions, illcond[m] = 1 if a pivot is 1e-14 of the largest, zero or not finite.
 void gjx_solution(Gjx& g, cplx* const* out, int* illcond, cudaStream_t s);
-// out[m] += the elimination applied to res[m] (n x q each).
+// After a double-float solve: out[m] += the elimination applied to res[m] (n x q each) in FP64 arithmetic.  Once:
+// the eliminated matrices are FP64 afterwards.
 void gjx_apply(Gjx& g, const cplx* const* res, cplx* const* out, cudaStream_t s);
 // In-place inverses; throws HBS_WARN_ILLCOND on a block that is singular or not finite.
 void gjx_invert(const std::vector<std::pair<cplx*, int>>& mats, cudaStream_t s, const char* what);
