@@ -284,6 +284,128 @@ __device__ __forceinline__ void gjx_panel(const GjxMat& mt, int t, int CS, int r
   }
 }
 
+// Panel t of a matrix with more rows than eight CTAs hold in registers (4096): every thread walks its rows r0 + tid,
+// + kT, ..., and the panel stays where it is, in L2, read and written once a column.  The exchanges are those
+// of gjx_panel, the columns in place.  The panel's passes bound it (rows x B x 32 bytes a column over eight SMs), so
+// the serial chain weighs more than below 4096; the strips' updates run beside it on all other SMs as there.
+// One FP64 system of 4400: 355 ms; an LU on one CTA, at its 8.3 GFLOP/s, would take 27 s.
+template <typename T, int B>
+__device__ __forceinline__ void gjx_panel_rows(const GjxMat& mt, int t, int CS, int rank, PanelSmem<T, B>& sm) {
+  const int n = mt.n, c0 = t * B, nb = min(B, n - c0);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int chunk = x_chunk(n, CS);
+  const int r0 = rank * chunk, r1 = min(n, r0 + chunk);
+  T* P = reinterpret_cast<T*>(mt.A) + (int64_t)c0 * n;
+  cg::cluster_group cl = cg::this_cluster();
+  if (t > 0) {
+    const int cp = c0 - B;
+    if (tid < B) sm.pprev[tid] = mt.piv[cp + tid];
+    if (tid < B * B) {
+      const int kk = tid / B, j = tid % B;
+      sm.X[kk][j] = j < nb ? P[(int64_t)j * n + mt.piv[cp + kk]] : x_zero<T>();
+    }
+  }
+  cl.sync();  // every CTA has started and has read the previous pivot rows
+  unsigned key = 0;  // this thread's best candidate for the next column
+  int krow = -1;
+  for (int i = r0 + tid; i < r1; i += kT) {
+    T a[B];
+#pragma unroll
+    for (int c = 0; c < B; ++c) a[c] = c < nb ? P[(int64_t)c * n + i] : x_zero<T>();
+    if (t > 0) {
+      bool isp = false;
+#pragma unroll
+      for (int kk = 0; kk < B; ++kk) isp |= sm.pprev[kk] == i;
+      if (isp) {
+#pragma unroll
+        for (int c = 0; c < B; ++c) a[c] = x_zero<T>();
+      }
+      const T* wr = P - (int64_t)B * n + i;
+#pragma unroll 1
+      for (int k = 0; k < B; ++k) {
+        const T w = wr[(int64_t)k * n];
+#pragma unroll
+        for (int c = 0; c < B; ++c) {
+          x_mac(w, sm.X[k][c], a[c]);
+          x_norm(a[c]);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < B; ++c)
+        if (c < nb) P[(int64_t)c * n + i] = a[c];
+    }
+    const unsigned k = mt.colof[i] < 0 ? x_key(a[0]) : 0u;
+    if (k > key) { key = k; krow = i; }
+  }
+#pragma unroll 1
+  for (int s = 0; s < nb; ++s) {
+    const unsigned wmax = __reduce_max_sync(0xffffffffu, key);
+    const int wl = __ffs(__ballot_sync(0xffffffffu, key == wmax)) - 1;
+    if (lane == 0) sm.wkey[warp] = wmax;
+    __syncthreads();
+    const unsigned wk = lane < kW ? sm.wkey[lane] : 0u;
+    const unsigned cmax = __reduce_max_sync(0xffffffffu, wk);
+    const int ww = __ffs(__ballot_sync(0xffffffffu, lane < kW && wk == cmax)) - 1;
+    const int par = s & 1;
+    if (warp == ww) {
+      if (lane == wl) {
+        sm.mine.key = cmax;
+        sm.mine.prow = krow;
+        if (cmax > 0) {  // a CTA past the last row has no candidate
+#pragma unroll
+          for (int c = 0; c < B; ++c) sm.mine.row[c] = c < nb ? P[(int64_t)c * n + krow] : x_zero<T>();
+          sm.mine.ip = x_recip(P[(int64_t)s * n + krow]);
+        }
+      }
+      constexpr int kItems = (int)(sizeof(Cand<T, B>) / 16);
+      __syncwarp();
+      for (int e = lane; e < kItems * CS; e += 32) {
+        const int dst = e / kItems, item = e % kItems;
+        Cand<T, B>* rem = cl.map_shared_rank(&sm.cand[par][rank], dst);
+        reinterpret_cast<float4*>(rem)[item] = reinterpret_cast<const float4*>(&sm.mine)[item];
+      }
+    }
+    cl.sync();
+    const unsigned ck = lane < CS ? sm.cand[par][lane & 7].key : 0u;
+    const unsigned gmax = __reduce_max_sync(0xffffffffu, ck);
+    const Cand<T, B>* win = &sm.cand[par][__ffs(__ballot_sync(0xffffffffu, lane < CS && ck == gmax)) - 1];
+    const T ip = win->ip;
+    const int p = win->prow;
+    if (rank == 0 && tid == 0) {
+      mt.piv[c0 + s] = p;
+      mt.pmag[c0 + s] = x_key_value(win->key, (const T*)nullptr);
+      if (win->key <= 1u || !x_usable(ip)) *mt.singular = 1;
+    }
+    key = 0;
+    krow = -1;
+    for (int i = r0 + tid; i < r1; i += kT) {
+      T a[B];
+#pragma unroll
+      for (int c = 0; c < B; ++c) a[c] = c < nb ? P[(int64_t)c * n + i] : x_zero<T>();
+      const bool isp = i == p;
+      T as = x_zero<T>();
+#pragma unroll
+      for (int c = 0; c < B; ++c)
+        if (c == s) as = a[c];
+      const T l = isp ? ip : x_neg(x_mul(as, ip));
+      T next = x_zero<T>();
+#pragma unroll
+      for (int c = 0; c < B; ++c) {
+        if (c >= nb) break;
+        T v = isp ? x_zero<T>() : a[c];
+        x_mac(l, win->row[c], v);
+        x_norm(v);
+        if (c == s) v = l;
+        if (c == s + 1) next = v;
+        P[(int64_t)c * n + i] = v;
+      }
+      if (isp) mt.colof[p] = c0 + s;
+      const unsigned k = !isp && mt.colof[i] < 0 ? x_key(next) : 0u;
+      if (k > key) { key = k; krow = i; }
+    }
+  }
+}
+
 // Update u on the strip of columns [j0, j0 + 16) that are columns [jlo, jhi) of the system, but for
 // those of the panels u and t (skip; a solve's jlo lies past them), the rows of CTA `rank` of the
 // cluster.  Every CTA has read the old pivot rows before any of them is written.
@@ -388,7 +510,9 @@ __global__ void __launch_bounds__(kT, RPT == 1 ? 2 : 1) k_gjx(const GjxMat* mats
   const int cl = (int)blockIdx.x / CS, rank = (int)blockIdx.x % CS;
   if (cl < nm) {
     const GjxMat mt = mats[cl];
-    if (t * B < mt.n) gjx_panel<T, B, TPR, RPT>(mt, t, CS, rank, sm.p);
+    if (t * B >= mt.n) return;
+    if constexpr (RPT > 0) gjx_panel<T, B, TPR, RPT>(mt, t, CS, rank, sm.p);
+    else gjx_panel_rows<T, B>(mt, t, CS, rank, sm.p);
     return;
   }
   const GjxMat mt = mats[(cl - nm) / strips];
@@ -597,12 +721,11 @@ void launch_any(const GjxMat* dm, int nm, int nmax, int qmax, int CS, bool inver
   if (4 * chunk <= kT) launch_steps<T, B, 4, 1>(dm, nm, nmax, qmax, CS, invert, s);
   else if (2 * chunk <= kT) launch_steps<T, B, 2, 1>(dm, nm, nmax, qmax, CS, invert, s);
   else if (chunk <= kT) launch_steps<T, B, 1, 1>(dm, nm, nmax, qmax, CS, invert, s);
-  else launch_steps<T, B, 1, 2>(dm, nm, nmax, qmax, CS, invert, s);
+  else if (chunk <= 2 * kT) launch_steps<T, B, 1, 2>(dm, nm, nmax, qmax, CS, invert, s);
+  else launch_steps<T, B, 1, 0>(dm, nm, nmax, qmax, CS, invert, s);  // CS is 8 then (gjx_cluster)
 }
 
 }  // namespace
-
-bool gjx_fits(int n) { return n <= kT * 8 * 2; }
 
 // Default cluster size.  The fewest CTAs that hold a panel's rows one per thread (measured: 250 x 128
 // blocks 4.3 ms on one CTA, 4.7 on two; 430 x 8 1.9 ms on two, 2.1 on eight; 850 x 8 12.0 ms on
@@ -617,7 +740,7 @@ int gjx_cluster(int nm, int nmax, bool df) {
   return cs;
 }
 
-bool gjx_cluster_fits(int cs, int nmax) { return nmax <= kT * cs * (cs == 8 ? 2 : 1); }
+bool gjx_cluster_fits(int cs, int nmax) { return cs == 8 || nmax <= kT * cs; }
 
 void gjx_eliminate(Gjx& g, const std::vector<GjxSys>& sys, bool df, bool invert, int CS, cudaStream_t s) {
   const int nm = (int)sys.size();

@@ -40,7 +40,6 @@ struct Gjx {
   DevBuf<double> pmag;
 };
 
-bool gjx_fits(int n);
 // Whether clusters of cs CTAs hold panels of nmax rows, the default cluster size, and the tuned one.
 bool gjx_cluster_fits(int cs, int nmax);
 int gjx_cluster(int nm, int nmax, bool df);

@@ -614,7 +614,7 @@ void batched_inverse(std::vector<InvJob>& jobs_in, cudaStream_t s, const char* w
   const bool all_big = few && (jobs_in.size() <= 128 || copy <= (4ll << 30));
   const bool use_big = all_big || (nbig <= 4096 && copy <= (4ll << 30));
   for (auto& j : jobs_in) {
-    if (use_big && (all_big || big_inverse(j.n)) && gjx_fits(j.n)) big.push_back({j.a, j.n});
+    if (use_big && (all_big || big_inverse(j.n))) big.push_back({j.a, j.n});
     else jobs.push_back(j);
   }
   if (!big.empty()) gjx_invert(big, s, what);

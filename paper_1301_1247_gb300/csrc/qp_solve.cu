@@ -943,165 +943,11 @@ __global__ void k_assemble(Dims D, const GroupJob* groups, const cplx* proj, dou
   }
 }
 
-// Batched dense solve S U = Rhs (Gaussian elimination with partial pivoting on the
-// augmented matrix), one CTA per group.  illcond[g] = 1 if a pivot fell below
-// 1e-14 times the largest pivot.
-template <int NT>
-__global__ void __launch_bounds__(NT) k_schur_solve(Dims D, const GroupJob* groups, cplx* Spool, cplx* Rpool,
-                                                    int* illcond) {
-  // Right-looking LU with partial pivoting of the augmented system [S | R] (one CTA per
-  // Bloch group), blocked by panels of NB columns: the panel is factored column by
-  // column, U12 = L11^{-1} A12 follows by forward substitution (one thread per column),
-  // and the trailing matrix gets one rank-NB update from shared-memory tiles of L21 and
-  // U12 with 4 x 4 register tiles per thread.
-  constexpr int NB = 16, TM = 64;
-  static_assert(NT == 256, "16 x 16 threads per trailing tile");
-  __shared__ long long redv[32];
-  __shared__ int redi[32];
-  __shared__ cplx sh_ip;
-  __shared__ cplx Ls[NB][TM + 1];
-  __shared__ cplx Us[NB][TM + 1];
-  __shared__ cplx L11[NB][NB + 1];
-  const GroupJob G = groups[blockIdx.x];
-  const int n = G.nsys, q = G.q, nc = n + q;
-  cplx* A = Spool + G.s_off;
-  cplx* B = Rpool + G.r_off;
-  auto col = [&](int j) -> cplx* { return j < n ? A + (int64_t)j * n : B + (int64_t)(j - n) * n; };
-  const int tid = threadIdx.x;
-  double pmax = 0.0, pmin = 1e300;
-  for (int k0 = 0; k0 < n; k0 += NB) {
-    const int nb = min(NB, n - k0);
-    for (int c = k0; c < k0 + nb; ++c) {
-      cplx* ac = A + (int64_t)c * n;
-      long long best = kNoKey;
-      int bi = 0x7fffffff;
-      for (int i = c + tid; i < n; i += NT) {
-        const long long v = nkey(cabs2(ac[i]));
-        if (better(v, i, best, bi)) { best = v; bi = i; }
-      }
-      long long kv;
-      int p;
-      block_argmax_key<NT>(best, bi, redv, redi, &kv, &p);
-      if (tid == 0) {  // pivot range for the conditioning flag (read by thread 0)
-        const double pv = __longlong_as_double(kv);
-        pmax = fmax(pmax, pv);
-        pmin = fmin(pmin, pv);
-      }
-      if (p != c) {
-        for (int j = tid; j < nc; j += NT) {
-          cplx* cj = col(j);
-          const cplx t = cj[c];
-          cj[c] = cj[p];
-          cj[p] = t;
-        }
-      }
-      __syncthreads();
-      if (tid == 0) {
-        const cplx dv = ac[c];
-        sh_ip = cabs2(dv) > 0.0 ? cdiv(cmk(1, 0), dv) : cmk(0, 0);
-      }
-      __syncthreads();
-      const cplx ip = sh_ip;
-      for (int i = c + 1 + tid; i < n; i += NT) ac[i] = cmul(ac[i], ip);
-      __syncthreads();
-      for (int j = c + 1; j < k0 + nb; ++j) {
-        cplx* aj = A + (int64_t)j * n;
-        const cplx ucj = aj[c];
-        for (int i = c + 1 + tid; i < n; i += NT) aj[i] = cfms(ac[i], ucj, aj[i]);
-      }
-      __syncthreads();
-    }
-    const int j0 = k0 + nb;
-    if (j0 >= nc) break;
-    for (int e = tid; e < NB * NB; e += NT) {
-      const int r = e % NB, cc = e / NB;
-      L11[r][cc] = (r < nb && cc < nb) ? A[(int64_t)(k0 + cc) * n + k0 + r] : cmk(0, 0);
-    }
-    __syncthreads();
-    for (int j = j0 + tid; j < nc; j += NT) {
-      cplx* aj = col(j) + k0;
-      cplx u[NB];
-#pragma unroll
-      for (int r = 0; r < NB; ++r) u[r] = r < nb ? aj[r] : cmk(0, 0);
-#pragma unroll
-      for (int cc = 0; cc < NB; ++cc)
-#pragma unroll
-        for (int r = cc + 1; r < NB; ++r) u[r] = cfms(L11[r][cc], u[cc], u[r]);
-#pragma unroll
-      for (int r = 0; r < NB; ++r)
-        if (r < nb) aj[r] = u[r];
-    }
-    __syncthreads();
-    const int rows = n - j0, cols = nc - j0;
-    const int tr = tid & 15, tc = tid >> 4;
-    for (int rt = 0; rt < rows; rt += TM) {
-      for (int ct = 0; ct < cols; ct += TM) {
-        for (int e = tid; e < TM * NB; e += NT) {
-          const int r = e % TM, kk = e / TM;
-          const int i = j0 + rt + r;
-          Ls[kk][r] = (i < n && kk < nb) ? A[(int64_t)(k0 + kk) * n + i] : cmk(0, 0);
-        }
-        for (int e = tid; e < TM * NB; e += NT) {
-          const int kk = e % NB, c = e / NB;
-          const int j = j0 + ct + c;
-          Us[kk][c] = (j < nc && kk < nb) ? col(j)[k0 + kk] : cmk(0, 0);
-        }
-        __syncthreads();
-        cplx acc[4][4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) acc[a][b] = cmk(0, 0);
-        for (int kk = 0; kk < nb; ++kk) {
-          cplx la[4], ub[4];
-#pragma unroll
-          for (int a = 0; a < 4; ++a) la[a] = Ls[kk][tr + 16 * a];
-#pragma unroll
-          for (int b = 0; b < 4; ++b) ub[b] = Us[kk][tc + 16 * b];
-#pragma unroll
-          for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] = cfma(la[a], ub[b], acc[a][b]);
-        }
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const int j = j0 + ct + tc + 16 * b;
-          if (j >= nc) continue;
-          cplx* cj = col(j);
-#pragma unroll
-          for (int a = 0; a < 4; ++a) {
-            const int i = j0 + rt + tr + 16 * a;
-            if (i < n) cj[i] = csub(cj[i], acc[a][b]);
-          }
-        }
-        __syncthreads();
-      }
-    }
-  }
-  // back substitution, one RHS per warp
-  const int lane = tid & 31, warp = tid >> 5;
-  for (int j = warp; j < q; j += NT / 32) {
-    cplx* b = B + (int64_t)j * n;
-    for (int i = n - 1; i >= 0; --i) {
-      cplx acc = cmk(0, 0);
-      for (int t = i + 1 + lane; t < n; t += 32) acc = cfma(A[(int64_t)t * n + i], b[t], acc);
-      for (int o = 16; o > 0; o >>= 1) {
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-      }
-      if (lane == 0) b[i] = cdiv(csub(b[i], acc), A[(int64_t)i * n + i]);
-      __syncwarp();
-    }
-  }
-  if (tid == 0) illcond[blockIdx.x] = (pmin <= 1e-28 * pmax) ? 1 : 0;
-}
-
 // Factor and solve every group's Schur system by blocked Gauss-Jordan elimination (gjx.cu).  In
 // the thread's double-float mode it runs in double-float and the solution is refined once
 // against the FP64 system (residual by an FP64 product, correction with the same elimination).
-// Systems larger than the elimination's panels hold take the one-CTA LU above.
-static void schur_solve(const Dims& D, const std::vector<GroupJob>& gjobs, const GroupJob* dg, cplx* Sp, cplx* Rp,
-                        int* ill, cudaStream_t s) {
+// ill[g] = 1 if a pivot fell below 1e-14 times the largest.
+static void schur_solve(const std::vector<GroupJob>& gjobs, cplx* Sp, cplx* Rp, int* ill, cudaStream_t s) {
   const int ng = (int)gjobs.size();
   const bool df = gemm_double_float();
   int nmax = 0;
@@ -1109,10 +955,6 @@ static void schur_solve(const Dims& D, const std::vector<GroupJob>& gjobs, const
   for (const auto& G : gjobs) {
     nmax = std::max(nmax, G.nsys);
     rend = std::max<int64_t>(rend, G.r_off + (int64_t)G.nsys * G.q);
-  }
-  if (!gjx_fits(nmax)) {
-    k_schur_solve<256><<<ng, 256, 0, s>>>(D, dg, Sp, Rp, ill);
-    return;
   }
   std::vector<GjxSys> sys;
   for (const auto& G : gjobs) sys.push_back({Sp + G.s_off, Rp + G.r_off, G.nsys, G.q});
@@ -1713,7 +1555,7 @@ static void reduced_batch(Handle& h, std::vector<GroupJob>& gjobs, std::vector<s
       sfl += 8.0 / 3.0 * n * n * n + 8.0 * n * n * G.q;
     }
     prof::KScope _ks("k_schur_solve", s, sfl, 0.0);
-    schur_solve(DD, gjobs, dg.get(), Sp.get(), Rp.get(), ill.get(), s);
+    schur_solve(gjobs, Sp.get(), Rp.get(), ill.get(), s);
   }
   HBS_LAUNCH_CHECK("k_schur_solve");
   ph.next("solve:bragg");
@@ -2127,7 +1969,7 @@ void solve_angles(Handle& h, const double* theta, int64_t n_theta, bool plain, R
     }
     {
       prof::KScope _ks("k_schur_solve", s, sfl, 0.0);
-      schur_solve(D, gjobs, dg.get(), Sp.get(), Rp.get(), ill.get(), s);
+      schur_solve(gjobs, Sp.get(), Rp.get(), ill.get(), s);
     }
     HBS_LAUNCH_CHECK("k_schur_solve");
     // ---- Bragg amplitudes
