@@ -317,7 +317,7 @@ hbs_status hbs_row_id(void* mt, int64_t m, int64_t n, double tol, int* rank, int
  * Batched in-place inverse of `count` complex128 blocks of size n x n (column-major,
  * back to back in device memory `a`), the per-node inversion step of Sec. 4 (D_tau^{-1}
  * in Eqs. def_muhD..def_muG): Gauss-Jordan elimination with partial pivoting, all
- * blocks in the same launches (small blocks in the shared memory of one CTA each; others one launch
+ * blocks of a piece in the same launches (small blocks in the shared memory of one CTA each; others one launch
  * per panel of columns, on clusters of CTAs).  precision as for hbs_zgemm: _DOUBLE_FLOAT and _TENSOR run the
  * eliminations in double-float arithmetic.  1 <= n <= 4096, 1 <= count <= 2^20, else
  * HBS_ERR_INVALID_ARG.  Returns HBS_WARN_ILLCOND when a pivot is exactly zero, a NaN or an infinity, or

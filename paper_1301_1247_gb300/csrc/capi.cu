@@ -694,7 +694,7 @@ hbs_status hbs_batched_inverse(void* a, int64_t n, int64_t count, int precision,
   GemmModeScope mode(precision);
   return guarded([&] {
     std::vector<InvJob> jobs((size_t)count);
-    for (int64_t i = 0; i < count; ++i) jobs[i] = {static_cast<cplx*>(a) + i * n * n, nullptr, (int)n, (int)i};
+    for (int64_t i = 0; i < count; ++i) jobs[i] = {static_cast<cplx*>(a) + i * n * n, (int)n, (int)i};
     batched_inverse(jobs, s, "hbs_batched_inverse");
     HBS_CUDA(cudaStreamSynchronize(s));
   });

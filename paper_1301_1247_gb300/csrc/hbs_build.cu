@@ -539,8 +539,6 @@ DevGeom Handle_geom(const Handle& h) {
   return g;
 }
 
-static bool big_inverse(int n) { return n > 72; }
-
 // Largest root (sum of the level-2 skeletons) for which level 1 is left uncompressed.  At the
 // top of the tree the level-1 ID and inversions are latency-bound work on two nodes; without
 // them the root inverts the level-2 skeletons' coupled system directly (the same system,
@@ -592,73 +590,72 @@ static std::vector<int> node_ids(std::vector<CpqrJob>& jobs, double tol, cudaStr
 }
 
 // Batched in-place inverses; throws on a singular block.
-void batched_inverse(std::vector<InvJob>& jobs_in, cudaStream_t s, const char* what) {
-  std::vector<InvJob> jobs;
-  std::vector<std::pair<cplx*, int>> big;
-  // Blocks of at most 56 go to the kernel that holds one in shared memory; so do blocks of at most 72 in
-  // batches of more than 512; the cluster elimination takes the others.  Double-float, shared memory against
-  // clusters: 33 x 64 0.086 / 0.120 ms, 49 x 128 0.148 / 0.178, 49 x 512 0.265 / 0.425, 64 x 300 0.311 / 0.311,
-  // 64 x 64 0.260 / 0.178 (one kernel that streamed the block from L2: 49 x 2048 1.25 ms, now 0.77).  The
-  // clusters work on a copy, which batches past 128 blocks may not always have the memory for: at most
-  // 4 GB there.
-  int64_t copy = 0;
-  size_t nbig = 0;
+//
+// Blocks of at most 56 go to the kernel that holds one in shared memory; so do blocks of at most 72 in batches
+// of more than 512, and of at most 96 in batches of more than 4096 blocks past 72; the cluster elimination takes
+// the others.  Shared memory against clusters, double-float: 33 x 64 0.086 / 0.120 ms, 49 x 128 0.148 / 0.178,
+// 49 x 512 0.265 / 0.425, 64 x 300 0.311 / 0.311, 64 x 64 0.260 / 0.178, 80 x 4097 7.0 / 8.4 (one kernel that
+// streamed the block from L2: 49 x 2048 1.25 ms, now 0.77).  The clusters work on copies, so their blocks go in
+// even pieces of at most 1 GB of copies, still enough to fill the chip, and at most 4096 blocks: 300 x 1000 in
+// 620 ms and 4200 x 100 in 14.8, where one CTA a block took 3137 and 23.5.
+constexpr int64_t kInversePiece = 1ll << 30;
+constexpr size_t kInversePieceBlocks = 4096;
+void batched_inverse(std::vector<InvJob>& jobs, cudaStream_t s, const char* what) {
   int nmax = 0;
-  for (const auto& j : jobs_in) nmax = std::max(nmax, j.n);
-  const bool few = jobs_in.size() <= 512 && nmax > 56;
-  for (const auto& j : jobs_in)
-    if (big_inverse(j.n) || few) {
-      copy += 16 * (int64_t)j.n * j.n;
-      ++nbig;
-    }
-  const bool all_big = few && (jobs_in.size() <= 128 || copy <= (4ll << 30));
-  const bool use_big = all_big || (nbig <= 4096 && copy <= (4ll << 30));
-  for (auto& j : jobs_in) {
-    if (use_big && (all_big || big_inverse(j.n))) big.push_back({j.a, j.n});
-    else jobs.push_back(j);
+  size_t past72 = 0;
+  for (const auto& j : jobs) {
+    nmax = std::max(nmax, j.n);
+    past72 += j.n > 72 ? 1 : 0;
   }
-  if (!big.empty()) gjx_invert(big, s, what);
-  if (jobs.empty()) return;
-  std::stable_partition(jobs.begin(), jobs.end(), [](const InvJob& j) { return j.n <= kSmallInverse; });
-  size_t nsmall = 0;
-  int smax = 0;
-  double fl[2] = {0.0, 0.0};
-  int64_t piv = 0;
-  for (size_t i = 0; i < jobs.size(); ++i) {
-    InvJob& j = jobs[i];
-    const bool small = j.n <= kSmallInverse;
-    j.job = (int)i;
-    fl[small ? 0 : 1] += 8.0 * (double)j.n * j.n * j.n;
-    if (small) {
-      ++nsmall;
-      smax = std::max(smax, j.n);
+  const int in_smem = jobs.size() <= 512 && nmax > 56 ? 0 : past72 > kInversePieceBlocks ? kSmallInverse : 72;
+  std::vector<InvJob> small;
+  std::vector<std::pair<cplx*, int>> all, piece;
+  const auto bytes = [](int n) { return (int64_t)n * n * (int64_t)sizeof(cplx); };
+  int64_t total = 0;
+  for (const auto& j : jobs) {
+    if (j.n <= in_smem) {
+      small.push_back(j);
     } else {
-      piv += j.n;
+      all.push_back({j.a, j.n});
+      total += bytes(j.n);
     }
   }
-  DevBuf<int> dpiv(std::max<int64_t>(piv, 1));
-  piv = 0;
-  for (size_t i = nsmall; i < jobs.size(); ++i) {
-    jobs[i].piv = dpiv.get() + piv;
-    piv += jobs[i].n;
+  const double pieces = (double)std::max<int64_t>((total + kInversePiece - 1) / kInversePiece,
+                                                  (int64_t)((all.size() + kInversePieceBlocks - 1) / kInversePieceBlocks));
+  int64_t copy = 0;
+  const auto flush = [&] {
+    if (!piece.empty()) gjx_invert(piece, s, what);
+    piece.clear();
+    copy = 0;
+  };
+  for (const auto& m : all) {
+    const int64_t b = bytes(m.second);
+    if (copy + b > kInversePiece || piece.size() == kInversePieceBlocks ||
+        (double)copy >= (double)total / pieces)
+      flush();
+    piece.push_back(m);
+    copy += b;
   }
-  DevBuf<InvJob> dj = upload_jobs(jobs, s);
-  DevBuf<int> flags(jobs.size());
+  flush();
+  if (small.empty()) return;
+  int smax = 0;
+  double fl = 0.0;
+  for (size_t i = 0; i < small.size(); ++i) {
+    small[i].job = (int)i;
+    smax = std::max(smax, small[i].n);
+    fl += 8.0 * (double)small[i].n * small[i].n * small[i].n;
+  }
+  DevBuf<InvJob> dj = upload_jobs(small, s);
+  DevBuf<int> flags(small.size());
   const bool df = gemm_double_float();  // double-float eliminations on handles built with double-float precision
-  if (nsmall > 0) {
-    prof::KScope _ks("k_gj_small", s, fl[0], 0.0);
+  {
+    prof::KScope _ks("k_gj_small", s, fl, 0.0);
     const size_t sm = small_inverse_smem(smax);
     HBS_CUDA(raise_smem_limit(df ? (const void*)k_gj_small<dfc> : (const void*)k_gj_small<cplx>, sm));
-    if (df) k_gj_small<dfc><<<(unsigned)nsmall, 128, sm, s>>>(dj.get(), flags.get());
-    else k_gj_small<cplx><<<(unsigned)nsmall, 128, sm, s>>>(dj.get(), flags.get());
+    if (df) k_gj_small<dfc><<<(unsigned)small.size(), 128, sm, s>>>(dj.get(), flags.get());
+    else k_gj_small<cplx><<<(unsigned)small.size(), 128, sm, s>>>(dj.get(), flags.get());
   }
   HBS_LAUNCH_CHECK("k_gj_small");
-  if (const unsigned nb = (unsigned)(jobs.size() - nsmall)) {
-    prof::KScope _ks("k_gj_inverse", s, fl[1], 0.0);
-    if (df) k_gj_inverse<256, true><<<nb, 256, 0, s>>>(dj.get() + nsmall, flags.get());
-    else k_gj_inverse<256, false><<<nb, 256, 0, s>>>(dj.get() + nsmall, flags.get());
-  }
-  HBS_LAUNCH_CHECK("k_gj_inverse");
   auto f = flags.download(s);
   for (int v : f)
     if (v) throw Error(HBS_WARN_ILLCOND, std::string("singular block in ") + what);
@@ -773,7 +770,7 @@ void build_hbs_multi(const std::vector<Handle*>& hs, cudaStream_t s) {
         h.Groot.alloc(std::max<int64_t>((int64_t)h.nroot * h.nroot, 1));
         dj.push_back({tk.g, lv.idx.get(), h.Groot.get(), h.nroot, ch.k[0], 0, ch.Dhat.get() + ch.dh_off[0],
                       ch.Dhat.get() + ch.dh_off[1]});
-        if (h.nroot > 0) ij.push_back({h.Groot.get(), nullptr, h.nroot, (int)ij.size()});
+        if (h.nroot > 0) ij.push_back({h.Groot.get(), h.nroot, (int)ij.size()});
         h.factor_bytes += 16.0 * h.nroot * h.nroot;
         h.apply_flops += 8.0 * h.nroot * h.nroot;
         lv.k.assign(1, 0);
@@ -1094,7 +1091,7 @@ void build_hbs_multi(const std::vector<Handle*>& hs, cudaStream_t s) {
             dj.push_back({tasks[i].g, lv.idx.get() + lv.off[j], d, lv.n[j], ch.k[2 * j], 0,
                           ch.Dhat.get() + ch.dh_off[2 * j], ch.Dhat.get() + ch.dh_off[2 * j + 1]});
           }
-          ij.push_back({d, nullptr, lv.n[j], (int)ij.size()});
+          ij.push_back({d, lv.n[j], (int)ij.size()});
         }
       }
       DevBuf<DJob> ddj = upload_jobs(dj, s);
@@ -1178,7 +1175,7 @@ void build_hbs_multi(const std::vector<Handle*>& hs, cudaStream_t s) {
       for (size_t i = 0; i < tasks.size(); ++i) {
         Level& lv = tasks[i].h->levels[tasks[i].l];
         for (int j = 0; j < lv.count; ++j)
-          if (lv.k[j] > 0) ij.push_back({S[i].get() + lv.dh_off[j], nullptr, lv.k[j], (int)ij.size()});
+          if (lv.k[j] > 0) ij.push_back({S[i].get() + lv.dh_off[j], lv.k[j], (int)ij.size()});
       }
       batched_inverse(ij, s, "skeleton block P^T D^-1 P");
     }
