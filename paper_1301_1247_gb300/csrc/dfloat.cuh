@@ -76,34 +76,6 @@ __device__ __forceinline__ dfc dfc_scale(float sh, float sl, const dfc& a) {
   return r;
 }
 
-// (h, l) = (ah, al) (bh, bl), and 1 / sqrt(a), 1 / a of a normal a > 0: the FP32 approximation y and
-// the first two terms of the series in its residual e (|e| < 2^-21), y (1 + e / 2 + 3 e^2 / 8) and
-// y (1 + e + e^2).  A dozen dependent FP32 operations; they sit on the serial chain of every pivot.
-__device__ __forceinline__ void df_mul(float ah, float al, float bh, float bl, float& h, float& l) {
-  const float p = __fmul_rn(ah, bh);
-  float e = fmaf(ah, bh, -p);
-  e = fmaf(ah, bl, e);
-  e = fmaf(al, bh, e);
-  h = __fadd_rn(p, e);
-  l = __fsub_rn(e, __fsub_rn(h, p));
-}
-__device__ __forceinline__ void df_rsqrt(float ah, float al, float& h, float& l) {
-  const float y = rsqrtf(ah);
-  const float p = __fmul_rn(y, y), pe = fmaf(y, y, -p);
-  const float e = __fsub_rn(fmaf(-ah, p, 1.0f), fmaf(ah, pe, __fmul_rn(al, p)));
-  const float c = __fmul_rn(y, fmaf(__fmul_rn(e, e), 0.375f, __fmul_rn(e, 0.5f)));
-  h = __fadd_rn(y, c);
-  l = __fsub_rn(c, __fsub_rn(h, y));
-}
-__device__ __forceinline__ void df_rcp(float ah, float al, float& h, float& l) {
-  float y;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(ah));
-  const float e = __fsub_rn(fmaf(-ah, y, 1.0f), __fmul_rn(al, y));
-  const float c = __fmul_rn(y, fmaf(e, e, e));
-  h = __fadd_rn(y, c);
-  l = __fsub_rn(c, __fsub_rn(h, y));
-}
-
 // 1 / d = conj(d) / |d|^2 (0 for d = 0)
 __device__ __forceinline__ dfc dfc_recip(const dfc& d) {
   float nh = 0.f, nl = 0.f;
@@ -111,7 +83,7 @@ __device__ __forceinline__ dfc dfc_recip(const dfc& d) {
   df_norm(nh, nl);
   if (!(nh > 0.f)) return {0.f, 0.f, 0.f, 0.f};
   float qh, ql;
-  df_rcp(nh, nl, qh, ql);
+  df_div(1.f, 0.f, nh, nl, qh, ql);
   const dfc c{d.rh, d.rl, -d.ih, -d.il};
   return dfc_scale(qh, ql, c);
 }
@@ -126,52 +98,53 @@ __device__ __forceinline__ dfc dfc_shfl(const dfc& a, int l) {
           __shfl_sync(0xffffffffu, a.il, l)};
 }
 
-// The Householder reflector of x = (x0, x_1, ...) in double-float arithmetic, ||x_1..||^2 = sig: beta =
-// -(x0/|x0|) ||x||, v0 = x0 - beta, tau = 2 / (|v0|^2 + sig) = 1 / (||x|| (||x|| + |x0|)).  One thread,
-// FP32 pipes only.
+// The Householder reflector of x = (x0, x_1, ...) in double-float arithmetic (the FP64
+// formulas of householder_scalars, with ||x_1..||^2 = sig): beta = -(x0/|x0|) ||x||,
+// v0 = x0 - beta, tau = 2 / (|v0|^2 + sig).  One thread, FP32 pipes only.
 __device__ __forceinline__ void df_householder(const dfc& x0, float sh, float sl, dfc* v0, dfc* beta, float* th,
                                                float* tl) {
   float a2h = 0.f, a2l = 0.f;
   df_abs2_acc(x0, a2h, a2l);
   df_norm(a2h, a2l);
+  // |x0| from x0 2^48 where the low part of its square would leave FP32's range
+  const float up = a2h < 1e-24f ? 281474976710656.0f : 1.0f, down = a2h < 1e-24f ? 3.552713678800501e-15f : 1.0f;
+  const dfc xs = {x0.rh * up, x0.rl * up, x0.ih * up, x0.il * up};
+  float ah = 0.f, al = 0.f, axh, axl;
+  df_abs2_acc(xs, ah, al);
+  df_norm(ah, al);
+  df_sqrt(ah, al, axh, axl);
+  axh *= down;
+  axl *= down;
   float t2h = a2h, t2l = a2l;
   df_add_to(sh, sl, t2h, t2l);
   df_norm(t2h, t2l);
-  if (!(t2h > 1e-36f)) {  // nothing left of the column
-    *v0 = *beta = {0.f, 0.f, 0.f, 0.f};
-    *th = *tl = 0.f;
-    return;
+  float xnh, xnl;
+  df_sqrt(t2h, t2l, xnh, xnl);
+  dfc v, b;
+  if (axh > 0.f) {
+    float fh, fl;  // ||x|| / |x0|
+    df_div(xnh, xnl, axh, axl, fh, fl);
+    b = dfc_scale(-fh, -fl, x0);
+    v = x0;  // x0 (1 + f)
+    df_mac(x0.rh, x0.rl, fh, fl, v.rh, v.rl);
+    df_mac(x0.ih, x0.il, fh, fl, v.ih, v.il);
+    dfc_norm(v);
+  } else {
+    b = {-xnh, -xnl, 0.f, 0.f};
+    v = {xnh, xnl, 0.f, 0.f};
   }
-  float rnh, rnl, xnh, xnl;  // 1 / ||x||, ||x||
-  df_rsqrt(t2h, t2l, rnh, rnl);
-  df_mul(t2h, t2l, rnh, rnl, xnh, xnl);
-  // the phase of x0, from x0 2^48 where its square would be too small; none below 2^-108
-  const float up = a2h < 1e-24f ? 281474976710656.0f : 1.0f;
-  const dfc xs = {x0.rh * up, x0.rl * up, x0.ih * up, x0.il * up};
-  float s2h = 0.f, s2l = 0.f;
-  df_abs2_acc(xs, s2h, s2l);
-  df_norm(s2h, s2l);
-  float axh = 0.f, axl = 0.f;
-  dfc ph = {1.f, 0.f, 0.f, 0.f};
-  if (s2h > 1e-36f) {
-    float rah, ral;
-    df_rsqrt(s2h, s2l, rah, ral);
-    ph = dfc_scale(rah, ral, xs);
-    df_mul(s2h, s2l, rah, ral, axh, axl);
-    axh /= up;
-    axl /= up;
+  float vvh = 0.f, vvl = 0.f;
+  df_abs2_acc(v, vvh, vvl);
+  df_add_to(sh, sl, vvh, vvl);
+  df_norm(vvh, vvl);
+  if (vvh > 0.f) {
+    df_div(2.f, 0.f, vvh, vvl, *th, *tl);
+  } else {
+    *th = 0.f;
+    *tl = 0.f;
   }
-  *beta = dfc_scale(-xnh, -xnl, ph);
-  dfc v = x0;
-  df_add_to(-beta->rh, -beta->rl, v.rh, v.rl);
-  df_add_to(-beta->ih, -beta->il, v.ih, v.il);
-  dfc_norm(v);
   *v0 = v;
-  float qh = xnh, ql = xnl, ih, il;
-  df_add_to(axh, axl, qh, ql);
-  df_norm(qh, ql);
-  df_rcp(qh, ql, ih, il);
-  df_mul(ih, il, rnh, rnl, *th, *tl);
+  *beta = b;
 }
 
 // Block-wide double-float sum formed in warp 0 (red: 2 NT floats).  The result is valid

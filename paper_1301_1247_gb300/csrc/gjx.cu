@@ -25,7 +25,7 @@
 // multiply-adds of the strips (FP32 pipes in double-float, FP64 pipe in FP64).
 //
 // Measured against the column-at-a-time elimination that it replaced (one grid barrier per column,
-// every column streamed through L2 at each): inverses in double-float of 16 blocks of 300 in 1.63
+// every column streamed through L2 at each): inverses in double-float of 16 blocks of 300 in 1.64
 // instead of 2.93 ms, 8 of 850 in 12.8 instead of 38.1, one of 1700 in about 13 instead of 40.5, 128 of
 // 250 in 4.6 instead of 20.3; in FP64 one of 1000 in 9.1 instead of 20.7.  The Schur system of one
 // Bloch phase (about 430 unknowns, double-float, with its refinement) takes 1.1 instead of 7.8 ms.
