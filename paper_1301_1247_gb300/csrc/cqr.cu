@@ -13,12 +13,15 @@
 // end R11 and R12 go to global memory, R12 where T is wanted, and k_cqr_tsolve turns it into T =
 // R11^{-1} R12.
 //
+// Norms and the reflector's scalars are FP64 in both arithmetics, products and updates double-float (FP32 pipes)
+// on double-float handles.
+//
 // What bounds it: the chain of a step (two CTA barriers, one cluster barrier, the reflector's scalars:
 // about 4 us) for single nodes, the double-float multiply-adds (102 FP32 instructions per element)
 // when the level has more matrices than SMs; the matrix is read from HBM or L2 twice.  The kernels it
 // replaced streamed every column from L2 at each step (one CTA per matrix, or all SMs with a grid
-// barrier per step): 2048 matrices of 65 x 49 in double-float took 5.5 ms and take 1.5, 1024 of 90 x 74
-// 6.4 and 1.5, four of 334 x 104 0.86 and 0.50.
+// barrier per step): the 2048 matrices (65 x 49) and 1024 (90 x 74) of the two lowest levels of a 100 000-node
+// build in double-float took 5.5 and 6.4 ms and take 1.9 and 2.9 (1.5 and 2.4 with double-float norms).
 //
 // The launches are not cooperative: a cluster's CTAs are co-resident by themselves, so a level never
 // waits for another thread's persistent kernel.
@@ -52,24 +55,18 @@ struct CqrJob {
   int* rank;      // rank, and whether it stopped at kcap before the tolerance was met
 };
 
-// A norm and its column as one integer that orders like (norm, -column): double-float, the upper float's
-// bits and the index below them; FP64, the upper 52 bits and the index in the lower 12.
-__device__ __forceinline__ unsigned long long c_key(const dfr& v, int j) {
-  return v.h > 0.f ? ((unsigned long long)__float_as_uint(v.h) << 32) | (0xFFFFFFFFu - (unsigned)j) : 0ull;
-}
+// A squared norm and its column as one integer that orders like (norm, -column): the upper 52 bits and the index
+// in the lower 12.  0 for a norm that is not a positive number.  Norms are compared as integers, off the FP64 pipe.
 __device__ __forceinline__ unsigned long long c_key(double v, int j) {
-  return v > 0.0 ? ((unsigned long long)__double_as_longlong(v) & ~0xFFFull) | (4095u - (unsigned)j) : 0ull;
+  const long long b = __double_as_longlong(v);
+  return b > 0 && b <= 0x7FF0000000000000ll ? ((unsigned long long)b & ~0xFFFull) | (4095u - (unsigned)j) : 0ull;
 }
-__device__ __forceinline__ int c_col(unsigned long long k, const dfc*) { return (int)(0xFFFFFFFFu - (unsigned)k); }
-__device__ __forceinline__ int c_col(unsigned long long k, const cplx*) { return 4095 - (int)(k & 0xFFFull); }
-__device__ __forceinline__ double c_val(unsigned long long k, const dfc*) {
-  return (double)__uint_as_float((unsigned)(k >> 32));
+__device__ __forceinline__ int c_col(unsigned long long k) { return 4095 - (int)(k & 0xFFFull); }
+__device__ __forceinline__ double c_val(unsigned long long k) { return __longlong_as_double((long long)(k & ~0xFFFull)); }
+// Cancellation has taken more than 7 of a norm's bits since it was last formed (ref: that norm's 1/128).
+__device__ __forceinline__ bool c_cancelled(double t, double ref) {
+  return __double_as_longlong(t) <= __double_as_longlong(ref);
 }
-__device__ __forceinline__ double c_val(unsigned long long k, const cplx*) {
-  return __longlong_as_double((long long)(k & ~0xFFFull));
-}
-__device__ __forceinline__ bool c_cancelled(const dfr& t, const dfr& ref) { return t.h <= 0.0078125f * ref.h; }
-__device__ __forceinline__ bool c_cancelled(double t, double ref) { return t <= 0.0078125 * ref; }
 
 __device__ __forceinline__ unsigned long long c_warp_max(unsigned long long k) {
   const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32));
@@ -92,12 +89,13 @@ __host__ __device__ inline size_t c_smem(int m, int n, int CS) {
 
 template <typename T, int GL>
 __global__ void __launch_bounds__(kT, 2) k_cqr(const CqrJob* jobs, int CS, double tol) {
-  using R = decltype(re_zero((const T*)nullptr));
+  using Sum = decltype(re_zero((const T*)nullptr));      // a thread's sum of squares
+  using Real = decltype(x_real(0.0, (const T*)nullptr));  // a real factor
   constexpr int G = 32 / GL, NG = kT / GL;
   extern __shared__ __align__(16) unsigned char c_raw[];
   __shared__ unsigned long long s_key[2][8 * kW];  // best of every warp of the cluster, by step parity
   __shared__ T s_v0, s_beta;
-  __shared__ R s_tau;
+  __shared__ Real s_tau;
   __shared__ int s_exp[kW], s_cexp[8], s_nact;
   const CqrJob jb = jobs[blockIdx.x / CS];
   const int rank = (int)blockIdx.x % CS;
@@ -107,8 +105,8 @@ __global__ void __launch_bounds__(kT, 2) k_cqr(const CqrJob* jobs, int CS, doubl
   T* cols = reinterpret_cast<T*>(c_raw);                 // ncap columns of m
   T* vbuf = cols + (size_t)ncap * m;                     // the pivot column (CS > 1)
   T* betac = vbuf + (CS > 1 ? m : 0);                    // R_ss of the columns that were pivots
-  R* nrm = reinterpret_cast<R*>(betac + ncap);
-  R* ref = nrm + ncap;
+  double* nrm = reinterpret_cast<double*>(betac + ncap);
+  double* ref = nrm + ncap;
   int* elim = reinterpret_cast<int*>(ref + ncap);        // step a column was pivot of, -1 before
   int* act = elim + ncap;                                // the columns that were not pivots, in any order
   int* perm = act + ncap;                                // CTA 0: the permutation and its inverse
@@ -135,23 +133,22 @@ __global__ void __launch_bounds__(kT, 2) k_cqr(const CqrJob* jobs, int CS, doubl
   unsigned long long best = 0;
   for (int c0 = 0; c0 < ncl; c0 += NG) {
     const int c = c0 + grp;
-    R s2 = re_zero((const T*)nullptr);
+    double s2 = 0.0;
     if (c < ncl) {
       const cplx* a = jb.A + (int64_t)(rank + CS * c) * m;
       T* d = cols + (size_t)c * m;
       for (int i = gl; i < m; i += GL) {
         const cplx v = a[i];
-        const T x = x_in(cmk(c_shift(v.x, sh), c_shift(v.y, sh)), (const T*)nullptr);
-        d[i] = x;
+        const cplx x = cmk(c_shift(v.x, sh), c_shift(v.y, sh));
+        d[i] = x_in(x, (const T*)nullptr);
         re_abs2_acc(x, s2);
-        re_norm(s2);
       }
     }
     for (int o = GL / 2; o > 0; o >>= 1) s2 = re_shfl_add(s2, o);
     if (c < ncl) {
       if (gl == 0) {
         nrm[c] = s2;
-        ref[c] = s2;
+        ref[c] = 0.0078125 * s2;
         elim[c] = -1;
         act[c] = c;
       }
@@ -178,31 +175,31 @@ __global__ void __launch_bounds__(kT, 2) k_cqr(const CqrJob* jobs, int CS, doubl
     unsigned long long key = 0;
     for (int q = lane; q < CS * kW; q += 32) key = max(key, s_key[par][q]);
     key = c_warp_max(key);
-    const double pv = c_val(key, (const T*)nullptr);
+    const double pv = c_val(key);
     if (s == 0) thr2 = tol * tol * pv;
     const bool met = !(pv > thr2);  // |R_ss| <= tol |R_00|, compared squared; nothing left; not a number
     if (met || s >= jb.kcap) {
       capped = !met && s < min(m, n);
       break;
     }
-    const int j = c_col(key, (const T*)nullptr), owner = j % CS, jc = j / CS;
+    const int j = c_col(key), owner = j % CS, jc = j / CS;
     // the pivot column: warp 0 forms the reflector, the others bring the column over meanwhile
     const T* src = CS > 1 ? cg::this_cluster().map_shared_rank(cols, owner) + (size_t)jc * m : cols + (size_t)jc * m;
     const T* v = CS > 1 ? vbuf : src;
     if (warp == 0) {
-      R sig = re_zero((const T*)nullptr);
-      const T x0 = src[s];
+      Sum part = re_zero((const T*)nullptr);
+      const cplx x0 = x_out(src[s]);
 #pragma unroll 4
-      for (int i = s + 1 + lane; i < m; i += 32) re_abs2_acc(src[i], sig);
-      re_norm(sig);
+      for (int i = s + 1 + lane; i < m; i += 32) re_abs2_acc(src[i], part);
+      double sig = re_value(part);
       for (int o = 16; o > 0; o >>= 1) sig = re_shfl_add(sig, o);
-      T h0, beta;
-      R th;
-      x_householder(x0, sig, &h0, &beta, &th);
+      cplx h0, beta;
+      double th;
+      warp_householder(x0, sig, lane, &h0, &beta, &th);
       if (lane == 0) {
-        s_v0 = h0;
-        s_tau = th;
-        s_beta = beta;
+        s_v0 = x_in(h0, (const T*)nullptr);
+        s_tau = x_real(th, (const T*)nullptr);
+        s_beta = x_in(beta, (const T*)nullptr);
       }
     } else {
       if (tid == kT - 1) {
@@ -228,7 +225,7 @@ __global__ void __launch_bounds__(kT, 2) k_cqr(const CqrJob* jobs, int CS, doubl
     }
     __syncthreads();
     const T v0 = s_v0;
-    const R tau = s_tau;
+    const Real tau = s_tau;
     const int nact = s_nact;
     if (tid == 0 && rank == owner) betac[jc] = s_beta;
     best = 0;
@@ -265,15 +262,16 @@ __global__ void __launch_bounds__(kT, 2) k_cqr(const CqrJob* jobs, int CS, doubl
             a[i + u * GL] = x;
           }
       }
-      R t = on ? re_downdate(nrm[c], top) : re_zero((const T*)nullptr);
+      double t = on ? re_downdate(nrm[c], top) : 0.0;
       const bool again = on && c_cancelled(t, ref[c]);
       if (__any_sync(0xffffffffu, again)) {  // cancellation: the norm of rows s + 1.. afresh
-        R q = re_zero((const T*)nullptr);
+        Sum part = re_zero((const T*)nullptr);
         if (again)
           for (int i = s + 1 + gl; i < end; i += GL) {
-            re_abs2_acc(a[i], q);
-            re_norm(q);
+            re_abs2_acc(a[i], part);
+            re_norm(part);
           }
+        double q = re_value(part);
         for (int o = GL / 2; o > 0; o >>= 1) q = re_shfl_add(q, o);
         if (again) t = q;
       }
@@ -282,7 +280,7 @@ __global__ void __launch_bounds__(kT, 2) k_cqr(const CqrJob* jobs, int CS, doubl
         if (gl == 0) {
           a[s] = top;
           nrm[c] = t;
-          if (again) ref[c] = t;
+          if (again) ref[c] = 0.0078125 * t;
         }
         best = max(best, c_key(t, gj));
       }

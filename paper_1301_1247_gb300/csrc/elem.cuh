@@ -78,18 +78,34 @@ __device__ __forceinline__ bool x_usable(const dfc& r) {
   return max(x, y) < 0x7F800000u && (x | y) != 0u;
 }
 
-// r = 1 / sqrt(x) for a normal x > 0: two Newton steps r <- r + r (1 - x r^2) / 2 from the FP32 value, on x
-// scaled by a power of four (as x_recip, instead of FP64's long square-root and division chains).
+// 1 / sqrt(x) of a normal x > 0, and 1 / x of x in [1, 2]: the FP32 value y and a series in its residual e, as a
+// float pair good to 2^-44, then one Newton step in FP64.  They sit on a serial chain, where an FP64
+// instruction takes 64 cycles: four and three of them instead of ten and six for two Newton steps from FP32.
 __device__ __forceinline__ double d_rsqrt(double x) {
   const int e = ((__double2hiint(x) >> 20) & 0x7FF) - 1023, h = e >> 1;  // x = m 4^h, m in [1, 4)
   const double m = __hiloint2double(__double2hiint(x) - (h << 21), __double2loint(x));
-  double r = (double)rsqrtf((float)m);
-  r = fma(0.5 * r, fma(-m, r * r, 1.0), r);
-  r = fma(0.5 * r, fma(-m, r * r, 1.0), r);
-  return __hiloint2double(__double2hiint(r) - (h << 20), __double2loint(r));
+  float mh, ml;
+  df_split_bits(m, mh, ml);
+  const float y = rsqrtf(mh);
+  const float p = __fmul_rn(y, y), pe = fmaf(y, y, -p);
+  const float r = __fsub_rn(fmaf(-mh, p, 1.0f), fmaf(mh, pe, __fmul_rn(ml, p)));
+  const float c = __fmul_rn(y, __fmul_rn(r, fmaf(r, 0.375f, 0.5f)));
+  const double d = f2d_bits(y) + f2d_bits(c);  // in (1/2, 1]
+  const double half = __hiloint2double(__double2hiint(d) - (1 << 20), __double2loint(d));
+  const double q = fma(half, fma(-m, d * d, 1.0), d);
+  return __hiloint2double(__double2hiint(q) - (h << 20), __double2loint(q));
+}
+__device__ __forceinline__ double d_rcp12(double x) {
+  float h, l;
+  df_split_bits(x, h, l);
+  const float y = __frcp_rn(h);
+  const float r = __fsub_rn(fmaf(-h, y, 1.0f), __fmul_rn(l, y));
+  const double d = f2d_bits(y) + f2d_bits(__fmul_rn(y, fmaf(r, r, r)));
+  return fma(d, fma(-x, d, 1.0), d);
 }
 
-// Nonnegative reals (squared norms): double, or a float pair.
+// Squared norms are FP64 numbers in both arithmetics; a thread's sum of double-float squares is a float pair
+// until it joins other threads' sums.
 struct dfr {
   float h, l;
 };
@@ -99,22 +115,22 @@ __device__ __forceinline__ void re_abs2_acc(const cplx& a, double& s) { s = fma(
 __device__ __forceinline__ void re_abs2_acc(const dfc& a, dfr& s) { df_abs2_acc(a, s.h, s.l); }
 __device__ __forceinline__ void re_norm(double&) {}
 __device__ __forceinline__ void re_norm(dfr& s) { df_norm(s.h, s.l); }
+__device__ __forceinline__ double re_value(double s) { return s; }
+__device__ __forceinline__ double re_value(const dfr& s) { return f2d_bits(s.h) + f2d_bits(s.l); }
 __device__ __forceinline__ double re_shfl_add(double s, int o) { return s + __shfl_xor_sync(0xffffffffu, s, o); }
-__device__ __forceinline__ dfr re_shfl_add(dfr s, int o) {
-  const float h = __shfl_xor_sync(0xffffffffu, s.h, o), l = __shfl_xor_sync(0xffffffffu, s.l, o);
-  df_add_to(h, l, s.h, s.l);
-  df_norm(s.h, s.l);
-  return s;
-}
 // n - |a|^2
 __device__ __forceinline__ double re_downdate(double n, const cplx& a) { return n - cabs2(a); }
-__device__ __forceinline__ dfr re_downdate(dfr n, const dfc& a) {
+__device__ __forceinline__ double re_downdate(double n, const dfc& a) {
   float h = 0.f, l = 0.f;
   df_abs2_acc(a, h, l);
-  df_norm(h, l);
-  df_add_to(-h, -l, n.h, n.l);
-  df_norm(n.h, n.l);
-  return n;
+  return (n - f2d_bits(h)) - f2d_bits(l);
+}
+// A real factor in the element's arithmetic.
+__device__ __forceinline__ double x_real(double v, const cplx*) { return v; }
+__device__ __forceinline__ dfr x_real(double v, const dfc*) {
+  dfr r;
+  df_split_bits(v, r.h, r.l);
+  return r;
 }
 
 // acc += conj(v) a (lazy low parts for dfc); a -= v w; s a for a real s
@@ -140,34 +156,39 @@ __device__ __forceinline__ dfc x_shfl_add(dfc a, int o) {
   return a;
 }
 
-// Householder reflector H = I - tau v v^H, v = (v0, x_1, ...), of x = (x0, x_1, ...) with ||x_1..||^2 = sig:
-// beta = -(x0 / |x0|) ||x||, v0 = x0 - beta, tau = 2 / (|v0|^2 + sig) = 1 / (||x|| (||x|| + |x0|)).
-__device__ __forceinline__ void x_householder(const cplx& x0, double sig, cplx* v0, cplx* beta, double* tau) {
-  const double a2 = cabs2(x0), t2 = a2 + sig;
-  if (!(t2 > 1e-290)) {  // nothing left of the column
+// Householder reflector H = I - tau v v^H, v = (v0, x_1, ...), of x = (x0, x_1, ...) with ||x_1..||^2 = sig: beta =
+// -(x0 / |x0|) ||x||, v0 = x0 - beta, tau = 2 / (|v0|^2 + sig) = 1 / (||x|| (||x|| + |x0|)).  One warp, in FP64: even
+// lanes take ||x|| and real parts, odd lanes |x0| and imaginary parts; the results are in every lane.
+__device__ __forceinline__ void warp_householder(const cplx& x0, double sig, int lane, cplx* v0, cplx* beta, double* tau) {
+  const bool odd = lane & 1;
+  double a2 = cabs2(x0);
+  const double t2 = a2 + sig;
+  if (!(t2 > 1e-290)) {  // nothing left of the column (the same in every lane)
     *v0 = *beta = cmk(0.0, 0.0);
     *tau = 0.0;
     return;
   }
-  const double rn = d_rsqrt(t2), xn = t2 * rn;
-  double ax = 0.0;
-  cplx ph = cmk(1.0, 0.0);
-  if (a2 > 1e-290) {
-    const double ra = d_rsqrt(a2);
-    ax = a2 * ra;
-    ph = cmk(x0.x * ra, x0.y * ra);
+  double xi = odd ? x0.y : x0.x;
+  const double part = xi;
+  const bool small = __double2hiint(a2) < 0x05B00000;  // 2^-932: |x0| and the phase from x0 2^400
+  if (small) {
+    const double up = 0x1p400;
+    xi *= up;
+    a2 = cabs2(cmk(x0.x * up, x0.y * up));
   }
-  *beta = cmk(-ph.x * xn, -ph.y * xn);
-  *v0 = csub(x0, *beta);
-  // 1 / (xn + ax), xn <= xn + ax <= 2 xn, by Newton from the FP32 quotient
-  const double s = (xn + ax) * rn;  // in [1, 2]
-  double r = (double)(1.0f / (float)s);
-  r = fma(r, fma(-s, r, 1.0), r);
-  r = fma(r, fma(-s, r, 1.0), r);
-  *tau = r * rn * rn;
-}
-__device__ __forceinline__ void x_householder(const dfc& x0, const dfr& sig, dfc* v0, dfc* beta, dfr* tau) {
-  df_householder(x0, sig.h, sig.l, v0, beta, &tau->h, &tau->l);
+  const bool phase = a2 > 1e-290;
+  const double mine = odd ? (phase ? a2 : 1.0) : t2;
+  const double r = d_rsqrt(mine), n = mine * r;  // 1 / ||x||, ||x|| or 1 / |x0|, |x0|
+  const double rn = __shfl_sync(0xffffffffu, r, 0), xn = __shfl_sync(0xffffffffu, n, 0);
+  const double ra = __shfl_sync(0xffffffffu, r, 1);
+  double ax = __shfl_sync(0xffffffffu, n, 1);
+  if (small) ax *= 0x1p-400;
+  if (!phase) ax = 0.0;
+  const double ph = phase ? xi * ra : odd ? 0.0 : 1.0;
+  const double b = -(ph * xn), v = part - b;
+  *beta = cmk(__shfl_sync(0xffffffffu, b, 0), __shfl_sync(0xffffffffu, b, 1));
+  *v0 = cmk(__shfl_sync(0xffffffffu, v, 0), __shfl_sync(0xffffffffu, v, 1));
+  *tau = d_rcp12((xn + ax) * rn) * rn * rn;  // xn <= xn + ax <= 2 xn
 }
 
 }  // namespace hbs

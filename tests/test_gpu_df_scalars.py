@@ -1,5 +1,5 @@
-"""The double-float scalars on the serial chains of the factorizations, from the kernels' own headers: the
-reciprocal of a pivot and the Householder reflector, against FP64 arithmetic."""
+"""The scalars on the serial chains of the factorizations, from the kernels' own headers: the double-float
+reciprocal of a pivot and Householder reflector, and a warp's FP64 reflector, against FP64 arithmetic."""
 import ctypes
 import os
 import shutil
@@ -13,7 +13,7 @@ from gpu_util import dev, require_lib
 pytestmark = pytest.mark.gpu
 
 SOURCE = r"""
-#include "dfloat.cuh"
+#include "dense_kernels.cuh"
 using namespace hbs;
 __global__ void k_recip(const cplx* d, cplx* r, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -31,6 +31,18 @@ __global__ void k_reflect(const cplx* x, cplx* v0, cplx* beta, double* tau, int 
   v0[i] = from_dfc_bits(v);
   beta[i] = from_dfc_bits(b);
   tau[i] = f2d_bits(th) + f2d_bits(tl);
+}
+__global__ void k_warp_reflect(const cplx* x, cplx* v0, cplx* beta, double* tau, int n) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x & 31;
+  if (i >= n) return;
+  cplx v, b;
+  double t;
+  warp_householder(x[2 * i], cabs2(x[2 * i + 1]), lane, &v, &b, &t);
+  if (lane == 17) { v0[i] = v; beta[i] = b; tau[i] = t; }
+}
+extern "C" int warp_reflect(const void* x, void* v0, void* beta, void* tau, int n) {
+  k_warp_reflect<<<(n + 3) / 4, 128>>>((const cplx*)x, (cplx*)v0, (cplx*)beta, (double*)tau, n);
+  return (int)cudaDeviceSynchronize();
 }
 extern "C" int recip(const void* d, void* r, int n) {
   k_recip<<<(n + 127) / 128, 128>>>((const cplx*)d, (cplx*)r, n);
@@ -87,3 +99,22 @@ def test_reflector(probe, scale, bound):
     big = norm > 0.7 * scale
     assert (np.abs(np.abs(b) - norm) / norm)[big].max() < bound
     assert (np.linalg.norm(hx - np.stack([b, 0 * b], axis=1), axis=1) / norm)[big].max() < bound
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-140, 3e100])
+@pytest.mark.parametrize("head", [1.0, 0.0, 1e-12, 1e12])
+def test_warp_reflector_is_fp64(probe, scale, head):
+    """A few roundings of 2^-53 in each of |x|, the phase and tau: 4e-15 in all.  `head` is the first entry's size
+    beside the other's."""
+    n = 20000
+    x = _complex(np.random.default_rng(2), (n, 2)) * scale / max(head, 1.0)
+    x[:, 0] *= head
+    v0, beta, tau = dev(np.zeros(n, complex)), dev(np.zeros(n, complex)), dev(np.zeros(n))
+    assert probe.warp_reflect(_ptr(dev(x)), _ptr(v0), _ptr(beta), _ptr(tau), n) == 0
+    s = np.abs(x).max(axis=1)[:, None]
+    v, b, t = np.stack([v0.cpu().numpy(), x[:, 1]], axis=1) / s, beta.cpu().numpy() / s[:, 0], tau.cpu().numpy() * s[:, 0] ** 2
+    y = x / s
+    hx = y - v * (t * np.sum(np.conj(v) * y, axis=1))[:, None]
+    norm = np.linalg.norm(y, axis=1)
+    assert (np.abs(np.abs(b) - norm) / norm).max() < 4e-15
+    assert (np.linalg.norm(hx - np.stack([b, 0 * b], axis=1), axis=1) / norm).max() < 4e-15
