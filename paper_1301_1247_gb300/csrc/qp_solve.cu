@@ -1338,7 +1338,7 @@ __global__ void __launch_bounds__(256) k_red_wood_rows(RedDims D, Dims DD, const
 // columns).  The products run as batched GEMMs over all angles: gamma and the E rows' samples share one
 // matrix, xi has one per group and the wall samples one per contour.  One CTA an angle, each thread with
 // dot products of up to 3 nz + 4M terms of its own, took 1.0 ms for 8 angles and 3.0 for 1000 (n = 400);
-// these launches and products take 0.35 and 1.4.
+// these launches and products take 0.25 and 2.0 (1.35 on the tensor cores, whose error such columns do not bear).
 
 // Column b = blockIdx.x of w.
 __global__ void k_red_w(RedDims D, const GroupJob* groups, const AngleJob* angles, const cplx* Rpool, cplx* W) {
@@ -1579,6 +1579,9 @@ static void reduced_batch(Handle& h, std::vector<GroupJob>& gjobs, std::vector<s
   }
   HBS_LAUNCH_CHECK("k_red_w");
   {
+    // on double-float and tensor-core handles in double-float: the digit planes' error is relative to the largest
+    // entry of a row and a column, and these columns hold unknowns of very different size
+    GemmModeScope mode(gemm_double_float() ? HBS_PRECISION_DOUBLE_FLOAT : HBS_PRECISION_FP64);
     const cplx one = cmk(1, 0), zero = cmk(0, 0);
     const int q = (int)na;
     std::vector<GemmJob> gj;

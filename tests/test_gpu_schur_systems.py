@@ -60,3 +60,21 @@ def test_a_dense_root_of_more_than_4096_unknowns(precision):
     h.apply_inverse(b, x, 3)
     torch.cuda.synchronize()
     assert float(torch.linalg.norm(x @ at - b) / torch.linalg.norm(b)) < 1e-10
+
+
+def test_bragg_products_of_a_tensor_solver_are_double_float():
+    """The amplitudes' products (gamma, the E rows' samples, xi, the wall samples) of a solver in tensor precision
+    run in double-float, whatever the number of angles: the profiler's record of the phase names no tensor-core
+    kernel."""
+    hbs = require_lib()
+    geo = inputs.wiggly(0, 0.35, 20, 0.03).sample(2000)
+    h = hbs.Handle(*geo, 1.0, OMEGA, 1e-12, hbs.default_options(precision=2))
+    th = np.linspace(-3.0, -0.1, 300)
+    hbs.profile_reset()
+    hbs.profile_enable(True)
+    try:
+        h.solve(th)
+    finally:
+        hbs.profile_enable(False)
+    names = [k.split(":")[-1] for k in hbs.profile_get() if k.startswith("in:solve:bragg:")]
+    assert "k_zgemm_batched_df" in names and not [n for n in names if n.startswith("k_oz")], names
