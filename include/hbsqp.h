@@ -62,7 +62,7 @@ typedef struct hbs_geometry {
  * refinement against the FP64 system) run in the same arithmetic. */
 #define HBS_PRECISION_DOUBLE_FLOAT 1
 /* As HBS_PRECISION_DOUBLE_FLOAT, and the larger dense products (inner dimension >= 96 and at least 48
- * rows; in large batches >= 32 and at least 96 rows) run on the tcgen05 tensor cores: every FP64 row of op(A) and column
+ * rows) run on the tcgen05 tensor cores: every FP64 row of op(A) and column
  * of B is scaled by a power of two and cut into seven 7-bit integer digits held exactly
  * in bf16; the digit products are accumulated exactly, in FP32 tensor memory over 224
  * values of k and as 64-bit integers beyond, and rounded once (relative error about 2^-46 of

@@ -427,18 +427,7 @@ static void launch_gemms(std::vector<GemmJob>& jobs_all, cudaStream_t s) {
   if (jobs_all.empty()) return;
   // large products on the tensor cores when the thread's mode asks for it
   std::vector<GemmJob> jobs_in, jobs_tc;
-  if (gemm_tensor()) {
-    double work = 0.0;
-    for (const auto& j : jobs_all)
-      if (ozaki_eligible_short(j)) work += (double)j.m * j.n * j.k;
-    const bool shorts = work >= kOzakiShortWork;
-    for (const auto& j : jobs_all) {
-      if (ozaki_eligible(j) || (shorts && ozaki_eligible_short(j))) jobs_tc.push_back(j);
-      else jobs_in.push_back(j);
-    }
-  } else {
-    jobs_in = jobs_all;
-  }
+  for (const auto& j : jobs_all) (gemm_tensor() && ozaki_eligible(j) ? jobs_tc : jobs_in).push_back(j);
   ozaki_gemm_batched(jobs_tc, s);
   if (jobs_in.empty()) return;
   double fl = 0.0, by = 0.0;

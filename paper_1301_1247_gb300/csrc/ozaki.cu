@@ -27,9 +27,8 @@
 // product run while the outputs of the last are written; only the read of the accumulators
 // itself, which fill 448 of tensor memory's 512 columns, stands between two periods.
 //
-// Short products pay for their outputs: per 128 x 32 outputs 4 400 cycles to read the accumulators and 8
-// 200 of FP64 additions to round them, beside 7 200 of MMAs for k = 49 (with integer rounding the
-// outputs took 22 000).  690 x 8192 x 49: 0.124 ms, and 0.66 ms in double-float.
+// Per 128 x 32 outputs 4 400 cycles go to reading the accumulators and 8 200 to the FP64 additions that round them
+// (22 000 with integer rounding), beside 450 of MMAs for every stage.
 //
 // What bounds it: the MMAs (28 per 16 k, 3584 columns of N in all) and, within a factor of two, the
 // 70 KB that each stage brings from L2.  690 x 192 x 100 000: 2.36 ms, 1.40 PFLOP/s of executed
@@ -601,11 +600,12 @@ __global__ void k_oz_reduce(const cplx* W, int m, int n, int splits, cplx beta, 
 
 }  // namespace
 
-// Products worth the tensor cores: k >= 96 and half a tile's rows; of those with 32 <= k < 96, which the
-// digit planes cost as much as the MMAs, the ones that nearly fill their 128-row tiles, and only when
-// the batch has enough of them (kOzakiShortWork): the path takes two more launches and a wait.  (At most 2^26 values of k: the 64-bit sums hold 2^27.)
+// Products worth the tensor cores: k >= 96 and half a tile's rows.  (At most 2^26 values of k: the 64-bit sums hold
+// 2^27.)  Shorter ones stay in double-float although they were faster here (690 x 2048 x 49 0.112 ms against
+// 0.165): the digit planes' error is relative to the largest entry of a row and a column, double-float's to each
+// term.  Against FP64 on the operands of the builds the short products' normwise error was up to 24 times
+// double-float's (8.9e-13 and 3.7e-14 for 138 x 72 x 72), and operands graded over 12 decades left 4e-4 for 2e-14.
 bool ozaki_eligible(const GemmJob& j) { return j.k >= 96 && j.k <= (1 << 26) && j.m >= 48 && j.n >= 8; }
-bool ozaki_eligible_short(const GemmJob& j) { return j.k >= 32 && j.k < 96 && j.m >= 96 && j.n >= 16; }
 
 // A batch of products on the tensor cores (see the head of this file): exponents and digit
 // planes of every operand (two launches), one persistent MMA launch over all tiles, and a

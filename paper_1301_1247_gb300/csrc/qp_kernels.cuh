@@ -95,10 +95,6 @@ void run_gemms(std::vector<GemmJob>& jobs, cudaStream_t s);
 // Tensor-core (digit-plane) products of a batch of jobs (ozaki.cu); eligible: large enough
 // to pay.
 bool ozaki_eligible(const GemmJob& j);
-// Short products (32 <= k < 96) go there too when a batch has kOzakiShortWork multiply-adds of them
-// (690 x 2048 x 49, 6.9e7: 165 us in double-float, 112 there; 20 000 x 49 x 49, 4.8e7: 138 and 129).
-bool ozaki_eligible_short(const GemmJob& j);
-constexpr double kOzakiShortWork = 5e7;
 void ozaki_gemm_batched(const std::vector<GemmJob>& jobs, cudaStream_t s);
 std::vector<int> batched_id(std::vector<CpqrJob>& jobs, double tol, cudaStream_t s);
 // cqr.cu: the same with each matrix in the shared memory of one cluster; the cluster size for matrices up to
