@@ -59,7 +59,9 @@ typedef struct hbs_geometry {
  * two floats and multiplied and accumulated error-free on the FP32 pipes (about 48
  * significant bits, relative error near 1e-14 per product).  The updates of the interpolative
  * decompositions, the inversions, the Hankel polynomials and the Schur solves (with one step of
- * refinement against the FP64 system) run in the same arithmetic. */
+ * refinement against the FP64 system, its correction in FP64) run in the same arithmetic; the norms and
+ * reflectors of the node matrices' decompositions are FP64, and the periodizer's interpolation coefficients
+ * take the digit planes described below, which are the more accurate there. */
 #define HBS_PRECISION_DOUBLE_FLOAT 1
 /* As HBS_PRECISION_DOUBLE_FLOAT, and the larger dense products (inner dimension >= 96 and at least 48
  * rows) run on the tcgen05 tensor cores: every FP64 row of op(A) and column
@@ -402,7 +404,9 @@ hbs_status hbs_row_id_static(void* mt, int64_t m, int64_t n, double tol, int* ra
  *  - HBS_INJECT_RANK_CAP: interpolative decompositions of the persistent QR (tree
  *    levels of at most 128 nodes, the neighbour and periodizer IDs, hbs_row_id with
  *    n > 4096) may reach rank `value` at most (0 = no cap); one that needs more
- *    returns HBS_ERR_RANK, as an overflow of the supported maximum would.
+ *    returns HBS_ERR_RANK, as an overflow of the supported maximum would;
+ *  - HBS_INJECT_ID_RESIDUAL: the next `value` checks of a build's periodizer IDs that were
+ *    found on candidate contour nodes count as failed, so that the build repeats them on all nodes.
  * Returns HBS_ERR_INVALID_ARG for an unknown kind or a negative value.
  *
  * hbs_barrier_selftest runs the library's bounded grid barrier (the one the
@@ -415,6 +419,7 @@ hbs_status hbs_row_id_static(void* mt, int64_t m, int64_t n, double tol, int* ra
 #define HBS_INJECT_CLEAR 0
 #define HBS_INJECT_ALLOC_FAILURE 1
 #define HBS_INJECT_RANK_CAP 2
+#define HBS_INJECT_ID_RESIDUAL 3
 hbs_status hbs_fault_inject(int kind, int64_t value);
 hbs_status hbs_barrier_selftest(int ctas, int absent_cta, double limit_s, int* passed, void* stream);
 

@@ -35,8 +35,10 @@ inline void cuda_check(cudaError_t e, const char* what) {
 cudaStream_t& current_stream();
 
 // Fault injection for tests of the error paths (hbs_fault_inject): true when the caller's
-// device allocation is the one chosen to fail; the largest rank an ID may reach (0 = none).
+// device allocation is the one chosen to fail; the largest rank an ID may reach (0 = none); true when the
+// check of a periodizer ID is to count as failed.
 bool injected_alloc_failure();
+bool injected_id_residual();
 
 // Raise a kernel's limit on dynamic shared memory to at least `bytes` (cudaFuncSetAttribute)
 // on the current device.  The limit only ever grows, under a lock: two host threads that

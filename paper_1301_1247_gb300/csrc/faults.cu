@@ -3,7 +3,7 @@
 // Nothing here makes a GPU fault, trap or hang.  An injected allocation failure is raised on
 // the host before cudaMallocAsync is called; an injected rank cap lowers the largest rank the
 // persistent QR may reach, so that it stops short of the tolerance exactly as a real
-// overflow would.  The barrier self-test runs the library's own grid barrier (gridsync.cuh)
+// overflow would; an injected residual makes the check of a periodizer ID read as failed.  The barrier self-test runs the library's own grid barrier (gridsync.cuh)
 // with one CTA that leaves before a barrier: the others wait for it only until a short limit,
 // then return, and the host reports HBS_ERR_TIMEOUT as the solver's kernels do.
 #include <atomic>
@@ -18,6 +18,7 @@ namespace hbs {
 namespace {
 std::atomic<int64_t> g_alloc_countdown{-1};  // allocations left before the failing one (-1: off)
 std::atomic<int> g_rank_cap{0};
+std::atomic<int64_t> g_id_checks{0};  // checks of periodizer IDs that are still to fail
 }  // namespace
 
 bool injected_alloc_failure() {
@@ -25,6 +26,13 @@ bool injected_alloc_failure() {
   while (v >= 0) {
     if (g_alloc_countdown.compare_exchange_weak(v, v - 1, std::memory_order_relaxed)) return v == 0;
   }
+  return false;
+}
+
+bool injected_id_residual() {
+  int64_t v = g_id_checks.load(std::memory_order_relaxed);
+  while (v > 0)
+    if (g_id_checks.compare_exchange_weak(v, v - 1, std::memory_order_relaxed)) return true;
   return false;
 }
 
@@ -47,6 +55,7 @@ extern "C" hbs_status hbs_fault_inject(int kind, int64_t value) {
     case HBS_INJECT_CLEAR:
       hbs::g_alloc_countdown.store(-1);
       hbs::g_rank_cap.store(0);
+      hbs::g_id_checks.store(0);
       return HBS_OK;
     case HBS_INJECT_ALLOC_FAILURE:
       if (value < 0) break;
@@ -55,6 +64,10 @@ extern "C" hbs_status hbs_fault_inject(int kind, int64_t value) {
     case HBS_INJECT_RANK_CAP:
       if (value < 0 || value > (1 << 30)) break;
       hbs::g_rank_cap.store((int)value);
+      return HBS_OK;
+    case HBS_INJECT_ID_RESIDUAL:
+      if (value < 0) break;
+      hbs::g_id_checks.store(value);
       return HBS_OK;
     default:
       break;

@@ -286,22 +286,24 @@ void build_periodizer(Handle& h, cudaStream_t s, bool with_hbs, const std::share
   const int nce = 12 * S;
   // The three families' IDs run in one persistent QR launch (one after another they took
   // longer: their pivot steps then add up).  Skeletons are chosen among candidates: every
-  // cstride-th contour node of each block and the last.  Along the contour a member changes like
-  // e^{i k y} e^{i s x}, so a step of 0.6 / max(d, the obstacle's height) between candidates leaves
-  // at least ten to an oscillation, as the neighbour ID below has many nodes to a wavelength; the
-  // contour's bend, of width w and depth c, is resolved with a step of 0.3 of either.  Every
-  // member's coefficients follow by least squares against the skeleton, T = R11^{-1} Q1^H A, which
-  // for the candidates is the QR's own T.  The QR is bound by its passes over the candidates, one
-  // a pivot: with a third of the columns it takes 1.7 ms instead of
-  // 2.9 (ranks up to 150, 512 samples), and what replaces the rest of the QR is one product.  Each ID is checked on the second subsample
-  // (all members rebuilt from the skeleton).
+  // cstride-th contour node of each block and the last.  Every member's coefficients follow by least squares
+  // against the skeleton, T = R11^{-1} Q1^H A, which for the candidates is the QR's own T.  The QR is
+  // bound by its passes over the candidates, one a pivot: with a third of the columns it takes 1.7 ms instead
+  // of 2.9 (ranks up to 150, 512 samples), and what replaces the rest of the QR is one product.
+  // Each ID is checked on the second subsample (all members rebuilt from the skeleton).
+  //
+  // The skeletons are held to a quarter of the tolerance (ranks larger by about 3 %), which leaves smaller residuals
+  // than every member a candidate and the whole tolerance did, for omega 8 to 110 and contours 0.7 to 4 deep
+  // and wide.  How fine the candidates have to be depends on phases k y + s x that no simple bound covers
+  // (|ds/dk| = |k / s| grows towards the branch points); in all those cases they outnumber the rank
+  // many times.  So the step is a rule of thumb and the check decides: a residual of the wall families above
+  // 1e-13 sends the families through again with every member a candidate.
   double ylo = h.hy[0], yhi = h.hy[0];
   for (double y : h.hy) {
     ylo = std::min(ylo, y);
     yhi = std::max(yhi, y);
   }
   const double cstep = std::min(0.6 / std::max(d, yhi - ylo), 0.3 * std::min(h.cc, h.cw));
-  const int cstride = std::max(1, std::min(3, (int)(cstep / h.ch + 1e-9)));
   struct Family {
     int family, ncols;
     DevBuf<cplx> A, A2, Mc;
@@ -312,7 +314,6 @@ void build_periodizer(Handle& h, cudaStream_t s, bool with_hbs, const std::share
   fams[0].family = 0; fams[0].ncols = ny;
   fams[1].family = 1; fams[1].ncols = ny;
   fams[2].family = 2; fams[2].ncols = nce;
-  std::vector<PqrSpec> fspecs;
   for (Family& f : fams) {
     const int ncols = f.ncols;
     f.A.alloc((size_t)ns * ncols);
@@ -325,92 +326,121 @@ void build_periodizer(Handle& h, cudaStream_t s, bool with_hbs, const std::share
                                                                        ns2, ncols, f.A2.get(), ns2);
     }
     HBS_LAUNCH_CHECK("k_fill_family_sub");
-    const int block = f.family < 2 ? M : nce, stride = f.family < 2 ? cstride : 1;
-    for (int c = 0; c < ncols; ++c)
-      if ((c % block) % stride == 0 || c % block == block - 1) f.cand.push_back(c);
-    const int64_t nc = (int64_t)f.cand.size();
-    f.Mc.alloc((size_t)ns * nc);
-    DevBuf<int64_t> dcand;
-    dcand.upload(f.cand, s);
-    {
-      prof::KScope _ks("k_gather_cols", s);
-      k_gather_cols<<<grid_1d(ns * nc), 256, 0, s>>>(f.A.get(), ns, ns, dcand.get(), nc, f.Mc.get(), ns);
-    }
-    HBS_LAUNCH_CHECK("k_gather_cols");
-    f.perm.alloc(nc);
-    fspecs.push_back({f.Mc.get(), ns, nc, (int)std::min<int64_t>(ns, nc), f.perm.get(), nullptr});
   }
-  PqrOut fqr;
-  pqr_run(fspecs, ptol, s, fqr, /*equal_steps=*/true);  // family ranks are alike (~100-200 at w = 60)
-  const std::vector<int> fpiv = fqr.piv.download(s);
   std::vector<int> fperm[3];
   DevBuf<cplx>* Touts[3] = {&h.TY, &h.TC, &h.TE};
   int franks[3];
-  DevBuf<cplx> Qc[3], Tall[3], G2[3], B2[3];
-  DevBuf<int64_t> dord[3];
-  QcJobs qcj{};
-  std::vector<GemmJob> tj, bj;  // T' = Q1^H A, and the members rebuilt on the check sample
-  for (int fi = 0; fi < 3; ++fi) {
-    Family& f = fams[fi];
-    const int ncols = f.ncols, r = franks[fi] = fqr.rank[fi];
-    std::vector<char> skel(ncols, 0);
-    std::vector<int64_t> order;  // the skeleton members, then the others
-    for (int i = 0; i < r; ++i) {
-      order.push_back(f.cand[fpiv[fqr.koff[fi] + i]]);
-      skel[order.back()] = 1;
+  // The IDs with every cstride-th contour node a candidate; returns the wall families' residual.
+  const auto identify = [&](int cstride) {
+    std::vector<PqrSpec> fspecs;
+    for (Family& f : fams) {
+      const int ncols = f.ncols;
+      f.cand.clear();
+      const int block = f.family < 2 ? M : nce, stride = f.family < 2 ? cstride : 1;
+      for (int c = 0; c < ncols; ++c)
+        if ((c % block) % stride == 0 || c % block == block - 1) f.cand.push_back(c);
+      const int64_t nc = (int64_t)f.cand.size();
+      f.Mc.alloc((size_t)ns * nc);
+      DevBuf<int64_t> dcand;
+      dcand.upload(f.cand, s);
+      {
+        prof::KScope _ks("k_gather_cols", s);
+        k_gather_cols<<<grid_1d(ns * nc), 256, 0, s>>>(f.A.get(), ns, ns, dcand.get(), nc, f.Mc.get(), ns);
+      }
+      HBS_LAUNCH_CHECK("k_gather_cols");
+      f.perm.alloc(nc);
+      fspecs.push_back({f.Mc.get(), ns, nc, (int)std::min<int64_t>(ns, nc), f.perm.get(), nullptr});
     }
-    for (int c = 0; c < ncols; ++c)
-      if (!skel[c]) order.push_back(c);
-    fperm[fi].assign(order.begin(), order.end());
-    Touts[fi]->alloc(std::max<int64_t>((int64_t)r * (ncols - r), 1));
-    if (r == 0) continue;
-    dord[fi].upload(order, s);
-    Qc[fi].alloc((size_t)ns * r);
-    Tall[fi].alloc((size_t)r * ncols);
-    G2[fi].alloc((size_t)ns2 * r);
-    B2[fi].alloc((size_t)ns2 * ncols);
-    qcj.j[fi] = {f.Mc.get(), fqr.piv.get() + fqr.koff[fi], fqr.v0.get() + fqr.koff[fi], fqr.tau.get() + fqr.koff[fi],
-                 r, Qc[fi].get()};
-    const cplx one = cmk(1.0, 0.0), zero = cmk(0.0, 0.0);
-    tj.push_back(GemmJob{Qc[fi].get(), f.A.get(), Tall[fi].get(), r, ncols, ns, ns, ns, r, one, zero, 0, 0, 0, 1});
-    bj.push_back(
-        GemmJob{G2[fi].get(), Tall[fi].get(), B2[fi].get(), ns2, ncols, r, ns2, r, ns2, one, zero, 0, 0, 0, 0});
-  }
-  h.pid_residual = 0.0;
-  if (!tj.empty()) {
-    {
-      prof::KScope _ks("k_form_qc", s);
-      k_form_qc<<<dim3(*std::max_element(franks, franks + 3), 3), 256, 0, s>>>(qcj, ns);
-    }
-    HBS_LAUNCH_CHECK("family Q1");
-    run_gemms(tj, s);
+    PqrOut fqr;
+    pqr_run(fspecs, 0.25 * ptol, s, fqr, /*equal_steps=*/true);  // family ranks are alike (~100-200 at w = 60)
+    const std::vector<int> fpiv = fqr.piv.download(s);
+    DevBuf<cplx> Qc[3], Tall[3], G2[3], B2[3];
+    DevBuf<int64_t> dord[3];
+    QcJobs qcj{};
+    std::vector<GemmJob> tj, bj;  // T' = Q1^H A, and the members rebuilt on the check sample
     for (int fi = 0; fi < 3; ++fi) {
       Family& f = fams[fi];
-      const int ncols = f.ncols, r = franks[fi], rest = ncols - r;
+      const int ncols = f.ncols, r = franks[fi] = fqr.rank[fi];
+      std::vector<char> skel(ncols, 0);
+      std::vector<int64_t> order;  // the skeleton members, then the others
+      for (int i = 0; i < r; ++i) {
+        order.push_back(f.cand[fpiv[fqr.koff[fi] + i]]);
+        skel[order.back()] = 1;
+      }
+      for (int c = 0; c < ncols; ++c)
+        if (!skel[c]) order.push_back(c);
+      fperm[fi].assign(order.begin(), order.end());
+      Touts[fi]->alloc(std::max<int64_t>((int64_t)r * (ncols - r), 1));
       if (r == 0) continue;
-      pqr_solve_r11(f.Mc.get(), ns, fqr, fi, r, Tall[fi].get(), r, ncols, s);
-      prof::KScope _ks("k_gather_cols", s);
-      if (rest > 0)
-        k_gather_cols<<<grid_1d((int64_t)r * rest), 256, 0, s>>>(Tall[fi].get(), r, r, dord[fi].get() + r, rest,
-                                                                 Touts[fi]->get(), r);
-      k_gather_cols<<<grid_1d((int64_t)ns2 * r), 256, 0, s>>>(f.A2.get(), ns2, ns2, dord[fi].get(), r, G2[fi].get(),
-                                                              ns2);
+      dord[fi].upload(order, s);
+      Qc[fi].alloc((size_t)ns * r);
+      Tall[fi].alloc((size_t)r * ncols);
+      G2[fi].alloc((size_t)ns2 * r);
+      B2[fi].alloc((size_t)ns2 * ncols);
+      qcj.j[fi] = {f.Mc.get(), fqr.piv.get() + fqr.koff[fi], fqr.v0.get() + fqr.koff[fi], fqr.tau.get() + fqr.koff[fi],
+                   r, Qc[fi].get()};
+      const cplx one = cmk(1.0, 0.0), zero = cmk(0.0, 0.0);
+      tj.push_back(GemmJob{Qc[fi].get(), f.A.get(), Tall[fi].get(), r, ncols, ns, ns, ns, r, one, zero, 0, 0, 0, 1});
+      bj.push_back(
+          GemmJob{G2[fi].get(), Tall[fi].get(), B2[fi].get(), ns2, ncols, r, ns2, r, ns2, one, zero, 0, 0, 0, 0});
     }
-    run_gemms(bj, s);
-    DevBuf<double> acc(6);
-    HBS_CUDA(cudaMemsetAsync(acc.get(), 0, 6 * sizeof(double), s));
-    for (int fi = 0; fi < 3; ++fi) {
-      if (franks[fi] == 0) continue;
-      const Family& f = fams[fi];
-      prof::KScope _ks("k_diff_norm2", s);
-      k_diff_norm2<<<grid_1d((int64_t)ns2 * f.ncols), 256, 0, s>>>(B2[fi].get(), ns2, f.A2.get(), ns2, ns2, f.ncols,
-                                                                    acc.get() + 2 * fi);
+    h.pid_residual = 0.0;
+    double walls = 0.0;
+    if (!tj.empty()) {
+      {
+        prof::KScope _ks("k_form_qc", s);
+        k_form_qc<<<dim3(*std::max_element(franks, franks + 3), 3), 256, 0, s>>>(qcj, ns);
+      }
+      HBS_LAUNCH_CHECK("family Q1");
+      {
+        // not in double-float, whose products of 512 terms leave residuals of 5e-14 to 8e-14: the digit planes leave
+        // the 2e-14 to 4e-14 of FP64, at ranks below those that they pay for too (FP64 products would
+        // take the pipe that the compression's QRs need beside them)
+        if (gemm_double_float() && ns >= 96) {
+          ozaki_gemm_batched(tj, s);
+        } else {
+          GemmModeScope mode(HBS_PRECISION_FP64);
+          run_gemms(tj, s);
+        }
+      }
+      for (int fi = 0; fi < 3; ++fi) {
+        Family& f = fams[fi];
+        const int ncols = f.ncols, r = franks[fi], rest = ncols - r;
+        if (r == 0) continue;
+        pqr_solve_r11(f.Mc.get(), ns, fqr, fi, r, Tall[fi].get(), r, ncols, s);
+        prof::KScope _ks("k_gather_cols", s);
+        if (rest > 0)
+          k_gather_cols<<<grid_1d((int64_t)r * rest), 256, 0, s>>>(Tall[fi].get(), r, r, dord[fi].get() + r, rest,
+                                                                   Touts[fi]->get(), r);
+        k_gather_cols<<<grid_1d((int64_t)ns2 * r), 256, 0, s>>>(f.A2.get(), ns2, ns2, dord[fi].get(), r, G2[fi].get(),
+                                                                ns2);
+      }
+      {
+        GemmModeScope mode(gemm_double_float() ? HBS_PRECISION_TENSOR : HBS_PRECISION_FP64);
+        run_gemms(bj, s);  // reads up to 3e-14 high in double-float or on the digit planes
+      }
+      DevBuf<double> acc(6);
+      HBS_CUDA(cudaMemsetAsync(acc.get(), 0, 6 * sizeof(double), s));
+      for (int fi = 0; fi < 3; ++fi) {
+        if (franks[fi] == 0) continue;
+        const Family& f = fams[fi];
+        prof::KScope _ks("k_diff_norm2", s);
+        k_diff_norm2<<<grid_1d((int64_t)ns2 * f.ncols), 256, 0, s>>>(B2[fi].get(), ns2, f.A2.get(), ns2, ns2, f.ncols,
+                                                                      acc.get() + 2 * fi);
+      }
+      HBS_LAUNCH_CHECK("k_diff_norm2");
+      const std::vector<double> ha = acc.download(s);
+      for (int fi = 0; fi < 3; ++fi) {
+        const double r = ha[2 * fi + 1] > 0 ? std::sqrt(ha[2 * fi] / ha[2 * fi + 1]) : 0.0;
+        h.pid_residual = std::max(h.pid_residual, r);
+        if (fi < 2) walls = std::max(walls, r);
+      }
     }
-    HBS_LAUNCH_CHECK("k_diff_norm2");
-    const std::vector<double> ha = acc.download(s);
-    for (int fi = 0; fi < 3; ++fi)
-      if (ha[2 * fi + 1] > 0) h.pid_residual = std::max(h.pid_residual, std::sqrt(ha[2 * fi] / ha[2 * fi + 1]));
-  }
+    return walls;
+  };
+  const int cstride = std::max(1, std::min(3, (int)(cstep / h.ch + 1e-9)));
+  const double walls = identify(cstride);
+  if (cstride > 1 && (!(walls <= 1e-13) || injected_id_residual())) identify(1);
   std::vector<int>& permY = fperm[0];
   std::vector<int>& permC = fperm[1];
   std::vector<int>& permE = fperm[2];
