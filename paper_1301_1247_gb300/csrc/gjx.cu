@@ -800,7 +800,7 @@ void gjx_invert(const std::vector<std::pair<cplx*, int>>& mats, cudaStream_t s, 
   int n_pow = 1, c_pow = 1;
   while (n_pow < nmax) n_pow *= 2;
   while (c_pow < nm) c_pow *= 2;
-  const std::string tkey = "inverse/n" + std::to_string(n_pow) + "/j" + std::to_string(c_pow) + (df ? "/df" : "");
+  const std::string tkey = "inverse/cluster/n" + std::to_string(n_pow) + "/j" + std::to_string(c_pow) + (df ? "/df" : "");
   const int CS = gjx_tuned_cluster(tkey, nm, nmax, df);
   Gjx g;
   {

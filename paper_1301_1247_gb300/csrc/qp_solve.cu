@@ -991,7 +991,7 @@ static void schur_solve(const std::vector<GroupJob>& gjobs, cplx* Sp, cplx* Rp, 
   int n_pow = 1, g_pow = 1;
   while (n_pow < nmax) n_pow *= 2;
   while (g_pow < ng) g_pow *= 2;
-  const std::string tkey = "schur/n" + std::to_string(n_pow) + "/g" + std::to_string(g_pow) + (df ? "/df" : "");
+  const std::string tkey = "schur/cluster/n" + std::to_string(n_pow) + "/g" + std::to_string(g_pow) + (df ? "/df" : "");
   const int cs = gjx_tuned_cluster(tkey, ng, nmax, df);
   int var = 0;
   while ((1 << var) < cs) ++var;
