@@ -944,7 +944,8 @@ static int pqr_grid(size_t smem) {
     HBS_CUDA(cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev));
     return sm;
   }();
-  HBS_CUDA(raise_smem_limit((const void*)k_pqr<DF>, smem));
+  // at least 64 KB: the kernel's static shared memory counts too against the 48 KB it may have without asking
+  HBS_CUDA(raise_smem_limit((const void*)k_pqr<DF>, std::max<size_t>(smem, 64 * 1024)));
   int per_sm = 0;
   HBS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pqr<DF>, kNT, smem));
   if (per_sm < 1) throw Error(HBS_ERR_CUDA, "persistent QR kernel does not fit on an SM");
