@@ -847,7 +847,7 @@ static void launch_apply(const Gjx& g, int qblocks, const cplx* const* res, cplx
   const auto smem = [&](int c) { return (size_t)2 * QB * sizeof(cplx) * ((g.nmax + c - 1) / c); };
   while (CS > 1 && (int64_t)g.nm * qblocks * CS > 1216 && smem(CS / 2) <= 48 * 1024) CS /= 2;
   const auto fn = k_gjx_apply<PanelWidth<dfc>::value, QB>;
-  HBS_CUDA(raise_smem_limit((const void*)fn, smem(CS)));
+  HBS_CUDA(raise_smem_limit((const void*)fn, std::max<size_t>(smem(CS), 64 * 1024)));  // static memory counts too
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(g.nm * qblocks * CS));
   cfg.blockDim = dim3(kT);

@@ -1644,7 +1644,7 @@ static void reduced_batch(Handle& h, std::vector<GroupJob>& gjobs, std::vector<s
   {
     prof::KScope _ks("k_red_bragg", s);
     const size_t shm = (size_t)S2 * sizeof(cplx);
-    HBS_CUDA(raise_smem_limit((const void*)k_red_bragg, shm));
+    HBS_CUDA(raise_smem_limit((const void*)k_red_bragg, std::max<size_t>(shm, 64 * 1024)));  // static memory counts too
     k_red_bragg<<<(unsigned)na, 256, shm, s>>>(R, DD, dg.get(), da.get(), Eb.get(), XL.get(), XR.get(), EP.get(),
                                                Rp.get(), h.y0, cbuf.get(), dbuf.get(), fbuf.get());
   }
