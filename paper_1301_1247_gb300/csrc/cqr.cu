@@ -380,8 +380,7 @@ void launch_gl(const CqrJob* dj, int nj, size_t sm, int CS, double tol, cudaStre
 
 // Lanes per column: 8, 16 or 32, so that a CTA's groups (32, 16, 8) have about one column each at the start.
 template <typename T>
-void launch_cqr(const CqrJob* dj, int nj, int mmax, int nmax, int CS, double tol, cudaStream_t s) {
-  const size_t sm = c_smem<T>(mmax, nmax, CS);
+void launch_cqr(const CqrJob* dj, int nj, size_t sm, int nmax, int CS, double tol, cudaStream_t s) {
   const int cols = (nmax + CS - 1) / CS;
   if (cols > 20) launch_gl<T, 8>(dj, nj, sm, CS, tol, s);
   else if (cols > 10) launch_gl<T, 16>(dj, nj, sm, CS, tol, s);
@@ -405,6 +404,7 @@ SideStream side_borrow(cudaStream_t like) {
   HBS_CUDA(cudaStreamGetPriority(like, &x.prio));
   {
     std::lock_guard<std::mutex> lk(g_side_mu);
+    g_side.reserve(16);  // giving back does not allocate
     for (size_t i = 0; i < g_side.size(); ++i)
       if (g_side[i].dev == x.dev && g_side[i].prio == x.prio) {
         x = g_side[i];
@@ -472,53 +472,49 @@ std::vector<int> cqr_run(const std::vector<CpqrJob>& js_in, double tol, cudaStre
   }
   DevBuf<CqrJob> dj;
   dj.upload(jobs, s);
-  // every class but the last on a side stream, between two events
-  std::vector<SideStream> side;
-  struct GiveBack {
-    std::vector<SideStream>& v;
-    ~GiveBack() {
-      for (const auto& x : v) side_return(x);
+  // Every class but the last on a side stream, between two events.  Joined whatever happens: the buffers above and
+  // the caller's matrices are freed in the order of s, and a launch that fails must not leave the
+  // classes before it reading them.
+  struct Sides {
+    cudaStream_t s;
+    std::vector<SideStream> v;
+    bool joined = false;
+    explicit Sides(cudaStream_t st) : s(st) { v.reserve(8); }
+    void join() {
+      for (const auto& x : v) {
+        HBS_CUDA(cudaEventRecord(x.ev, x.s));
+        HBS_CUDA(cudaStreamWaitEvent(s, x.ev, 0));
+      }
+      joined = true;
     }
-  } give_back{side};
+    ~Sides() {
+      for (const auto& x : v) {
+        if (!joined && (cudaEventRecord(x.ev, x.s) != cudaSuccess || cudaStreamWaitEvent(s, x.ev, 0) != cudaSuccess))
+          cudaStreamSynchronize(x.s);
+        side_return(x);
+      }
+    }
+  } side(s);
   for (int q0 = 0; q0 < nj;) {
-    int q1 = q0, mmax = 0, nmax = 0;
-    while (q1 < nj && size[order[q1]] == size[order[q0]]) {
-      mmax = std::max(mmax, js[q1].m);
+    const int CS = size[order[q0]];
+    int q1 = q0, nmax = 0;
+    size_t sm = 0;
+    for (; q1 < nj && size[order[q1]] == CS; ++q1) {
       nmax = std::max(nmax, js[q1].n);
-      ++q1;
-    }
-    // the largest m and n may belong to different matrices: the smallest size that holds both
-    int CS = size[order[q0]];
-    const auto bytes = [&](int c) { return df ? c_smem<dfc>(mmax, nmax, c) : c_smem<cplx>(mmax, nmax, c); };
-    while (CS < 8 && bytes(CS) > kSmemMax) CS *= 2;
-    if (bytes(CS) > kSmemMax) {  // not together: halve the class
-      q1 = q0 + std::max(1, (q1 - q0) / 2);
-      mmax = nmax = 0;
-      for (int q = q0; q < q1; ++q) {
-        mmax = std::max(mmax, js[q].m);
-        nmax = std::max(nmax, js[q].n);
-      }
-      if (bytes(8) > kSmemMax) {  // one at a time
-        q1 = q0 + 1;
-        mmax = js[q0].m;
-        nmax = js[q0].n;
-      }
+      sm = std::max(sm, df ? c_smem<dfc>(js[q1].m, js[q1].n, CS) : c_smem<cplx>(js[q1].m, js[q1].n, CS));
     }
     cudaStream_t on = s;
     if (q1 < nj) {
-      side.push_back(side_borrow(s));
-      on = side.back().s;
-      HBS_CUDA(cudaEventRecord(side.back().ev, s));
-      HBS_CUDA(cudaStreamWaitEvent(on, side.back().ev, 0));
+      side.v.push_back(side_borrow(s));
+      on = side.v.back().s;
+      HBS_CUDA(cudaEventRecord(side.v.back().ev, s));
+      HBS_CUDA(cudaStreamWaitEvent(on, side.v.back().ev, 0));
     }
-    if (df) launch_cqr<dfc>(dj.get() + q0, q1 - q0, mmax, nmax, CS, tol, on);
-    else launch_cqr<cplx>(dj.get() + q0, q1 - q0, mmax, nmax, CS, tol, on);
+    if (df) launch_cqr<dfc>(dj.get() + q0, q1 - q0, sm, nmax, CS, tol, on);
+    else launch_cqr<cplx>(dj.get() + q0, q1 - q0, sm, nmax, CS, tol, on);
     q0 = q1;
   }
-  for (const auto& x : side) {
-    HBS_CUDA(cudaEventRecord(x.ev, x.s));
-    HBS_CUDA(cudaStreamWaitEvent(s, x.ev, 0));
-  }
+  side.join();
   HBS_LAUNCH_CHECK("k_cqr");
   const std::vector<int> h = dr.download(s);
   int kmax = 0, ncmax = 0;
