@@ -406,7 +406,9 @@ hbs_status hbs_row_id_static(void* mt, int64_t m, int64_t n, double tol, int* ra
  *    n > 4096) may reach rank `value` at most (0 = no cap); one that needs more
  *    returns HBS_ERR_RANK, as an overflow of the supported maximum would;
  *  - HBS_INJECT_ID_RESIDUAL: the next `value` checks of a build's periodizer IDs that were
- *    found on candidate contour nodes count as failed, so that the build repeats them on all nodes.
+ *    found on candidate contour nodes count as failed, so that the build repeats them on all nodes;
+ *  - HBS_INJECT_DEVICE_FULL: as HBS_INJECT_ALLOC_FAILURE, but the failure is the device's lack
+ *    of memory, after which hbs_build_batch builds once more with less memory in use at a time.
  * Returns HBS_ERR_INVALID_ARG for an unknown kind or a negative value.
  *
  * hbs_barrier_selftest runs the library's bounded grid barrier (the one the
@@ -420,6 +422,7 @@ hbs_status hbs_row_id_static(void* mt, int64_t m, int64_t n, double tol, int* ra
 #define HBS_INJECT_ALLOC_FAILURE 1
 #define HBS_INJECT_RANK_CAP 2
 #define HBS_INJECT_ID_RESIDUAL 3
+#define HBS_INJECT_DEVICE_FULL 4
 hbs_status hbs_fault_inject(int kind, int64_t value);
 hbs_status hbs_barrier_selftest(int ctas, int absent_cta, double limit_s, int* passed, void* stream);
 

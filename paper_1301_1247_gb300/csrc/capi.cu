@@ -8,7 +8,6 @@
 #include <future>
 #include <mutex>
 #include <string>
-#include <system_error>
 #include <thread>
 #include <utility>
 #include <vector>
@@ -322,20 +321,24 @@ static size_t available_bytes() {
 // their solves: 203 ms one after another, 169 with two workers, 154 with four, 148 with eight (the
 // persistent QRs exclude one another).  Device, arithmetic modes and allocation stream are each
 // thread's own; the solvers' buffers pass to the caller's stream with the final synchronization.
-// A worker's scratch grows with its solver (some 4096 complex values a node at most in the shapes seen): no more
-// workers start than half of the available memory holds.  join() waits for all and rethrows the first
+// No more workers start than half of the available memory holds (periodizer_scratch), none if not even one:
+// join() is then where the periodizers are built, one after another.  join() waits for all and rethrows the first
 // error; the destructor joins too.
 class BatchPeriodizers {
  public:
-  BatchPeriodizers(const std::vector<Handle*>& hs, std::shared_future<void> compressed)
+  BatchPeriodizers(const std::vector<Handle*>& hs, std::shared_future<void> compressed, bool beside)
       : hs_(hs), compressed_(std::move(compressed)) {
     // the largest first: the last ones to start are then short
     std::stable_sort(hs_.begin(), hs_.end(), [](const Handle* a, const Handle* b) { return a->N > b->N; });
     int dev = 0;
     HBS_CUDA(cudaGetDevice(&dev));
     const bool df = gemm_double_float(), tc = gemm_tensor();
-    const size_t scratch = (size_t)hs_[0]->N * 4096 * sizeof(cplx);
-    const size_t n = std::max<size_t>(1, std::min({(size_t)4, hs_.size(), available_bytes() / 2 / scratch}));
+    std::vector<size_t> scratch;
+    for (const Handle* h : hs_) scratch.push_back(periodizer_scratch(*h));
+    std::sort(scratch.rbegin(), scratch.rend());
+    size_t n = 0, room = available_bytes() / 2;
+    while (beside && n < std::min<size_t>(4, hs_.size()) && scratch[n] <= room) room -= scratch[n++];
+    threads_.reserve(n);
     auto work = [this, dev, df, tc] {
       cudaStream_t s = nullptr;
       try {
@@ -360,16 +363,18 @@ class BatchPeriodizers {
     for (size_t i = 0; i < n; ++i) {
       try {
         threads_.emplace_back(work);
-      } catch (const std::system_error&) {  // no more threads to be had: those there do the work
-        if (threads_.empty()) throw;
+      } catch (const std::exception&) {  // no more threads to be had: those there do the work, or join()
         break;
       }
     }
   }
   ~BatchPeriodizers() { wait(); }
-  void join() {
+  // On the caller's stream s the periodizers that no worker took.
+  void join(cudaStream_t s) {
     wait();
     if (err_) std::rethrow_exception(err_);
+    compressed_.get();  // the compression's error, if no worker has met it
+    for (size_t j; (j = next_.fetch_add(1)) < hs_.size();) build_periodizer(*hs_[j], s, false, &compressed_);
   }
 
  private:
@@ -407,8 +412,8 @@ hbs_status hbs_build_batch(const hbs_geometry* geoms, const double* omegas, int6
       return HBS_ERR_OOM;
     }
   }
-  hbs_status st = guarded([&] {
-    auto t0 = std::chrono::steady_clock::now();
+  // With beside, the periodizers run beside the compression; without, one after another behind it.
+  const auto build = [&](bool beside) {
     std::vector<Handle*> hs(count);
     for (int64_t i = 0; i < count; ++i) {
       hs[i] = &hh[i]->h;
@@ -417,7 +422,7 @@ hbs_status hbs_build_batch(const hbs_geometry* geoms, const double* omegas, int6
     GemmModeScope gm(hs[0]->opts.precision);
     HBS_CUDA(cudaStreamSynchronize(s));  // the geometries are in place for the workers' streams
     std::promise<void> done;
-    BatchPeriodizers workers(hs, done.get_future().share());
+    BatchPeriodizers workers(hs, done.get_future().share(), beside);
     try {
       {
         prof::Phase ph("build:hbs_compress_invert", s);
@@ -428,9 +433,24 @@ hbs_status hbs_build_batch(const hbs_geometry* geoms, const double* omegas, int6
     } catch (...) {
       done.set_exception(std::current_exception());
     }
-    workers.join();
+    workers.join(s);
+    HBS_CUDA(cudaStreamSynchronize(s));
+  };
+  hbs_status st = guarded([&] {
+    auto t0 = std::chrono::steady_clock::now();
+    try {
+      build(true);
+    } catch (const DeviceFull&) {  // what fits one after another is still built
+      cudaStreamSynchronize(s);
+      for (auto*& p : hh) {
+        delete p;
+        p = nullptr;
+      }
+      for (auto*& p : hh) p = new hbs_handle();
+      build(false);
+    }
     const double sec = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-    for (Handle* h : hs) h->build_seconds = sec;
+    for (auto* p : hh) p->h.build_seconds = sec;
   });
   if (st != HBS_OK) {
     for (auto* p : hh) delete p;

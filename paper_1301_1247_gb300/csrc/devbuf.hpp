@@ -21,11 +21,17 @@ struct Error : public std::runtime_error {
   Error(hbs_status c, const std::string& m) : std::runtime_error(m), code(c) {}
 };
 
+// An allocation that the device had no memory for (HBS_ERR_OOM).
+struct DeviceFull : public Error {
+  explicit DeviceFull(const std::string& m) : Error(HBS_ERR_OOM, m) {}
+};
+
 inline void cuda_check(cudaError_t e, const char* what) {
   if (e != cudaSuccess) {
     cudaGetLastError();
-    throw Error(e == cudaErrorMemoryAllocation ? HBS_ERR_OOM : HBS_ERR_CUDA,
-                std::string(what) + ": " + cudaGetErrorString(e));
+    const std::string m = std::string(what) + ": " + cudaGetErrorString(e);
+    if (e == cudaErrorMemoryAllocation) throw DeviceFull(m);
+    throw Error(HBS_ERR_CUDA, m);
   }
 }
 
@@ -35,9 +41,10 @@ inline void cuda_check(cudaError_t e, const char* what) {
 cudaStream_t& current_stream();
 
 // Fault injection for tests of the error paths (hbs_fault_inject): true when the caller's
-// device allocation is the one chosen to fail; the largest rank an ID may reach (0 = none); true when the
-// check of a periodizer ID is to count as failed.
+// device allocation is the one chosen to fail, or to find the device full; the largest rank an ID may reach
+// (0 = none); true when the check of a periodizer ID is to count as failed.
 bool injected_alloc_failure();
+bool injected_device_full();
 bool injected_id_residual();
 
 // Raise a kernel's limit on dynamic shared memory to at least `bytes` (cudaFuncSetAttribute)
@@ -87,6 +94,7 @@ class DevBuf {
     void* p = nullptr;
     if (injected_alloc_failure())
       throw Error(HBS_ERR_OOM, "device allocation failed (injected by hbs_fault_inject)");
+    if (injected_device_full()) throw DeviceFull("device memory exhausted (injected by hbs_fault_inject)");
     HBS_CUDA(cudaMallocAsync(&p, n * sizeof(T), current_stream()));
     p_ = static_cast<T*>(p);
     n_ = n;

@@ -17,17 +17,21 @@
 namespace hbs {
 namespace {
 std::atomic<int64_t> g_alloc_countdown{-1};  // allocations left before the failing one (-1: off)
+std::atomic<int64_t> g_full_countdown{-1};   // the same for the one that finds the device full
 std::atomic<int> g_rank_cap{0};
 std::atomic<int64_t> g_id_checks{0};  // checks of periodizer IDs that are still to fail
 }  // namespace
 
-bool injected_alloc_failure() {
-  int64_t v = g_alloc_countdown.load(std::memory_order_relaxed);
+static bool count_down(std::atomic<int64_t>& left) {
+  int64_t v = left.load(std::memory_order_relaxed);
   while (v >= 0) {
-    if (g_alloc_countdown.compare_exchange_weak(v, v - 1, std::memory_order_relaxed)) return v == 0;
+    if (left.compare_exchange_weak(v, v - 1, std::memory_order_relaxed)) return v == 0;
   }
   return false;
 }
+
+bool injected_alloc_failure() { return count_down(g_alloc_countdown); }
+bool injected_device_full() { return count_down(g_full_countdown); }
 
 bool injected_id_residual() {
   int64_t v = g_id_checks.load(std::memory_order_relaxed);
@@ -56,6 +60,7 @@ extern "C" hbs_status hbs_fault_inject(int kind, int64_t value) {
       hbs::g_alloc_countdown.store(-1);
       hbs::g_rank_cap.store(0);
       hbs::g_id_checks.store(0);
+      hbs::g_full_countdown.store(-1);
       return HBS_OK;
     case HBS_INJECT_ALLOC_FAILURE:
       if (value < 0) break;
@@ -64,6 +69,10 @@ extern "C" hbs_status hbs_fault_inject(int kind, int64_t value) {
     case HBS_INJECT_RANK_CAP:
       if (value < 0 || value > (1 << 30)) break;
       hbs::g_rank_cap.store((int)value);
+      return HBS_OK;
+    case HBS_INJECT_DEVICE_FULL:
+      if (value < 0) break;
+      hbs::g_full_countdown.store(value);
       return HBS_OK;
     case HBS_INJECT_ID_RESIDUAL:
       if (value < 0) break;

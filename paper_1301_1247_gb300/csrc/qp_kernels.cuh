@@ -157,6 +157,7 @@ __global__ void k_diff_norm2(const cplx* a, int64_t lda, const cplx* b, int64_t 
 // two share the device until the transposed sweep, which needs both.
 // with_hbs: runs the compression beside it on a thread of its own.  compressed: the compression runs
 // elsewhere and is waited for before V is formed.
+size_t periodizer_scratch(const Handle& h);
 void build_periodizer(Handle& h, cudaStream_t s, bool with_hbs = false,
                       const std::shared_future<void>* compressed = nullptr);
 void solve_angles(Handle& h, const double* theta, int64_t n_theta, bool plain, Result& out, cudaStream_t s);

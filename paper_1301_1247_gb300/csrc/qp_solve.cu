@@ -160,6 +160,33 @@ struct QrShareScope {
 };
 }  // namespace
 
+// Device memory that build_periodizer may have in use besides the compression's, from the sizes known before it:
+// the wall families on their subsample (8 M members, contour nodes M and samples as chosen there), and per unknown
+// the neighbour matrix, its digit planes and the blocks of rsel columns.  The ranks are bounds of those seen for
+// omega d up to 110.  Against the memory pool's high-water mark, for 400 to 60 000 nodes, omega 5 to 100, FP64 and
+// tensor, sound-soft and dielectric: 1.2 to 5.3 times as much (64 KB a node was a fifth of it for the smallest).
+size_t periodizer_scratch(const Handle& h) {
+  const double d = h.d, cw = h.opts.contour_w > 0 ? h.opts.contour_w : 2.0, ch = h.opts.contour_h > 0 ? h.opts.contour_h : 0.2;
+  double xmax = 0.0, lo = 1e300, hi = -1e300, perim = 0.0;
+  for (int64_t i = 0; i < h.N; ++i) {
+    const int64_t j = (i + 1) % h.N;
+    xmax = std::max(xmax, std::fabs(h.hx[i]));
+    lo = std::min(lo, h.hy[i]);
+    hi = std::max(hi, h.hy[i]);
+    perim += std::hypot(h.hx[j] - h.hx[i], h.hy[j] - h.hy[i]);
+  }
+  const double smin = 37.0 / (2.0 * (d - xmax));
+  double reach = h.opts.contour_k > 0 ? h.opts.contour_k : std::sqrt(h.omega * h.omega + smin * smin) + 2.0 * cw;
+  reach += 0.5 * h.omega;  // the second contour's crossing point is below that
+  const double M = h.opts.m > 0 ? h.opts.m : 2.0 * reach / ch;
+  const double S = std::max<double>(h.opts.n_bragg_samples, 48.0 + h.omega * d / M_PI);
+  const double samples = std::min(h.N / (double)h.comps, std::min(16384.0, 512.0 + 12.0 * perim * std::max(h.omega, reach) / (2.0 * M_PI)));
+  const double wd = h.omega * std::max(d, hi - lo);
+  const double families = (2.0 * 8.0 * M + 12.0 * S) * samples * h.comps * 6.0;
+  const double unknown = 2.75 * (1000.0 + 4.0 * wd) + 8.0 * (400.0 + 8.0 * wd);
+  return (size_t)(16.0 * (families + unknown * (double)h.N));
+}
+
 void build_periodizer(Handle& h, cudaStream_t s, bool with_hbs, const std::shared_future<void>* compressed) {
   HbsWorker hbs_worker;
   if (with_hbs) hbs_worker.start(h);

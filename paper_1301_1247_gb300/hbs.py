@@ -427,7 +427,7 @@ def batched_inverse(a, n, count, precision=0, stream=None):
     return st
 
 
-INJECT_CLEAR, INJECT_ALLOC_FAILURE, INJECT_RANK_CAP, INJECT_ID_RESIDUAL = 0, 1, 2, 3
+INJECT_CLEAR, INJECT_ALLOC_FAILURE, INJECT_RANK_CAP, INJECT_ID_RESIDUAL, INJECT_DEVICE_FULL = 0, 1, 2, 3, 4
 
 
 def fault_inject(kind, value=0):
