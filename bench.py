@@ -62,10 +62,12 @@ def kernel_peak(name, prec):
                 "against the measured cuBLAS bf16 burst rate in MEASURED_PEAKS.json")
     # kernels whose updates run in double-float on double-float and tensor-precision handles:
     # FP32-pipe instructions per FP64-equivalent flop (a complex multiply-add is 4 error-free
-    # multiply-adds of 12 instructions, 48 per 8 flops; the pivoted QR's update, 102 per 16)
-    df_per = {"k_zgemm_batched_df": 48.0 / 8.0, "k_pqr": 102.0 / 16.0, "k_cpqr": 102.0 / 16.0, "k_cqr": 102.0 / 16.0,
-              "k_schur_solve": 48.0 / 8.0, "k_pgj": 48.0 / 8.0, "k_gj_inverse": 48.0 / 8.0,
-              "k_bgj_panel": 48.0 / 8.0, "k_gjx": 48.0 / 8.0, "k_gj_small": 48.0 / 8.0}
+    # multiply-adds of 12 instructions, 48 per 8 flops; the pivoted QR's update, 102 per 16).  The last five
+    # names are those of kernels in records made before the cluster QR and elimination.
+    df_per = {"k_zgemm_batched_df": 48.0 / 8.0, "k_pqr": 102.0 / 16.0, "k_cqr": 102.0 / 16.0, "k_gjx": 48.0 / 8.0,
+              "k_gjx_solve": 48.0 / 8.0, "k_gj_small": 48.0 / 8.0,
+              "k_cpqr": 102.0 / 16.0, "k_schur_solve": 48.0 / 8.0, "k_pgj": 48.0 / 8.0, "k_gj_inverse": 48.0 / 8.0,
+              "k_bgj_panel": 48.0 / 8.0}
     if name == "k_zgemm_batched_df" or (prec >= 1 and name in df_per):
         per = df_per[name]
         return ("alu", FP32_INSTR_PEAK / per / 1e12,
@@ -80,6 +82,8 @@ FLOP_COUNT_NOTE = {
     "k_pqr": "8 m n k per m x n block of rank k (interpolative decomposition; Householder executes ~2x)",
     "k_cqr": "8 m n k per m x n block of rank k (interpolative decomposition; Householder executes ~2x)",
     "k_gjx": "8 n^3 per n x n block (Gauss-Jordan inverse)",
+    "k_gj_small": "8 n^3 per n x n block (Gauss-Jordan inverse)",
+    "k_gjx_solve": "4 n^3 + 8 n^2 q per system (Gauss-Jordan elimination of full columns; LU counts 8/3 n^3)",
     "k_zgemm_batched_df": "8 m n k per product",
     "k_zgemm_batched": "8 m n k per product",
     "k_oz_mma": "executed bf16 digit-plane flops on padded tiles",

@@ -86,7 +86,8 @@ def main():
              "// i < kHankelIntervals, P = kHankelPerUnit, in t = 2(P z - i) - 1 (first coefficient",
              "// halved).  Layout: [interval][function][coefficient]; kHankelChebDF holds each",
              "// coefficient as a float pair (hi, lo), hi + lo = c to 2^-48.  kHankelPoly, kHankelPolyDF: the",
-             "// same polynomials in powers of t, layout [interval][power][function] (the kernels' form).",
+             "// same polynomials in powers of t, layout [interval][power][function].  The kernels read these two",
+             "// only; the Chebyshev forms are what they are derived from and are checked against.",
              "#pragma once",
              f"constexpr int kHankelIntervals = {NI};",
              f"constexpr int kHankelDegree = {ND};",

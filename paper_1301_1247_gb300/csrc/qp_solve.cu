@@ -1024,7 +1024,11 @@ static void schur_solve(const std::vector<GroupJob>& gjobs, cplx* Sp, cplx* Rp, 
   while ((1 << var) < cs) ++var;
   Gjx g;
   {
+    // every row of the columns to the right and of the right-hand sides, a column at a time: half of an inverse
+    double fl = 0.0;
+    for (const auto& m : sys) fl += 4.0 * m.n * (double)m.n * m.n + 8.0 * m.n * (double)m.n * m.q;
     tune::Timed timed(tkey, var, 4, s);
+    prof::KScope _ks("k_gjx_solve", s, fl, 0.0);
     gjx_eliminate(g, sys, df, /*invert=*/false, cs, s);
   }
   DevBuf<cplx> X(std::max<int64_t>(rend, 1));
@@ -1036,7 +1040,10 @@ static void schur_solve(const std::vector<GroupJob>& gjobs, cplx* Sp, cplx* Rp, 
   DevBuf<cplx*> dx, dr;
   dx.upload(xp, s);
   dr.upload(rp, s);
-  gjx_solution(g, dx.get(), ill, s);
+  {
+    prof::KScope _ks("k_gjx_solution_out", s);
+    gjx_solution(g, dx.get(), ill, s);
+  }
   if (df) {  // R <- R - S X (FP64), then X += the elimination applied to it
     GemmModeScope fp64(HBS_PRECISION_FP64);
     std::vector<GemmJob> gj;
@@ -1605,16 +1612,8 @@ static void reduced_batch(Handle& h, std::vector<GroupJob>& gjobs, std::vector<s
   }
   HBS_LAUNCH_CHECK("k_red_assemble");
   DevBuf<int> ill(ng);
-  {
-    double sfl = 0.0;
-    for (auto& G : gjobs) {
-      const double n = G.nsys;
-      sfl += 8.0 / 3.0 * n * n * n + 8.0 * n * n * G.q;
-    }
-    prof::KScope _ks("k_schur_solve", s, sfl, 0.0);
-    schur_solve(gjobs, Sp.get(), Rp.get(), ill.get(), s);
-  }
-  HBS_LAUNCH_CHECK("k_schur_solve");
+  schur_solve(gjobs, Sp.get(), Rp.get(), ill.get(), s);
+  HBS_LAUNCH_CHECK("Schur systems");
   ph.next("solve:bragg");
   std::vector<AngleJob> ajobs;
   int64_t oo = 0;
@@ -2022,16 +2021,8 @@ void solve_angles(Handle& h, const double* theta, int64_t n_theta, bool plain, R
     }
     HBS_LAUNCH_CHECK("k_assemble");
     DevBuf<int> ill(ng);
-    double sfl = 0.0;
-    for (auto& G : gjobs) {
-      const double n = 2.0 * l + 2.0 * M + G.nw;
-      sfl += 8.0 / 3.0 * n * n * n + 8.0 * n * n * G.q;
-    }
-    {
-      prof::KScope _ks("k_schur_solve", s, sfl, 0.0);
-      schur_solve(gjobs, Sp.get(), Rp.get(), ill.get(), s);
-    }
-    HBS_LAUNCH_CHECK("k_schur_solve");
+    schur_solve(gjobs, Sp.get(), Rp.get(), ill.get(), s);
+    HBS_LAUNCH_CHECK("Schur systems");
     // ---- Bragg amplitudes
     ph.next("solve:bragg");
     int64_t oo = 0;
