@@ -477,9 +477,9 @@ def run_ours(args, ws, rank, local):
         "scaling": "weak", "vs_baseline": None,
         "dtype": {0: "f64 (complex128)",
                   1: "f64 (complex128) data; double-float (2xFP32) arithmetic for the dense products, the QR and "
-                     "Gauss-Jordan updates, the Hankel series and the Schur LU (refined once in FP64)",
+                     "Gauss-Jordan updates, the Hankel series and the Schur eliminations (refined once in FP64)",
                   2: "f64 (complex128) data; double-float (2xFP32) arithmetic for the dense products, the QR and "
-                     "Gauss-Jordan updates, the Hankel series and the Schur LU (refined once in FP64); products with "
+                     "Gauss-Jordan updates, the Hankel series and the Schur eliminations (refined once in FP64); products with "
                      "k >= 96 on tcgen05 tensor cores from exact bf16 digit planes"}[prec],
         "data": "synthetic", "err_vs_fp64_plain_path": err["max"] if err else None,
         "err_vs_fp64_plain_path_detail": err,

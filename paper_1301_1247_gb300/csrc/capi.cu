@@ -318,7 +318,7 @@ static size_t available_bytes() {
 // a chain of kernels that rarely fill the chip (a pivoted QR of 100-200 dependent steps, small
 // products, host reads between them), so several share the device with one another and with the
 // batch's compression, which they wait for only before V is formed.  16 solvers of 400 to 20 000 nodes and
-// their solves: 203 ms one after another, 169 with two workers, 154 with four, 148 with eight (the
+// their solves: 204 ms one after another, 176 with two workers, 163 with four, 156 with eight (the
 // persistent QRs exclude one another).  Device, arithmetic modes and allocation stream are each
 // thread's own; the solvers' buffers pass to the caller's stream with the final synchronization.
 // No more workers start than half of the available memory holds (periodizer_scratch), none if not even one:

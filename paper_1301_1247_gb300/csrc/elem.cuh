@@ -53,7 +53,8 @@ __device__ __forceinline__ dfc x_shfl(const dfc& v, int l) { return dfc_shfl(v, 
 // Pivot keys: |v|^2 to float precision (double-float), or the exponent and upper significand bits of |v|^2
 // (FP64), as unsigned integers that order alike; 1 is an exact zero and 0 no candidate.  A square
 // carries no sign, so a sign bit belongs to a NaN and is dropped: a key made from it could wrap to 0, and a column
-// whose candidates all have key 0 has no pivot row.  A NaN's key is above every number's.
+// whose candidates all have key 0 has no pivot row.  A NaN's key is above every number's.  In FP64 the pivot chosen
+// is the column's largest to 2^-20 of its square, so that no multiplier passes 1 + 2^-20.
 __device__ __forceinline__ unsigned x_key(const cplx& v) {
   const double m = cabs2(v);
   const unsigned hi = (unsigned)__double2hiint(m) & 0x7FFFFFFFu;

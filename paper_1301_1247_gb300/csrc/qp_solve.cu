@@ -145,10 +145,10 @@ struct HbsWorker {
 
 namespace {
 // Keeps this thread's QRs to their share of the device while the compression runs beside it: every other SM
-// from 6000 unknowns on, where the compression is the longer chain.  Build and solve, one CTA an SM
-// against every other SM (double-float with tensor cores): star of 800 nodes 10.6 / 11.3 ms, 2000 13.1 / 14.8,
-// 4000 16.6 / 17.4, 6000 17.1 / 17.1, 8000 19.5 / 18.7, 12 000 24.2 / 22.4; wiggly of 6000 21.0 / 19.5, 20 000
-// 33.2 / 31.0, FP64 56.2 / 54.3 and 121.6 / 119.9.  Two fifths of the SMs were slower again.
+// from 6000 unknowns on, where the compression is the longer chain by far.  Build and solve, one CTA an SM
+// against every other SM (tensor-core products): star of 800 nodes 8.6 / 9.2 ms, 2000 11.1 / 11.3, 4000 14.8 / 13.3,
+// 6000 16.1 / 14.5, 8000 17.4 / 15.8, 12 000 21.4 / 19.9; wiggly of 6000 22.0 / 19.9, 20 000 37.1 / 34.7, FP64 60.8 /
+// 53.3 and 121.0 / 120.3.  Two fifths of the SMs were slower again.
 constexpr int64_t kQrBesideUnknowns = 6000;
 struct QrShareScope {
   QrShare prev;

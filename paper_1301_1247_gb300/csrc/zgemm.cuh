@@ -84,7 +84,7 @@ __device__ __forceinline__ void tile_slice(const T (*As)[GBM + 1], const T (*Bs)
 // last slice of k ends at K.  (With 16 x 16 threads of 2 x 2 outputs and whole slices, a 690 x 49
 // x 49 leaf product executed 1.49 multiply-adds for each that counts; now 1.06.  The transposed
 // sweep of N = 10^5 to 690 rows, its double-float products: 37.4 -> 33.7 ms; the apply of a 10^4
-// inverse to 192 columns in FP64: 8.4 -> 7.2 ms, 0.94 of the FP64 pipe's 1.26 TFLOP/s.)  A loop of
+// inverse to 192 columns in FP64: 8.4 -> 7.2 ms, 0.94 TFLOP/s of the FP64 pipe's 1.26, edges not counted.)  A loop of
 // the double-float multiply-add alone, operands in registers, reaches 5.1 of the 6.7 TFLOP/s that
 // its instruction count allows (three-operand FMAs issue at 0.8 per cycle).
 //
