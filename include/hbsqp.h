@@ -401,9 +401,8 @@ hbs_status hbs_row_id_static(void* mt, int64_t m, int64_t n, double tol, int* ra
  *  - HBS_INJECT_ALLOC_FAILURE: the device allocation `value` allocations from now
  *    (0 = the next one) fails before cudaMallocAsync is called; the call that made
  *    it returns HBS_ERR_OOM and frees what it had allocated.  One failure per arming;
- *  - HBS_INJECT_RANK_CAP: interpolative decompositions of the persistent QR (tree
- *    levels of at most 128 nodes, the neighbour and periodizer IDs, hbs_row_id with
- *    n > 4096) may reach rank `value` at most (0 = no cap); one that needs more
+ *  - HBS_INJECT_RANK_CAP: interpolative decompositions (tree levels, the neighbour and
+ *    periodizer IDs, hbs_row_id with n > 4096) may reach rank `value` at most (0 = no cap); one that needs more
  *    returns HBS_ERR_RANK, as an overflow of the supported maximum would;
  *  - HBS_INJECT_ID_RESIDUAL: the next `value` checks of a build's periodizer IDs that were
  *    found on candidate contour nodes count as failed, so that the build repeats them on all nodes;

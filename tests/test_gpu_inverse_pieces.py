@@ -30,3 +30,18 @@ def test_inverse_in_pieces(count, n, precision):
         bad[where] = 0
         assert hbs.batched_inverse(bad, n, count, precision) == hbs.HBS_WARN_ILLCOND
         del bad
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("n", [3585, 4096])
+def test_the_largest_blocks(n, precision):
+    """Two rows a thread on eight CTAs, up to the last one.  An entry of A X sums n products of about 1/4 n^-1/2, each
+    within 2^-44 (a 48-bit inverse whose error grows with its pivots): n^1/2 2^-46 at random, 1e-11 with room."""
+    import torch
+    hbs = require_lib()
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    a = torch.randn((1, n, n), generator=gen, device="cuda", dtype=torch.complex128)
+    a += 4 * np.sqrt(n) * torch.eye(n, device="cuda", dtype=torch.complex128)
+    x = a.clone()
+    assert hbs.batched_inverse(x, n, 1, precision) == hbs.HBS_OK
+    assert float((a[0] @ x[0] - torch.eye(n, device="cuda")).abs().max()) < 1e-11
