@@ -407,7 +407,8 @@ hbs_status hbs_row_id_static(void* mt, int64_t m, int64_t n, double tol, int* ra
  *  - HBS_INJECT_ID_RESIDUAL: the next `value` checks of a build's periodizer IDs that were
  *    found on candidate contour nodes count as failed, so that the build repeats them on all nodes;
  *  - HBS_INJECT_DEVICE_FULL: as HBS_INJECT_ALLOC_FAILURE, but the failure is the device's lack
- *    of memory, after which hbs_build_batch builds once more with less memory in use at a time.
+ *    of memory, after which hbs_build_batch builds once more with less memory in use at a time
+ *    and the inversions of many blocks go on with half as many at a time.
  * Returns HBS_ERR_INVALID_ARG for an unknown kind or a negative value.
  *
  * hbs_barrier_selftest runs the library's bounded grid barrier (the one the

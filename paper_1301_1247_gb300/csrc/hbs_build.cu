@@ -578,6 +578,18 @@ static std::vector<int> node_ids(std::vector<CpqrJob>& jobs, double tol, cudaStr
   return ranks;
 }
 
+// A piece whose copies the device has no memory for is halved, down to single blocks.
+static void invert_piece(const std::pair<cplx*, int>* first, size_t count, cudaStream_t s, const char* what) {
+  try {
+    gjx_invert({first, first + count}, s, what);
+    return;
+  } catch (const DeviceFull&) {  // before anything is written
+    if (count == 1) throw;
+  }
+  invert_piece(first, count / 2, s, what);
+  invert_piece(first + count / 2, count - count / 2, s, what);
+}
+
 // Batched in-place inverses; throws on a singular block.
 //
 // Blocks of at most 56 go to the kernel that holds one in shared memory; so do blocks of at most 72 in batches
@@ -613,7 +625,7 @@ void batched_inverse(std::vector<InvJob>& jobs, cudaStream_t s, const char* what
                                                   (int64_t)((all.size() + kInversePieceBlocks - 1) / kInversePieceBlocks));
   int64_t copy = 0;
   const auto flush = [&] {
-    if (!piece.empty()) gjx_invert(piece, s, what);
+    if (!piece.empty()) invert_piece(piece.data(), piece.size(), s, what);
     piece.clear();
     copy = 0;
   };

@@ -45,3 +45,25 @@ def test_the_largest_blocks(n, precision):
     x = a.clone()
     assert hbs.batched_inverse(x, n, 1, precision) == hbs.HBS_OK
     assert float((a[0] @ x[0] - torch.eye(n, device="cuda")).abs().max()) < 1e-11
+
+
+@pytest.mark.parametrize("after", [0, 2, 6])
+def test_a_full_device_halves_the_piece(after):
+    """An allocation of the working copies that finds the device full: the blocks go in two pieces.  A single
+    block's copy has no second chance."""
+    import torch
+    hbs = require_lib()
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    a = torch.randn((9, 130, 130), generator=gen, device="cuda", dtype=torch.complex128)
+    a += 4 * np.sqrt(130) * torch.eye(130, device="cuda", dtype=torch.complex128)
+    try:
+        x = a.clone()
+        hbs.fault_inject(hbs.INJECT_DEVICE_FULL, after)
+        assert hbs.batched_inverse(x, 130, 9, 1) == hbs.HBS_OK
+        hbs.fault_inject(hbs.INJECT_DEVICE_FULL, after)
+        with pytest.raises(hbs.HbsError) as e:
+            hbs.batched_inverse(a[0].clone(), 130, 1, 1)
+        assert e.value.status == hbs.HBS_ERR_OOM
+    finally:
+        hbs.fault_inject(hbs.INJECT_CLEAR)
+    assert float((a @ x - torch.eye(130, device="cuda")).abs().max()) < 1e-12
